@@ -210,7 +210,7 @@ double model_gcells_2d(const stencil_desc &d, int sms, const Cand2D &k, int bps,
     // the launch geometry of prepare2: one-warp blocks over (tile column, row) units in
     // segments of at least 4 rows; each segment streams 2T extra rows (Sec. 3.2's pipeline
     // fill and drain), and a small grid leaves SMs with fewer resident warps
-    const int halo = (k.T + 3) / 4 * 4;
+    const int halo = (k.T + k.V - 1) / k.V * k.V;   // tb2d_halo
     const long long cx = 32LL * k.V - 2 * halo;
     const long long units = (d.nx + cx - 1) / cx * (long long)d.ny;
     const long long ctas = std::min<long long>((long long)sms * bps, std::max<long long>(1, units / 4));
@@ -227,7 +227,7 @@ double model_gcells_2d(const stencil_desc &d, int sms, const Cand2D &k, int bps,
     m.steps = steps > 0 ? steps : 1000;
     m.T = k.T;
     m.bx = 32 * k.V;
-    m.halo_x = (k.T + 3) / 4 * 4;
+    m.halo_x = halo;
     m.sms = sms;
     m.sm_hz = 2.07e9;
     m.hbm_gbs = 6800.0;
@@ -1189,7 +1189,7 @@ static int plan_create(stencil_plan *out, const stencil_desc *desc)
             if (rc == ST_OK) rc = prepare2(p, p->T, &c);
             if (rc == ST_OK && p->stor) {
                 // coded grids: rows padded to 8 cells (16 bytes), codes per (row, tile column)
-                p->cx = 32 * p->V - 2 * ((p->T + 3) / 4 * 4);
+                p->cx = tb2d_tile_width(c->shape) - 2 * tb2d_halo(c->shape);
                 p->ntx = (d.nx + p->cx - 1) / p->cx;
                 p->ld_q = ((long long)d.nx + 7) / 8 * 8;
                 const size_t qb = (size_t)p->ld_q * d.ny * 2, mb = (size_t)p->ntx * d.ny * sizeof(float2);
@@ -1390,7 +1390,7 @@ int stencil_run(stencil_plan p, const void *grid_in, void *grid_out, const void 
         // contracted Hotspot 2D kernels stage sdc*(p + amb*Rz) (Table 2's source and ambient
         // terms folded into one map)
         e = hot_source(pw, d.nx, p->src, p->ld_src, d.nx, d.ny, coeffs[4], coeffs[3], coeffs[0],
-                       p->stream);
+                       p->V, p->stream);
         if (e != cudaSuccess) return map_cuda(e);
         pw = p->src;
     }
@@ -1448,7 +1448,7 @@ int stencil_run_trajectory(stencil_plan p, const void *grid_in, void *states, lo
         // contracted Hotspot kernels stage sdc*(p + amb*Rz) (Table 2's source and ambient terms
         // folded into one map)
         const cudaError_t e = hot_source(pw, d.nx, p->src, p->ld_src, d.nx, d.ny, coeffs[4],
-                                         coeffs[3], coeffs[0], p->stream);
+                                         coeffs[3], coeffs[0], c->shape.V, p->stream);
         if (e != cudaSuccess) return map_cuda(e);
         pw = p->src;
     }
@@ -1544,7 +1544,7 @@ int stencil_plan_get_info(stencil_plan p, stencil_plan_info *info)
         const int warps = std::max(p->W, 1);   // W = 0 marks the one-warp in-place variant
         info->bx = 32 * p->V * warps;
         info->by = 0;
-        info->halo = (p->T + 3) / 4 * 4;
+        info->halo = tb2d_halo(c->shape);
         info->vec = p->V;
         info->warps = warps;
         info->ctas = c->ctas;

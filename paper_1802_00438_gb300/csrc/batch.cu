@@ -54,9 +54,9 @@ namespace {
 // workload, T = 8: 1921 / 1973 / 1980 / 1978 / 1961 GCell/s for L = 128 / 160 / 192 / 224 / 256)
 constexpr int kRows = 192;
 constexpr long long kWaitNs = 1000LL * 1000 * 1000;   // 1 s: a wait of a healthy batch is far shorter
-// (T, V) of the compiled queue kernel: 4 cells per lane (with 8, the launch ran at half the
-// rate on the 64-grid workload: 816 against 1713 GCell/s, one 255-register block per SMSP pair;
-// T = 12 with 4 cells, 255 registers, 1763 against 1980 for T = 8)
+// (T, V) of the compiled queue kernel: 4 cells per lane (64-grid workload: 12.8 ms; with 8, 255
+// registers and two warps per scheduler, 14.1 ms at its best L; T = 12 with 4 cells, 255
+// registers, was 12 % slower than T = 8)
 const int kCand[][2] = {{8, 4}};
 
 int status(cudaError_t e)
@@ -150,7 +150,7 @@ int stencil_batch_create_ex(stencil_batch *out, const stencil_batch_grid *grids,
         if (best < 0) rc = ST_ERR_UNSUPPORTED;
     }
     const int T = B->qT, V = B->qV;
-    const int halo = (T + 3) / 4 * 4, cx = 32 * V - 2 * halo;
+    const int halo = rc == ST_OK ? (T + V - 1) / V * V : 0, cx = 32 * V - 2 * halo;   // tb2d_halo
 
     // Buffers: pass 0 reads grid_in, the last pass writes grid_out, every pass between them
     // reads and writes two grid-sized scratch buffers with rows padded to 32 cells.  So the

@@ -115,10 +115,21 @@ cudaError_t lp_decode(int stor, const void *src, long long ld_q, const float2 *m
 // cc = 1 - 2cx - 2cy is exact, cz = sdc*Rz
 void hot_coeffs_src(const float *k, float *kf);
 
-// Hotspot source map dst = sdc*(p + amb*Rz) (rows ld_d floats apart), read by the contracted
-// kernels
+// Position of cell x of a source-map row inside its 8-cell group when every group of V cells
+// is stored in pair order: cell c < V/2 at 2c, cell c >= V/2 at 2(c - V/2) + 1.  A thread of the
+// contracted kernels works on the pairs (cell p, cell p + V/2), and reads them as they lie.
+template <int V>
+__host__ __device__ constexpr int src_pos(int x)
+{
+    const int c = x % V;
+    return x % 8 - c + (c < V / 2 ? 2 * c : 2 * (c - V / 2) + 1);
+}
+
+// Hotspot source map dst = sdc*(p + amb*Rz) in pair order for V cells per thread (4 or 8; rows
+// ld_d floats apart, 16-byte aligned, padded to whole 8-cell groups, the padding written as 0),
+// read by the contracted kernels
 cudaError_t hot_source(const float *p, long long ld_p, float *dst, long long ld_d, int nx, int ny,
-                       float amb, float rz, float sdc, cudaStream_t st);
+                       float amb, float rz, float sdc, int V, cudaStream_t st);
 
 bool tb2d_available(const Shape2D &s);
 int tb2d_block_threads(const Shape2D &s);

@@ -89,25 +89,36 @@ __global__ void __launch_bounds__(256) k_lp_decode(const uint16_t *__restrict__ 
 }
 
 // Hotspot source row: sdc*(p + amb*Rz), each operation rounded once; one block row per grid
-// row, four cells per thread (16-byte accesses when rows are aligned)
+// row, eight cells per thread (16-byte reads when rows are aligned).  Each group of V cells is
+// written in pair order (src_pos), cells past the row's end as 0; dst rows are padded to whole
+// 8-cell groups.
+template <int V>
 __global__ void __launch_bounds__(256) k_hot_source(const float *__restrict__ p, long long ld_p,
                                                     float *__restrict__ dst, long long ld_d, int nx,
                                                     float amb, float rz, float sdc, int vec)
 {
     const int y = blockIdx.y;
-    const int x = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
+    const int x = 8 * (blockIdx.x * blockDim.x + threadIdx.x);
     if (x >= nx) return;
     const float a = __fmul_rn(amb, rz);
     const float *src = p + (long long)y * ld_p + x;
-    float *d = dst + (long long)y * ld_d + x;
-    if (vec) {
-        const float4 v = *reinterpret_cast<const float4 *>(src);
-        *reinterpret_cast<float4 *>(d) =
-            make_float4(__fmul_rn(sdc, __fadd_rn(v.x, a)), __fmul_rn(sdc, __fadd_rn(v.y, a)),
-                        __fmul_rn(sdc, __fadd_rn(v.z, a)), __fmul_rn(sdc, __fadd_rn(v.w, a)));
+    float v[8], o[8];
+    if (vec && x + 8 <= nx) {
+        const float4 q0 = *reinterpret_cast<const float4 *>(src);
+        const float4 q1 = *reinterpret_cast<const float4 *>(src + 4);
+        v[0] = q0.x; v[1] = q0.y; v[2] = q0.z; v[3] = q0.w;
+        v[4] = q1.x; v[5] = q1.y; v[6] = q1.z; v[7] = q1.w;
+#pragma unroll
+        for (int j = 0; j < 8; j++) v[j] = __fmul_rn(sdc, __fadd_rn(v[j], a));
     } else {
-        for (int j = 0; j < 4 && x + j < nx; j++) d[j] = __fmul_rn(sdc, __fadd_rn(src[j], a));
+#pragma unroll
+        for (int j = 0; j < 8; j++) v[j] = x + j < nx ? __fmul_rn(sdc, __fadd_rn(src[j], a)) : 0.f;
     }
+#pragma unroll
+    for (int j = 0; j < 8; j++) o[src_pos<V>(j)] = v[j];
+    float *d = dst + (long long)y * ld_d + x;
+    *reinterpret_cast<float4 *>(d) = make_float4(o[0], o[1], o[2], o[3]);
+    *reinterpret_cast<float4 *>(d + 4) = make_float4(o[4], o[5], o[6], o[7]);
 }
 
 }  // namespace
@@ -145,17 +156,19 @@ void hot_coeffs_src(const float *k, float *kf)
 }
 
 cudaError_t hot_source(const float *p, long long ld_p, float *dst, long long ld_d, int nx, int ny,
-                       float amb, float rz, float sdc, cudaStream_t st)
+                       float amb, float rz, float sdc, int V, cudaStream_t st)
 {
-    if (nx < 1 || ny < 1) return cudaErrorInvalidValue;
-    const int vec = ((uintptr_t)p % 16 == 0) && ((uintptr_t)dst % 16 == 0) && (nx % 4 == 0) &&
-                    (ld_p % 4 == 0) && (ld_d % 4 == 0);
-    const unsigned bx = (unsigned)((nx + 1023) / 1024);
+    if (nx < 1 || ny < 1 || (V != 4 && V != 8) || (uintptr_t)dst % 16 || ld_d % 8 ||
+        ld_d < ((long long)nx + 7) / 8 * 8)
+        return cudaErrorInvalidValue;
+    const int vec = ((uintptr_t)p % 16 == 0) && (ld_p % 4 == 0);
+    const unsigned bx = (unsigned)(((long long)nx + 2047) / 2048);
     // grid rows beyond the 65535 limit of gridDim.y go in slices
     for (long long y0 = 0; y0 < ny; y0 += 65535) {
         const unsigned rows = (unsigned)std::min<long long>(65535, ny - y0);
-        k_hot_source<<<dim3(bx, rows), 256, 0, st>>>(p + y0 * ld_p, ld_p, dst + y0 * ld_d, ld_d, nx,
-                                                     amb, rz, sdc, vec);
+        const auto k = V == 8 ? k_hot_source<8> : k_hot_source<4>;
+        k<<<dim3(bx, rows), 256, 0, st>>>(p + y0 * ld_p, ld_p, dst + y0 * ld_d, ld_d, nx, amb, rz,
+                                          sdc, vec);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }

@@ -19,7 +19,7 @@ static const Tb2dEntry *tb2d_find(const Shape2D &s)
 bool tb2d_available(const Shape2D &s) { return tb2d_find(s) != nullptr; }
 int tb2d_block_threads(const Shape2D &s) { return 32 * (s.W > 0 ? s.W : 1); }   // W <= 0: one warp
 int tb2d_tile_width(const Shape2D &s) { return 32 * s.V * (s.W > 0 ? s.W : 1); }
-int tb2d_halo(const Shape2D &s) { return (s.T + 3) / 4 * 4; }
+int tb2d_halo(const Shape2D &s) { return (s.T + s.V - 1) / s.V * s.V; }
 
 size_t tb2d_smem_bytes(const Shape2D &s)
 {

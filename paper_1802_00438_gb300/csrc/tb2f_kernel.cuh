@@ -24,15 +24,29 @@
 // issued as 5 and 6 operations; the plain-power Hotspot instances of the allocation-free entry
 // point issue 9).
 //
+// Packed arithmetic: every operation works on a pair of cells (fma.rn.f32x2 and its add and
+// multiply; each half is rounded like the scalar operation, so the results are the same bits).
+// The kernel is bound by instruction issue, not by the FMA pipe: a packed operation holds the
+// pipe for two cycles but takes one issue slot, and leaves the other to the shuffles, loads and
+// integer work.  A pair is cells p and p + V/2 of a thread, not neighbours: then the west and
+// east neighbours of a pair are the pairs p-1 and p+1 as they lie, and only the two outermost
+// pairs mix halves (pairs of adjacent cells would need ten register moves per eight cells and
+// stage).  Field rows, read once per pass from the ring, are paired by register moves; the
+// source map, read again by every stage, is stored in pair order (src_pos), so that a 16-byte
+// load yields two pairs.  Stage 0 keeps partial rows like the others: it reads one ring row per
+// iteration (the direct form read three, and would have to pair each).
+// Measured (GB300), before -> after: 16384^2 Hotspot 2928 -> 3045 GCell/s, diffusion 3753 ->
+// 4132, 8192^2 Hotspot with bf16 storage 2032 -> 2430, 3001 x 2003 Hotspot 1053 -> 1248.
+// What bounds it now (ncu, 6144^2): Hotspot FMA pipe 58 % busy, issue 57 %, shared memory 64 %
+// (every stage reads its source row), two warps per scheduler; diffusion 58 / 52 / 30 %.
+//
 // GPU mapping: one warp per block; a tile is BX = 32*V cells wide incl. halos of
 // H = roundup(T, 4) cells per side; thread = V consecutive cells; x-neighbours of a thread's
 // edge cells by shuffle (the warp edge is the tile edge, inside the halo).  Field and power
 // rows arrive through shared-memory rings filled by cp.async PF rows ahead.  The power ring
-// keeps a mirrored copy of its first PW-1 slots, so the PW = max(T, 2) power rows an
-// iteration reads are
-// consecutive slots: one base address per row, constant offsets per stage.  Stage 0 needs no
-// partial rows: its three time-0 rows are all in the field ring, and it evaluates the update
-// from them directly.
+// keeps a mirrored copy of its first PW-1 slots, so the PW = T + 1 power rows an iteration may
+// read are consecutive slots: one base address per row, constant offsets per stage.  The power
+// rows run one row ahead of the field rows (receiving row y, a stage starts row y+1).
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -53,18 +67,26 @@ __host__ __device__ constexpr bool stor_all(int s) { return (s & STOR_ALL) != 0;
 template <int KIND, int T, int V, int STOR = STOR_F32>
 struct TB2F {
     static constexpr int BX = 32 * V;
-    static constexpr int H = (T + 3) / 4 * 4;
+    // a multiple of V: tile origins and x = 0 then fall on a lane's first cell, and the source
+    // map's V-cell groups (pair order) on lanes, for every T of a plan
+    static constexpr int H = (T + V - 1) / V * V;
     static constexpr int CX = BX - 2 * H;
     static constexpr int PF = 4;                                    // rows requested ahead
-    // 16-bit storage: the rows in flight wait in the staging rings, so the float rings hold
-    // only the rows in use (decoded on arrival); float32 rows land in the float rings directly
+    // 16-bit storage: the rows in flight wait in the staging rings and are decoded on arrival,
+    // a field row into registers, a power row into the float ring; float32 rows land in the
+    // float rings directly
     static constexpr bool Q16 = stor_fmt(STOR) != STOR_F32;
-    static constexpr int NBF = Q16 ? 3 : PF + 3;                    // field rows i-2 .. i(+PF)
-    static constexpr int PW = T > 1 ? T : 2;                        // power rows read per row:
-                                                                    // i-PW+1 .. i
-    static constexpr int NBP = (KIND == KTHERM) ? (Q16 ? PW : PW + PF + 1) : 0;   // power ring
+    static constexpr int NBF = Q16 ? 0 : PF + 1;                    // field rows i .. i+PF
+    static constexpr int PW = T + 1;                                // power rows in use:
+                                                                    // i-T+1 .. i+1
+    static constexpr int NBP = (KIND == KTHERM) ? (Q16 ? PW : PW + PF) : 0;       // power ring
     static constexpr int NBPX = (KIND == KTHERM) ? (NBP + PW - 1) : 0;  // incl. mirror
-    static constexpr int NS = T > 1 ? T - 1 : 1;                    // partial-sum stages
+    static constexpr int NS = T;                                    // partial-sum stages
+    static constexpr int HV = V / 2;                                // packed pairs per thread
+    // the power ring holds the source map with each V-cell group in pair order (src_pos), so
+    // a 16-byte load yields two packed pairs; plain-power rows and float32 field rows arrive in
+    // grid order
+    static constexpr bool PPAIR = stor_src(STOR);
     static constexpr int ROWB = BX * 4;                             // bytes per ring row
     // 16-bit storage: rows arrive raw (32-byte header of block codes + 2 bytes per cell) in a
     // staging ring of PF+1 rows per input and are decoded into the float rings once
@@ -73,16 +95,14 @@ struct TB2F {
     static constexpr size_t SMEM = (size_t)(NBF + NBPX) * ROWB +
                                    (size_t)NBR * RAWB * (KIND == KTHERM ? 2 : 1);
     static_assert(V % 4 == 0 && V <= 8, "V must be 4 or 8");
-    // 16-bit storage: a lane decodes its V cells with one block code, so block boundaries
-    // (every CX cells from the tile's first compute cell, H cells in) must fall between lanes
-    static_assert(stor_fmt(STOR) == STOR_F32 || H % V == 0, "16-bit blocks split a lane's cells");
     static_assert(CX > 0, "tile narrower than its halos");
 };
 
+// Coefficients as pairs of equal values, the operands of the packed float32 operations.
 struct CoefF {
     // diffusion: cc, cw, ce, cs, cn; Hotspot: sdc, Rx, Ry, Rz, amb, sdc*Ry, -2*Ry; source-map
-    // Hotspot kernels (STOR_SRC): cc, cx, cy, cz, amb, cy, 0 (host-made, hot_coeffs_src)
-    float a0, a1, a2, a3, a4, a5, a6;
+    // Hotspot kernels (STOR_SRC): cc, cx, cy, -cz, amb, cy, 0 (host-made, hot_coeffs_src)
+    float2 a0, a1, a2, a3, a4, a5, a6;
 };
 
 __device__ __forceinline__ float4 lds128(uint32_t a)
@@ -189,7 +209,6 @@ struct CtxF {
     int lane;
     uint32_t oq[2];        // byte offsets in a ring row of my cells' 16-byte chunks
     uint32_t wq[2];        // byte offsets of the chunks I copy into a ring row
-    uint32_t ow4, oe4;     // byte offsets of the cells left and right of mine (clamped)
     // 16-bit storage
     uint32_t sRF, sRP;     // staging rings (raw field / raw power rows)
     const uint16_t *qin, *qpw;
@@ -203,49 +222,70 @@ struct CtxF {
     long long st_stride;
 };
 
-// my V cells of the ring row at byte address row
-template <int V>
-__device__ __forceinline__ void lds_row(uint32_t row, const CtxF &c, float (&v)[V])
+// my V cells of the ring row at byte address row, as pairs: (x, y) of v[p] are cells p and
+// p + V/2.  PAIR: the row is stored in pair order, each 16-byte load is two pairs as they are.
+template <int V, bool PAIR>
+__device__ __forceinline__ void lds_row(uint32_t row, const CtxF &c, float2 (&v)[V / 2])
 {
-#pragma unroll
-    for (int q = 0; q < V / 4; q++) {
-        const float4 t = lds128(row + c.oq[q]);
-        v[4 * q] = t.x; v[4 * q + 1] = t.y; v[4 * q + 2] = t.z; v[4 * q + 3] = t.w;
+    const float4 a = lds128(row + c.oq[0]);
+    if (V == 8) {
+        const float4 b = lds128(row + c.oq[1]);
+        if (PAIR) {
+            v[0] = make_float2(a.x, a.y);
+            v[1] = make_float2(a.z, a.w);
+            v[V / 2 - 2] = make_float2(b.x, b.y);
+            v[V / 2 - 1] = make_float2(b.z, b.w);
+        } else {
+            v[0] = make_float2(a.x, b.x);
+            v[1] = make_float2(a.y, b.y);
+            v[V / 2 - 2] = make_float2(a.z, b.z);
+            v[V / 2 - 1] = make_float2(a.w, b.w);
+        }
+    } else {
+        v[0] = PAIR ? make_float2(a.x, a.y) : make_float2(a.x, a.z);
+        v[1] = PAIR ? make_float2(a.z, a.w) : make_float2(a.y, a.w);
     }
 }
 
-template <int V, bool EDGE>
-__device__ __forceinline__ void nbf(const CtxF &c, const float (&d)[V], float w_in, float e_in,
-                                    float (&dw)[V], float (&de)[V])
+// cell j of a thread's packed row
+template <int H>
+__device__ __forceinline__ float cell(const float2 (&v)[H], int j)
 {
-    dw[0] = w_in;
-    de[V - 1] = e_in;
+    return j < H ? v[j].x : v[j - H].y;
+}
+
+// Clamped edges of a packed row, before its neighbours are formed: in a warp that holds
+// x = nx-1 the ghost cell to its right takes the edge cell's value (a ghost's own value is
+// never used), or e_in when the edge is the lane's last cell; x = 0 is always a lane's cell 0
+// (tile origins are multiples of V), whose west value is its own.
+template <int V>
+__device__ __forceinline__ void edge_fix(const CtxF &c, float2 (&d)[V / 2], float &w_in, float &e_in)
+{
+    constexpr int H = V / 2;
+    e_in = ((c.rmask >> (V - 1)) & 1u) ? d[H - 1].y : e_in;
+    w_in = (c.lmask & 1u) ? d[0].x : w_in;
 #pragma unroll
-    for (int j = 1; j < V; j++) dw[j] = d[j - 1];
-#pragma unroll
-    for (int j = 0; j < V - 1; j++) de[j] = d[j + 1];
-    if (EDGE) {
-#pragma unroll
-        for (int j = 0; j < V; j++) {
-            dw[j] = ((c.lmask >> j) & 1u) ? d[j] : dw[j];
-            de[j] = ((c.rmask >> j) & 1u) ? d[j] : de[j];
-        }
+    for (int j = V - 2; j >= 0; j--) {
+        const bool g = (c.rmask >> j) & 1u;
+        const float edge = cell(d, j);
+        if (j + 1 < H) d[j + 1 < H ? j + 1 : 0].x = g ? edge : d[j + 1 < H ? j + 1 : 0].x;
+        else d[j + 1 < H ? 0 : j + 1 - H].y = g ? edge : d[j + 1 < H ? 0 : j + 1 - H].y;
     }
 }
 
 // Start row y+1: Xq = its north term (+ its power for Hotspot), written over the finished P.
-template <int KIND, int V>
-__device__ __forceinline__ void qf(const CtxF &c, const CoefF &k, const float (&d)[V],
-                                   uint32_t p_next, float (&Xq)[V])
+template <int KIND, int V, bool PPAIR>
+__device__ __forceinline__ void qf(const CtxF &c, const CoefF &k, const float2 (&d)[V / 2],
+                                   uint32_t p_next, float2 (&Xq)[V / 2])
 {
     if (KIND == KDIFF) {
 #pragma unroll
-        for (int j = 0; j < V; j++) Xq[j] = __fmul_rn(k.a4, d[j]);
+        for (int j = 0; j < V / 2; j++) Xq[j] = __fmul2_rn(k.a4, d[j]);
     } else {
-        float p[V];
-        lds_row<V>(p_next, c, p);
+        float2 p[V / 2];
+        lds_row<V, PPAIR>(p_next, c, p);
 #pragma unroll
-        for (int j = 0; j < V; j++) Xq[j] = __fmaf_rn(k.a2, d[j], p[j]);
+        for (int j = 0; j < V / 2; j++) Xq[j] = __ffma2_rn(k.a2, d[j], p[j]);
     }
 }
 
@@ -255,63 +295,75 @@ __device__ __forceinline__ void qf(const CtxF &c, const CoefF &k, const float (&
 // SWAP = true: P' is built on top of Q in Xq and Q' is written to Xp (the caller alternates the
 // arrays every row).  SWAP = false: P' goes back to Xp and Q' to Xq (no alternation; the
 // register allocator decides whether that needs copies).
-template <int KIND, int V, int MODE, bool SWAP, bool SRC = false>
-__device__ __forceinline__ void stf(const CtxF &c, const CoefF &k, int y, bool fwd, float (&Xp)[V],
-                                    float (&Xq)[V], const float (&d)[V], float w_in, float e_in,
-                                    uint32_t p_y, uint32_t p_next, float (&out)[V])
+template <int KIND, int V, int MODE, bool SWAP, int STOR>
+__device__ __forceinline__ void stf(const CtxF &c, const CoefF &k, int y, bool fwd,
+                                    float2 (&Xp)[V / 2], float2 (&Xq)[V / 2], float2 (&d)[V / 2],
+                                    uint32_t p_y, uint32_t p_next, float2 (&out)[V / 2])
 {
+    constexpr int H = V / 2;
     constexpr bool SP = MODE == MODE_SPECIAL;
     constexpr bool ED = MODE != MODE_PLAIN;
+    constexpr bool PPAIR = stor_src(STOR);
     if (SP && fwd) {   // beyond this pass's step count: row y-1 of time s passes unchanged
 #pragma unroll
-        for (int j = 0; j < V; j++) {
+        for (int j = 0; j < H; j++) {
             out[j] = Xp[j];
             if (SWAP) Xq[j] = d[j];   // becomes "P" of the next row: forwarded one row later
             else Xp[j] = d[j];
         }
         return;
     }
-    const float cs = (KIND == KDIFF) ? k.a3 : k.a5;
+    const float2 cs = (KIND == KDIFF) ? k.a3 : k.a5;
 #pragma unroll
-    for (int j = 0; j < V; j++) out[j] = __fmaf_rn(cs, d[j], Xp[j]);
+    for (int j = 0; j < H; j++) out[j] = __ffma2_rn(cs, d[j], Xp[j]);
     if (SP && y == c.ny) {   // row ny-1 was completed on arrival (its south is itself)
 #pragma unroll
-        for (int j = 0; j < V; j++) out[j] = Xp[j];
+        for (int j = 0; j < H; j++) out[j] = Xp[j];
     }
-    if (SP && y == 0) qf<KIND, V>(c, k, d, p_y, Xq);   // top: the row above row 0 is row 0
-    float dw[V], de[V];
-    nbf<V, ED>(c, d, w_in, e_in, dw, de);
-    float(&Pn)[V] = SWAP ? Xq : Xp;   // where row y's P goes
-    float(&Qn)[V] = SWAP ? Xp : Xq;   // where row y+1's Q goes
-    if (KIND == KDIFF) {
+    if (SP && y == 0) qf<KIND, V, PPAIR>(c, k, d, p_y, Xq);   // top: the row above row 0 is row 0
+    // x-neighbours: west of pair p is pair p-1, east of pair p is pair p+1; only the outermost
+    // pairs take a value from the neighbour lane and one across the halves
+    float w_in = __shfl_sync(0xffffffffu, d[H - 1].y, (c.lane + 31) & 31);
+    float e_in = __shfl_sync(0xffffffffu, d[0].x, (c.lane + 1) & 31);
+    if (ED) edge_fix<V>(c, d, w_in, e_in);
+    float2(&Pn)[H] = SWAP ? Xq : Xp;   // where row y's P goes
+    float2(&Qn)[H] = SWAP ? Xp : Xq;   // where row y+1's Q goes
 #pragma unroll
-        for (int j = 0; j < V; j++) {
-            Pn[j] = __fmaf_rn(k.a0, d[j], Xq[j]);
-            Pn[j] = __fmaf_rn(k.a1, dw[j], Pn[j]);
-            Pn[j] = __fmaf_rn(k.a2, de[j], Pn[j]);
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < V; j++) {
-            if (SRC) {
+    for (int j = 0; j < H; j++) {
+        constexpr int L = H - 1;
+        const float2 dw = j > 0 ? d[j > 0 ? j - 1 : 0] : make_float2(w_in, d[L].x);
+        const float2 de = j < L ? d[j < L ? j + 1 : j] : make_float2(d[0].y, e_in);
+        if (KIND == KDIFF) {
+            float2 t = __ffma2_rn(k.a0, d[j], Xq[j]);
+            t = __ffma2_rn(k.a1, dw, t);
+            Pn[j] = __ffma2_rn(k.a2, de, t);
+        } else {
+            // the outermost pairs add their halves one by one: building a pair for the packed
+            // addition would cost as many register moves (16384^2 Hotspot 2967 -> 3045 GCell/s)
+            float2 ew;
+            if (j == 0 || j == L)
+                ew = make_float2(__fadd_rn(de.x, dw.x), __fadd_rn(de.y, dw.y));
+            else
+                ew = __fadd2_rn(de, dw);
+            if (stor_src(STOR)) {
                 // Q (cy*n + src) + cx*(e + w) + cc*c - cz*c: the expanded weights, cc exact
-                Pn[j] = __fmaf_rn(k.a1, __fadd_rn(de[j], dw[j]), Xq[j]);
-                Pn[j] = __fmaf_rn(k.a0, d[j], Pn[j]);
-                Pn[j] = __fmaf_rn(-k.a3, d[j], Pn[j]);
+                float2 t = __ffma2_rn(k.a1, ew, Xq[j]);
+                t = __ffma2_rn(k.a0, d[j], t);
+                Pn[j] = __ffma2_rn(k.a3, d[j], t);
             } else {
-                const float t2 = __fmaf_rn(-2.0f, d[j], __fadd_rn(de[j], dw[j]));
-                Pn[j] = __fmaf_rn(t2, k.a1, Xq[j]);
-                const float t3 = __fsub_rn(k.a4, d[j]);
-                Pn[j] = __fmaf_rn(t3, k.a3, Pn[j]);
-                Pn[j] = __fmaf_rn(k.a6, d[j], Pn[j]);
-                Pn[j] = __fmaf_rn(k.a0, Pn[j], d[j]);
+                const float2 t2 = __ffma2_rn(make_float2(-2.0f, -2.0f), d[j], ew);
+                float2 t = __ffma2_rn(t2, k.a1, Xq[j]);
+                const float2 t3 = __ffma2_rn(make_float2(-1.0f, -1.0f), d[j], k.a4);   // amb - c
+                t = __ffma2_rn(t3, k.a3, t);
+                t = __ffma2_rn(k.a6, d[j], t);
+                Pn[j] = __ffma2_rn(k.a0, t, d[j]);
             }
         }
     }
-    qf<KIND, V>(c, k, d, p_next, Qn);
+    qf<KIND, V, PPAIR>(c, k, d, p_next, Qn);
     if (SP && y == c.ny - 1) {   // bottom: complete row ny-1 now with south = itself
 #pragma unroll
-        for (int j = 0; j < V; j++) Pn[j] = __fmaf_rn(cs, d[j], Pn[j]);
+        for (int j = 0; j < H; j++) Pn[j] = __ffma2_rn(cs, d[j], Pn[j]);
     }
 }
 
@@ -319,8 +371,9 @@ __device__ __forceinline__ void stf(const CtxF &c, const CoefF &k, int y, bool f
 struct RowF {
     const float *gF, *gP;   // field / power pointers at column x0 + 4*lane of the next row to load
     float *gO;              // output pointer at my first cell of the next row to store
-    int colq[4];            // per 16-byte chunk: column offset to copy from (0 when off-grid)
-    int nbq[4];             // per chunk: bytes inside the grid (0..16)
+    int colq[2];            // per 16-byte chunk: column offset to copy from (0 when off-grid)
+    int nbq[2];             // per chunk: bytes inside the grid (0..16)
+    int colp[2], nbp[2];    // the same for source-map rows (pair order, padded rows)
     int rf, rp;             // ring slots of field row i / of power row i
     int i_store;            // first iteration that stores a row
     int i_load_end;         // iterations i < i_load_end queue row i+PF
@@ -334,96 +387,59 @@ struct RowF {
     int colr;
 };
 
+// my cells of the compute block to g (row-major, cell 0 at g)
+template <int V>
+__device__ __forceinline__ void st_cells(const CtxF &c, float *g, const float2 (&v)[V / 2])
+{
+    if (c.st_full) {
+#pragma unroll
+        for (int q = 0; q < V / 4; q++)
+            *reinterpret_cast<float4 *>(g + 4 * q) = make_float4(
+                cell(v, 4 * q), cell(v, 4 * q + 1), cell(v, 4 * q + 2), cell(v, 4 * q + 3));
+    } else if (c.st_any) {
+#pragma unroll
+        for (int j = 0; j < V; j++)
+            if (j >= c.st_lo && j < c.st_hi) g[j] = cell(v, j);
+    }
+}
+
 // Trajectory passes: the row `row` of step t+1 of the pass (stage t's output) into state t,
 // for the steps before the pass's last (whose rows go to the pass output) and the rows of
 // this segment, compute-block cells only.
 template <int V>
-__device__ __forceinline__ void tbf_store_state(const CtxF &c, int t, int row, const float (&v)[V])
+__device__ __forceinline__ void tbf_store_state(const CtxF &c, int t, int row,
+                                                const float2 (&v)[V / 2])
 {
     if (t >= c.tsteps - 1 || row < c.s0 || row >= c.s1) return;
     float *g = c.st_states + (long long)t * c.st_stride + (long long)row * c.ld_out + c.xt;
-    if (c.st_full) {
-#pragma unroll
-        for (int q = 0; q < V / 4; q++)
-            *reinterpret_cast<float4 *>(g + 4 * q) =
-                make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-    } else if (c.st_any) {
-#pragma unroll
-        for (int j = 0; j < V; j++)
-            if (j >= c.st_lo && j < c.st_hi) g[j] = v[j];
-    }
+    st_cells<V>(c, g, v);
 }
 
-// One row iteration.  PH selects which of A/B holds P (PH = 0: A) for every stage.
+// One row iteration.  PH selects which of A/B holds P (PH = 0: A) for every stage.  Stage s
+// receives row R0-s of time s (stage 0: row R0 in `out`) and emits row R0-s-1 of time s+1 in
+// `out`; pbase is the slot of power row R0+1, row R0+1-t sits t slots below it.
 template <int KIND, int T, int V, int MODE, int PH, bool SWAP, int STOR>
 __device__ __forceinline__ void tbf_iter(const CtxF &c, const CoefF &k,
-                                         float (&A)[TB2F<KIND, T, V>::NS][V],
-                                         float (&B)[TB2F<KIND, T, V>::NS][V], int i,
-                                         uint32_t fu, uint32_t fm, uint32_t fd, uint32_t pbase,
-                                         float *gO, const RowF &r, bool store)
+                                         float2 (&A)[TB2F<KIND, T, V>::NS][V / 2],
+                                         float2 (&B)[TB2F<KIND, T, V>::NS][V / 2], int i,
+                                         float2 (&out)[V / 2], uint32_t pbase, float *gO,
+                                         const RowF &r, bool store)
 {
     using C = TB2F<KIND, T, V, STOR>;
-    constexpr bool ED = MODE != MODE_PLAIN;
     const int R0 = c.y_start + i;
-    float d[V], out[V];
-    // stage 0: row R0-1 at time 1 straight from the time-0 rows R0-2, R0-1, R0 in the ring
-    // (fu, fm, fd are those rows, already clamped to the grid for the boundary rows)
-    {
-        float u[V], m[V], dd[V], w[V], e[V];
-        lds_row<V>(fu, c, u);
-        lds_row<V>(fm, c, m);
-        lds_row<V>(fd, c, dd);
-        nbf<V, ED>(c, m, lds32(fm + c.ow4), lds32(fm + c.oe4), w, e);
-        if (KIND == KDIFF) {
+    float2 d[V / 2];
 #pragma unroll
-            for (int j = 0; j < V; j++)
-                out[j] = diff5<false>(m[j], w[j], e[j], dd[j], u[j], k.a0, k.a1, k.a2, k.a3, k.a4);
-        } else {
-            float pv[V];
-            lds_row<V>(pbase - C::ROWB, c, pv);   // power of row R0-1
-            if (stor_src(STOR)) {
-                // the source-map form of the Hotspot update (see stf): src + cx*(e + w) +
-                // cy*(n + s) + cc*c - cz*c
+    for (int s = 0; s < T; s++) {
 #pragma unroll
-                for (int j = 0; j < V; j++) {
-                    float q = __fmaf_rn(k.a1, __fadd_rn(e[j], w[j]), pv[j]);
-                    q = __fmaf_rn(k.a2, __fadd_rn(u[j], dd[j]), q);
-                    q = __fmaf_rn(k.a0, m[j], q);
-                    out[j] = __fmaf_rn(-k.a3, m[j], q);
-                }
-            } else {
-#pragma unroll
-                for (int j = 0; j < V; j++)
-                    out[j] = hot2<false>(m[j], w[j], e[j], dd[j], u[j], pv[j], k.a0, k.a1, k.a2,
-                                         k.a3, k.a4);
-            }
-        }
-    }
-    // stages 1 .. T-1: stage s receives row R0-s of time s; pbase is the slot of power row
-    // R0 (ring-relative i), row i-t sits t slots below it
-#pragma unroll
-    for (int s = 1; s < T; s++) {
-        if (stor_all(STOR)) tbf_store_state<V>(c, s - 1, R0 - s, out);
-#pragma unroll
-        for (int j = 0; j < V; j++) d[j] = out[j];
-        const float w_in = __shfl_sync(0xffffffffu, d[V - 1], (c.lane + 31) & 31);
-        const float e_in = __shfl_sync(0xffffffffu, d[0], (c.lane + 1) & 31);
-        stf<KIND, V, MODE, SWAP, stor_src(STOR)>(c, k, R0 - s, s >= c.tsteps, PH == 0 ? A[s - 1] : B[s - 1],
-                                 PH == 0 ? B[s - 1] : A[s - 1], d, w_in, e_in,
-                           pbase - s * C::ROWB, pbase - (s - 1) * C::ROWB, out);
+        for (int j = 0; j < V / 2; j++) d[j] = out[j];
+        stf<KIND, V, MODE, SWAP, STOR>(c, k, R0 - s, s >= c.tsteps, PH == 0 ? A[s] : B[s],
+                                       PH == 0 ? B[s] : A[s], d, pbase - (s + 1) * C::ROWB,
+                                       pbase - s * C::ROWB, out);
+        if (stor_all(STOR) && s < T - 1) tbf_store_state<V>(c, s, R0 - s - 1, out);
     }
     if (store) {
         if (stor_fmt(STOR) == STOR_F32) {
-            if (c.st_full) {
-#pragma unroll
-                for (int q = 0; q < V / 4; q++)
-                    *reinterpret_cast<float4 *>(gO + 4 * q) =
-                        make_float4(out[4 * q], out[4 * q + 1], out[4 * q + 2], out[4 * q + 3]);
-            } else if (c.st_any) {
-#pragma unroll
-                for (int j = 0; j < V; j++)
-                    if (j >= c.st_lo && j < c.st_hi) gO[j] = out[j];
-            }
+            st_cells<V>(c, gO, out);
         } else {
             // encode the row segment of this tile as q = x - offset with the offset the value of
             // the block's first cell (tile column tx*CX: lane H/V, its cell 0, in the grid for
@@ -431,10 +447,11 @@ __device__ __forceinline__ void tbf_iter(const CtxF &c, const CoefF &k,
             // (11) significant bits of each cell's distance from the offset at any magnitude:
             // the error per cell is at most half an ulp of |x - offset| <= the block's spread,
             // and no block-wide minimum and maximum are needed
-            const float mid = __shfl_sync(0xffffffffu, out[0], C::H / V);
+            const float mid = __shfl_sync(0xffffffffu, out[0].x, C::H / V);
             unsigned q2[V / 2];   // pairs of codes, cell 2i in the low half
 #pragma unroll
-            for (int j = 0; j < V / 2; j++) q2[j] = f2q2<STOR>(out[2 * j] - mid, out[2 * j + 1] - mid);
+            for (int j = 0; j < V / 2; j++) 
+                q2[j] = f2q2<STOR>(cell(out, 2 * j) - mid, cell(out, 2 * j + 1) - mid);
             if (c.st_full) {
 #pragma unroll
                 for (int t = 0; t < V / 4; t++)
@@ -450,34 +467,54 @@ __device__ __forceinline__ void tbf_iter(const CtxF &c, const CoefF &k,
     }
 }
 
-// Decode my V cells of a staged raw row (header: codes of the blocks tx-1, tx, tx+1) into a
-// float ring row (and into its mirror when mirror != 0).
+// Decode my V cells of a staged raw row (header: codes of the blocks tx-1, tx, tx+1).
 template <int V, int STOR>
-__device__ __forceinline__ void tbf_decode(const CtxF &c, uint32_t raw, uint32_t dst, uint32_t mirror)
+__device__ __forceinline__ void tbf_decode(const CtxF &c, uint32_t raw, float2 (&x)[V / 2])
 {
     const uint2 cw = lds64u(raw + 8u * c.msel);
-    const float mid = __uint_as_float(cw.x), sc = __uint_as_float(cw.y);
+    const float2 mid = make_float2(__uint_as_float(cw.x), __uint_as_float(cw.x));
+    const float2 sc = make_float2(__uint_as_float(cw.y), __uint_as_float(cw.y));
+    constexpr int H = V / 2;
+    float q[V];
 #pragma unroll
     for (int t = 0; t < V / 4; t++) {
         const uint2 w = lds64u(raw + 32u + 2u * V * c.lane + 8u * t);
-        float x0 = __fmaf_rn(sc, q2f<STOR>(w.x & 0xffffu), mid);
-        float x1 = __fmaf_rn(sc, q2f<STOR>(w.x >> 16), mid);
-        float x2 = __fmaf_rn(sc, q2f<STOR>(w.y & 0xffffu), mid);
-        float x3 = __fmaf_rn(sc, q2f<STOR>(w.y >> 16), mid);
-        sts128(dst + c.oq[t], x0, x1, x2, x3);
-        if (mirror) sts128(mirror + c.oq[t], x0, x1, x2, x3);
+        q[4 * t] = q2f<STOR>(w.x & 0xffffu);
+        q[4 * t + 1] = q2f<STOR>(w.x >> 16);
+        q[4 * t + 2] = q2f<STOR>(w.y & 0xffffu);
+        q[4 * t + 3] = q2f<STOR>(w.y >> 16);
+    }
+#pragma unroll
+    for (int j = 0; j < H; j++) x[j] = __ffma2_rn(sc, make_float2(q[j], q[j + H]), mid);
+}
+
+// ... into a power ring row in pair order (and into its mirror when mirror != 0)
+template <int V, int STOR>
+__device__ __forceinline__ void tbf_decode_ring(const CtxF &c, uint32_t raw, uint32_t dst,
+                                                uint32_t mirror)
+{
+    float2 x[V / 2];
+    tbf_decode<V, STOR>(c, raw, x);
+#pragma unroll
+    for (int t = 0; t < V / 4; t++) {
+        sts128(dst + c.oq[t], x[2 * t].x, x[2 * t].y, x[2 * t + 1].x, x[2 * t + 1].y);
+        if (mirror) sts128(mirror + c.oq[t], x[2 * t].x, x[2 * t].y, x[2 * t + 1].x, x[2 * t + 1].y);
     }
 }
 
-// Queue tile row (row pointers in r) into field slot lf and power slot lp (plus its mirror);
-// with 16-bit storage, into staging slot lr instead.
+// Queue the next field row (pointers in r, if f) into field slot lf and the next power row
+// (if pw) into power slot lp plus its mirror; with 16-bit storage, both into staging slot lr
+// instead.  The power rows run one row ahead of the field rows (a stage that receives row y
+// starts row y+1).  Advances the row pointers.
 template <int KIND, int T, int V, int STOR>
-__device__ __forceinline__ void tbf_queue(const CtxF &c, const RowF &r, int lf, int lp, int lr)
+__device__ __forceinline__ void tbf_queue(const CtxF &c, RowF &r, bool f, bool pw, int lf, int lp,
+                                          int lr)
 {
     using C = TB2F<KIND, T, V, STOR>;
     if (stor_fmt(STOR) != STOR_F32) {
 #pragma unroll
         for (int in = 0; in < (KIND == KTHERM ? 2 : 1); in++) {
+            if (!(in == 0 ? f : pw)) continue;
             const uint32_t dr = (in == 0 ? c.sRF : c.sRP) + lr * C::RAWB;
             const uint16_t *src = in == 0 ? r.qF : r.qP;
             const float2 *m = in == 0 ? r.mF : r.mP;
@@ -490,66 +527,81 @@ __device__ __forceinline__ void tbf_queue(const CtxF &c, const RowF &r, int lf, 
                 const int b = min(max(c.tx - 1 + (c.lane >> 1), 0), c.ntx - 1);
                 cp4(dr + 4u * c.lane, reinterpret_cast<const float *>(m + b) + (c.lane & 1), 4);
             }
+            if (in == 0) {
+                r.qF += c.ld_q;
+                r.mF += c.ntx;
+            } else {
+                r.qP += c.ld_q;
+                r.mP += c.ntx;
+            }
         }
         return;
     }
     const uint32_t df = c.sF + lf * C::ROWB;
     const uint32_t dp = c.sP + lp * C::ROWB;
-    if (c.vec_in && (KIND == KDIFF || c.vec_pw)) {
+    if (f) {
+        if (c.vec_in) {
 #pragma unroll
-        for (int q = 0; q < V / 4; q++) {
-            cp16(df + c.wq[q], r.gF + r.colq[q], r.nbq[q]);
-            if (KIND == KTHERM) {
-                cp16(dp + c.wq[q], r.gP + r.colq[q], r.nbq[q]);
-                if (lp < C::PW - 1) cp16(dp + C::NBP * C::ROWB + c.wq[q], r.gP + r.colq[q], r.nbq[q]);
-            }
-        }
-    } else {   // rows not 16-byte aligned: element-wise copies
+            for (int q = 0; q < V / 4; q++) cp16(df + c.wq[q], r.gF + r.colq[q], r.nbq[q]);
+        } else {   // rows not 16-byte aligned: element-wise copies
 #pragma unroll
-        for (int q = 0; q < V / 4; q++)
+            for (int q = 0; q < V / 4; q++)
 #pragma unroll
-            for (int j = 0; j < 4; j++) {
-                const int nb = (4 * j < r.nbq[q]) ? 4 : 0;
-                const int col = nb ? r.colq[q] + j : 0;
-                cp4(df + c.wq[q] + 4 * j, r.gF + col, nb);
-                if (KIND == KTHERM) {
-                    cp4(dp + c.wq[q] + 4 * j, r.gP + col, nb);
-                    if (lp < C::PW - 1) cp4(dp + C::NBP * C::ROWB + c.wq[q] + 4 * j, r.gP + col, nb);
+                for (int j = 0; j < 4; j++) {
+                    const int nb = (4 * j < r.nbq[q]) ? 4 : 0;
+                    cp4(df + c.wq[q] + 4 * j, r.gF + (nb ? r.colq[q] + j : 0), nb);
                 }
+        }
+        r.gF += c.ld_in;
+    }
+    if (KIND == KTHERM && pw) {
+        // source-map rows are padded to 32 cells, every chunk of a group that reaches into the
+        // grid is whole (pair order puts the group's cells in both of its chunks)
+        if (C::PPAIR || c.vec_pw) {
+#pragma unroll
+            for (int q = 0; q < V / 4; q++) {
+                const int nb = C::PPAIR ? r.nbp[q] : r.nbq[q];
+                const float *src = r.gP + (C::PPAIR ? r.colp[q] : r.colq[q]);
+                cp16(dp + c.wq[q], src, nb);
+                if (lp < C::PW - 1) cp16(dp + C::NBP * C::ROWB + c.wq[q], src, nb);
             }
+        } else {
+#pragma unroll
+            for (int q = 0; q < V / 4; q++)
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    const int nb = (4 * j < r.nbq[q]) ? 4 : 0;
+                    const float *src = r.gP + (nb ? r.colq[q] + j : 0);
+                    cp4(dp + c.wq[q] + 4 * j, src, nb);
+                    if (lp < C::PW - 1) cp4(dp + C::NBP * C::ROWB + c.wq[q] + 4 * j, src, nb);
+                }
+        }
+        r.gP += c.ld_pw;
     }
 }
 
 // One row: wait for row i, run the stages, queue row i+PF, advance pointers and rings.
 template <int KIND, int T, int V, int MODE, int PH, bool SWAP, int STOR>
 __device__ __forceinline__ void tbf_step(const CtxF &c, const CoefF &k,
-                                         float (&A)[TB2F<KIND, T, V>::NS][V],
-                                         float (&B)[TB2F<KIND, T, V>::NS][V], int i, RowF &r)
+                                         float2 (&A)[TB2F<KIND, T, V>::NS][V / 2],
+                                         float2 (&B)[TB2F<KIND, T, V>::NS][V / 2], int i, RowF &r)
 {
     using C = TB2F<KIND, T, V, STOR>;
-    cp_async_wait<C::PF - 1>();   // row i has landed
+    cp_async_wait<C::PF - 1>();   // field row i and power row i+1 have landed
     __syncwarp();
-    if (stor_fmt(STOR) != STOR_F32) {       // decode row i into the float rings
-        tbf_decode<V, STOR>(c, c.sRF + r.rr * C::RAWB, c.sF + r.rf * C::ROWB, 0u);
+    float2 row[V / 2];
+    if (C::Q16) {
         if (KIND == KTHERM)   // (for STOR_SRC the coded map is the source map itself)
-            tbf_decode<V, STOR>(c, c.sRP + r.rr * C::RAWB, c.sP + r.rp * C::ROWB,
-                                r.rp < C::PW - 1 ? c.sP + (C::NBP + r.rp) * C::ROWB : 0u);
+            tbf_decode_ring<V, STOR>(c, c.sRP + r.rr * C::RAWB, c.sP + r.rp * C::ROWB,
+                                     r.rp < C::PW - 1 ? c.sP + (C::NBP + r.rp) * C::ROWB : 0u);
+        tbf_decode<V, STOR>(c, c.sRF + r.rr * C::RAWB, row);
         __syncwarp();
-    }
-    // field ring slots of rows i-2, i-1, i (rows above or below the grid clamp to its edge)
-    int su = r.rf - 2, sm = r.rf - 1, sd = r.rf;
-    su += (su < 0) ? C::NBF : 0;
-    sm += (sm < 0) ? C::NBF : 0;
-    if (MODE == MODE_SPECIAL) {
-        const int R = c.y_start + i - 1;    // stage 0's row
-        if (R == 0) su = sm;                // row -1 is row 0
-        if (R == c.ny - 1) sd = sm;         // row ny is row ny-1
+    } else {
+        lds_row<V, false>(c.sF + r.rf * C::ROWB, c, row);
     }
     const uint32_t pbase = c.sP + ((KIND == KTHERM && r.rp < C::PW - 1) ? C::NBP + r.rp : r.rp) * C::ROWB;
     const bool store = i >= r.i_store;
-    tbf_iter<KIND, T, V, MODE, PH, SWAP, STOR>(c, k, A, B, i, c.sF + su * C::ROWB,
-                                               c.sF + sm * C::ROWB, c.sF + sd * C::ROWB, pbase,
-                                               r.gO, r, store);
+    tbf_iter<KIND, T, V, MODE, PH, SWAP, STOR>(c, k, A, B, i, row, pbase, r.gO, r, store);
     if (store) {
         if (stor_fmt(STOR) == STOR_F32) r.gO += c.ld_out;
         else {
@@ -558,42 +610,27 @@ __device__ __forceinline__ void tbf_step(const CtxF &c, const CoefF &k,
         }
     }
     __syncwarp();
-    int lf = 0, lp = 0, lr = 0;   // slots of row i+PF: float rings, or the staging ring
+    int lf = 0, lp = 0, lr = 0;   // slots of rows i+PF (field), i+PF+1 (power), or the staging slot
     if (!C::Q16) {
-        lf = r.rf + C::PF;
-        lf -= (lf >= C::NBF) ? C::NBF : 0;
+        lf = r.rf == 0 ? C::NBF - 1 : r.rf - 1;   // row i-1's slot (NBF = PF + 1)
         if (KIND == KTHERM) {
             lp = r.rp + C::PF;
             lp -= (lp >= C::NBP) ? C::NBP : 0;
         }
     } else {
-        lr = r.rr + C::PF;
-        lr -= (lr >= C::NBR) ? C::NBR : 0;
+        lr = r.rr == 0 ? C::NBR - 1 : r.rr - 1;
     }
-    if (i < r.i_load_end) {
-        tbf_queue<KIND, T, V, STOR>(c, r, lf, lp, lr);
-        if (stor_fmt(STOR) == STOR_F32) {
-            r.gF += c.ld_in;
-            if (KIND == KTHERM) r.gP += c.ld_pw;
-        } else {
-            r.qF += c.ld_q;
-            r.mF += c.ntx;
-            if (KIND == KTHERM) {
-                r.qP += c.ld_q;
-                r.mP += c.ntx;
-            }
-        }
-    }
+    tbf_queue<KIND, T, V, STOR>(c, r, i < r.i_load_end, i + 1 < r.i_load_end, lf, lp, lr);
     cp_async_commit();
-    r.rf = (r.rf + 1 == C::NBF) ? 0 : r.rf + 1;
+    if (!C::Q16) r.rf = (r.rf + 1 == C::NBF) ? 0 : r.rf + 1;
     if (KIND == KTHERM) r.rp = (r.rp + 1 == C::NBP) ? 0 : r.rp + 1;
-    if (stor_fmt(STOR) != STOR_F32) r.rr = (r.rr + 1 == C::NBR) ? 0 : r.rr + 1;
+    if (C::Q16) r.rr = (r.rr + 1 == C::NBR) ? 0 : r.rr + 1;
 }
 
 template <int KIND, int T, int V, int MODE, bool SWAP, int STOR>
 __device__ __forceinline__ void tbf_step_rt(const CtxF &c, const CoefF &k,
-                                            float (&A)[TB2F<KIND, T, V>::NS][V],
-                                            float (&B)[TB2F<KIND, T, V>::NS][V], int i, RowF &r)
+                                            float2 (&A)[TB2F<KIND, T, V>::NS][V / 2],
+                                            float2 (&B)[TB2F<KIND, T, V>::NS][V / 2], int i, RowF &r)
 {
     if (SWAP && (i & 1)) tbf_step<KIND, T, V, MODE, 1, SWAP, STOR>(c, k, A, B, i, r);
     else tbf_step<KIND, T, V, MODE, 0, SWAP, STOR>(c, k, A, B, i, r);
@@ -603,8 +640,8 @@ __device__ __forceinline__ void tbf_step_rt(const CtxF &c, const CoefF &k,
 // walks them as segments of consecutive rows of one tile column.
 template <int KIND, int T, int V, bool SWAP, int STOR>
 __device__ __forceinline__ void tbf_range(const Pass2D &p, long long f, const long long fend,
-                                          float (&A)[TB2F<KIND, T, V>::NS][V],
-                                          float (&B)[TB2F<KIND, T, V>::NS][V], float *smem)
+                                          float2 (&A)[TB2F<KIND, T, V>::NS][V / 2],
+                                          float2 (&B)[TB2F<KIND, T, V>::NS][V / 2], float *smem)
 {
     using C = TB2F<KIND, T, V, STOR>;
     CtxF c;
@@ -638,12 +675,15 @@ __device__ __forceinline__ void tbf_range(const Pass2D &p, long long f, const lo
         c.oq[q] = 16u * ring_pos(min(V / 4 * c.lane + q, V / 4 * c.lane + V / 4 - 1));
         c.wq[q] = 16u * ring_pos(c.lane + 32 * min(q, V / 4 - 1));
     }
-    c.ow4 = ring_cell(c.lane > 0 ? V * c.lane - 1 : 0);
-    c.oe4 = ring_cell(c.lane < 31 ? V * c.lane + V : V * c.lane + V - 1);
     CoefF k;
-    k.a0 = p.kf[0]; k.a1 = p.kf[1]; k.a2 = p.kf[2]; k.a3 = p.kf[3]; k.a4 = p.kf[4];
-    k.a5 = p.kf[5];   // Hotspot: sdc * Ry
-    k.a6 = p.kf[6];   // Hotspot: -2 Ry (source-map kernels: unused)
+    const float a3 = stor_src(STOR) ? -p.kf[3] : p.kf[3];
+    k.a0 = make_float2(p.kf[0], p.kf[0]);
+    k.a1 = make_float2(p.kf[1], p.kf[1]);
+    k.a2 = make_float2(p.kf[2], p.kf[2]);
+    k.a3 = make_float2(a3, a3);
+    k.a4 = make_float2(p.kf[4], p.kf[4]);
+    k.a5 = make_float2(p.kf[5], p.kf[5]);   // Hotspot: sdc * Ry
+    k.a6 = make_float2(p.kf[6], p.kf[6]);   // Hotspot: -2 Ry (source-map kernels: unused)
     c.st_states = p.states;
     c.st_stride = p.state_stride;
 
@@ -679,6 +719,9 @@ __device__ __forceinline__ void tbf_range(const Pass2D &p, long long f, const lo
             const int x = c.x0 + 4 * (c.lane + 32 * q);   // chunk q of my lane
             r.nbq[q] = (x >= 0 && x < c.nx) ? min(16, 4 * (c.nx - x)) : 0;
             r.colq[q] = r.nbq[q] ? x : 0;
+            const bool in = x >= 0 && (x & ~(V - 1)) < c.nx;   // the chunk's group holds a grid cell
+            r.nbp[q] = in ? 16 : 0;
+            r.colp[q] = in ? x : 0;
         }
         c.tx = tx;
         c.msel = (c.xt < tx * C::CX) ? 0 : ((c.xt >= (tx + 1) * C::CX) ? 2 : 1);
@@ -696,38 +739,33 @@ __device__ __forceinline__ void tbf_range(const Pass2D &p, long long f, const lo
         r.gF = c.in + (long long)c.y_start * c.ld_in;
         r.gP = (KIND == KTHERM) ? c.pw + (long long)c.y_start * c.ld_pw : nullptr;
         r.rf = 0;
-        r.rp = 0;
         const int n_it = s1 + T - c.y_start;           // the last stage emits row s1-1 last
         r.i_store = s0 - c.y_start + T;                 // it emits row s0 at this iteration
         r.gO = c.out + (long long)s0 * c.ld_out + c.xt;
         r.i_load_end = c.last_row - c.y_start - C::PF + 1;
 
-        // queue the first PF rows
+        // queue the first PF field rows, and power rows 0 .. PF (row 0 with group 0: it enters
+        // only where the segment starts at the grid's top)
+        r.rp = KIND == KTHERM ? 1 : 0;   // slot of power row i+1 at i = 0
 #pragma unroll 1
         for (int j = 0; j < C::PF; j++) {
-            if (c.y_start + j <= c.last_row) {
-                tbf_queue<KIND, T, V, STOR>(c, r, C::Q16 ? 0 : j, (KIND == KTHERM && !C::Q16) ? j : 0, j);
-                if (stor_fmt(STOR) == STOR_F32) {
-                    r.gF += c.ld_in;
-                    if (KIND == KTHERM) r.gP += c.ld_pw;
-                } else {
-                    r.qF += c.ld_q;
-                    r.mF += c.ntx;
-                    if (KIND == KTHERM) {
-                        r.qP += c.ld_q;
-                        r.mP += c.ntx;
-                    }
-                }
-            }
+            const int y = c.y_start + j;
+            if (KIND == KTHERM && j == 0) tbf_queue<KIND, T, V, STOR>(c, r, false, true, 0, 0, C::PF);
+            tbf_queue<KIND, T, V, STOR>(c, r, y <= c.last_row, y + 1 <= c.last_row, j, j + 1, j);
             cp_async_commit();
+        }
+        if (KIND == KTHERM && C::Q16) {   // decode power row 0
+            cp_async_wait<C::PF - 1>();
+            __syncwarp();
+            tbf_decode_ring<V, STOR>(c, c.sRP + C::PF * C::RAWB, c.sP, c.sP + C::NBP * C::ROWB);
         }
 
         // rows that need boundary handling: the grid's top rows (for every stage), its bottom
         // rows, and every row of a pass that forwards trailing stages
         const bool partial = (c.tsteps < T);
-        const int i_a = partial ? n_it : ((c.y_start == 0) ? min(T + 1, n_it) : 0);
-        // (a stage meets row 0 at i <= T when the segment starts at the top, and rows ny-1 / ny
-        // from i = ny - y_start on; the bounds below keep one row of margin)
+        const int i_a = partial ? n_it : ((c.y_start == 0) ? min(T, n_it) : 0);
+        // (stage s meets row 0 at i = s when the segment starts at the top, and rows ny-1 / ny
+        // from i = ny-1 - y_start on)
         const int i_b = partial ? n_it : max(i_a, min(n_it, c.ny - 1 - c.y_start));
         int i = 0;
 #pragma unroll 1
@@ -773,11 +811,11 @@ __global__ void __launch_bounds__(32) k_tb2f(const Pass2D p)
 {
     using C = TB2F<KIND, T, V, STOR>;
     extern __shared__ __align__(16) float smem[];
-    float A[C::NS][V], B[C::NS][V];
+    float2 A[C::NS][V / 2], B[C::NS][V / 2];
 #pragma unroll
     for (int s = 0; s < C::NS; s++)
 #pragma unroll
-        for (int j = 0; j < V; j++) A[s][j] = B[s][j] = 0.f;
+        for (int j = 0; j < V / 2; j++) A[s][j] = B[s][j] = make_float2(0.f, 0.f);
     long long f, fend;
     if (p.starts) {
         f = __ldg(p.starts + blockIdx.x);

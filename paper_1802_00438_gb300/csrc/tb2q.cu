@@ -75,19 +75,22 @@ __device__ bool q_wait(const int *flags, int row, int x0, int x1, int y0, int y1
     return true;
 }
 
+// (12 blocks per SM: three warps per scheduler, at most 168 registers.  Without the bound both
+// kinds' loops took 184 registers and two warps per scheduler: 64-grid workload 14.7 ms against
+// 12.8 ms)
 template <int T, int V>
-__global__ void __launch_bounds__(32) k_tb2f_queue(const QueueBatch2D q)
+__global__ void __launch_bounds__(32, 12) k_tb2f_queue(const QueueBatch2D q)
 {
     using CD = TB2F<KDIFF, T, V, STOR_F32>;
     // partial rows updated in place (no two-row unroll; measured on the 64-grid workload:
     // 1980 against 1729 GCell/s with 192-row items)
     constexpr bool SW = false;
     extern __shared__ __align__(16) float smem[];
-    float A[CD::NS][V], B[CD::NS][V];
+    float2 A[CD::NS][V / 2], B[CD::NS][V / 2];
 #pragma unroll
     for (int s = 0; s < CD::NS; s++)
 #pragma unroll
-        for (int j = 0; j < V; j++) A[s][j] = B[s][j] = 0.f;
+        for (int j = 0; j < V / 2; j++) A[s][j] = B[s][j] = make_float2(0.f, 0.f);
     const int lane = threadIdx.x;
     unsigned smid;
     asm volatile("mov.u32 %0, %%smid;\n" : "=r"(smid));
@@ -121,25 +124,38 @@ __global__ void __launch_bounds__(32) k_tb2f_queue(const QueueBatch2D q)
         const int r0 = w.seg * q.L, r1 = min(G.ny, r0 + q.L);
         if (w.k < 0) {
             // source map of the tile's compute block: sdc*(p + amb*Rz), each operation rounded
-            // once (the plans' k_hot_source); 16-byte accesses where the rows allow, the warp's
-            // lanes spread over the block's rows and columns so many loads are in flight
+            // once, in pair order, row padding 0 (the plans' k_hot_source); 16-byte accesses
+            // where the rows allow, the warp's lanes spread over the block's rows and columns so
+            // many loads are in flight
             const float a = __fmul_rn(G.amb, G.rz), sdc = G.sdc;
-            constexpr int CXQ = 32 * V - 2 * ((T + 3) / 4 * 4);
+            constexpr int CXQ = TB2F<KTHERM, T, V, STOR_SRC>::CX;
             const int x0 = w.tx * CXQ, x1 = min(G.nx, x0 + CXQ);
-            const int nq = (x1 - x0 + 3) / 4;               // 4-cell chunks per row
-            const bool vec = (G.nx % 4 == 0);   // the source rows are padded: aligned always
+            const int nq = (x1 - x0 + V - 1) / V;           // V-cell groups per row
+            const bool vec = (G.nx % 4 == 0) && (uintptr_t)G.power % 16 == 0;
             for (int c = lane; c < nq * (r1 - r0); c += 32) {
-                const int y = r0 + c / nq, x = x0 + 4 * (c % nq);
+                const int y = r0 + c / nq, x = x0 + V * (c % nq);
                 const float *pr = G.power + (long long)y * G.nx + x;
-                float *d = G.src + (long long)y * G.ld_src + x;
-                if (vec) {
-                    const float4 v = *reinterpret_cast<const float4 *>(pr);
-                    *reinterpret_cast<float4 *>(d) =
-                        make_float4(__fmul_rn(sdc, __fadd_rn(v.x, a)), __fmul_rn(sdc, __fadd_rn(v.y, a)),
-                                    __fmul_rn(sdc, __fadd_rn(v.z, a)), __fmul_rn(sdc, __fadd_rn(v.w, a)));
+                float v[V], o[V];
+                if (vec && x + V <= x1) {
+#pragma unroll
+                    for (int t = 0; t < V / 4; t++) {
+                        const float4 q4 = *reinterpret_cast<const float4 *>(pr + 4 * t);
+                        v[4 * t] = q4.x; v[4 * t + 1] = q4.y; v[4 * t + 2] = q4.z; v[4 * t + 3] = q4.w;
+                    }
+#pragma unroll
+                    for (int j = 0; j < V; j++) v[j] = __fmul_rn(sdc, __fadd_rn(v[j], a));
                 } else {
-                    for (int j = 0; j < 4 && x + j < x1; j++) d[j] = __fmul_rn(sdc, __fadd_rn(pr[j], a));
+#pragma unroll
+                    for (int j = 0; j < V; j++)
+                        v[j] = x + j < x1 ? __fmul_rn(sdc, __fadd_rn(pr[j], a)) : 0.f;
                 }
+#pragma unroll
+                for (int j = 0; j < V; j++) o[src_pos<V>(j)] = v[j];
+                float *d = G.src + (long long)y * G.ld_src + x;
+#pragma unroll
+                for (int t = 0; t < V / 4; t++)
+                    *reinterpret_cast<float4 *>(d + 4 * t) =
+                        make_float4(o[4 * t], o[4 * t + 1], o[4 * t + 2], o[4 * t + 3]);
             }
         } else if (w.k < G.P) {
             const Pass2D &p = q.passes[G.pass_base + w.k];

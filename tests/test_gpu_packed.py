@@ -1,0 +1,42 @@
+"""Contracted 2D kernels on widths around the edges of their packed pairs, V-cell groups and tile
+columns (240 compute cells with 8 cells per thread, 112 to 120 with 4), where the source map's
+pair order, its padded groups and the clamp fix-ups can go wrong; float32 and 16-bit storage.
+Bars: max relative error <= 1e-5 against the float32 oracle (the contracted kernels' bar);
+16-bit storage: relative L2 <= 1e-2 (the storage bar)."""
+import numpy as np
+import pytest
+
+import synth
+from test_gpu_parity import TOL, eng, gpu_run, max_rel  # noqa: F401  (eng: fixture)
+
+pytestmark = pytest.mark.gpu
+
+WIDTHS = [3, 4, 5, 7, 8, 9, 12, 111, 112, 113, 119, 121, 239, 240, 241, 247, 249, 480, 485]
+
+
+@pytest.mark.parametrize("kind", [0, 1])
+@pytest.mark.parametrize("T,vec,rows", [(1, 8, 2), (4, 8, 2), (6, 8, 2), (8, 8, 1), (8, 8, 2), (8, 4, 2),
+                                        (12, 4, 1)])
+def test_widths(eng, orc, kind, T, vec, rows):  # noqa: F811
+    for n, nx in enumerate(WIDTHS):
+        w = synth.make(kind, 2, nx, 21 + n % 3, seed=8100 + 7 * n + kind)
+        steps = 2 * T + 1 + n % 2
+        g, info = gpu_run(eng, w, steps, T=T, vec=vec, rows=rows, resident=-1)
+        assert (info["T"], info["vec"], info["partial_rows"]) == (T, vec, rows)
+        o = orc.run(kind, w.u0, w.coef, steps, w.power)
+        assert max_rel(g, o) <= TOL, (nx, steps, max_rel(g, o))
+
+
+@pytest.mark.parametrize("storage", [1, 2])
+@pytest.mark.parametrize("kind", [0, 1])
+def test_widths_16bit(eng, orc, kind, storage):  # noqa: F811
+    import torch
+    for n, nx in enumerate(WIDTHS):
+        w = synth.make(kind, 2, nx, 21, seed=8300 + 7 * n + kind)
+        u = torch.from_numpy(w.u0).cuda()
+        p = None if w.power is None else torch.from_numpy(w.power).cuda()
+        plan = eng.Plan(kind, 2, nx, 21, storage=storage)
+        g = plan.run(u, torch.full_like(u, float("nan")), w.coef, 19, power=p).cpu().numpy()
+        plan.close()
+        o = orc.run(kind, w.u0, w.coef, 19, w.power, dtype=np.float64)
+        assert np.linalg.norm(g - o) <= 1e-2 * np.linalg.norm(o), nx
