@@ -720,11 +720,11 @@ int stencil_adjoint_backward(stencil_adjoint a, const float *grad_out, const flo
     stn::Tma3D mo, m0, m1, ms, mp;
     std::memset(&mo, 0, sizeof(mo));
     m0 = m1 = ms = mp = mo;
-    bool tma = stn::tma3d_encode(&mo.in, grad_out, a->nx, a->ny, 1, AX, AY) &&
-               stn::tma3d_encode(&m0.in, a->lam[0], a->nx, a->ny, 1, AX, AY) &&
-               stn::tma3d_encode(&m1.in, a->lam[1], a->nx, a->ny, 1, AX, AY) &&
-               stn::tma3d_encode(&ms.in, a->seg, a->nx, a->ny, a->ckpt, AX, AY);
-    if (tma && power) tma = stn::tma3d_encode(&mp.in, power, a->nx, a->ny, 1, AX, AY);
+    bool tma = stn::tma3d_encode(&mo.in, grad_out, a->nx, a->ny, 1, a->nx, AX, AY) &&
+               stn::tma3d_encode(&m0.in, a->lam[0], a->nx, a->ny, 1, a->nx, AX, AY) &&
+               stn::tma3d_encode(&m1.in, a->lam[1], a->nx, a->ny, 1, a->nx, AX, AY) &&
+               stn::tma3d_encode(&ms.in, a->seg, a->nx, a->ny, a->ckpt, a->nx, AX, AY);
+    if (tma && power) tma = stn::tma3d_encode(&mp.in, power, a->nx, a->ny, 1, a->nx, AX, AY);
     p.use_tma = tma ? 1 : 0;
     p.err = a->err;
     const int smem = adj_smem(a->kind);

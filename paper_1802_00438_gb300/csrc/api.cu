@@ -94,9 +94,8 @@ struct PassCfg3D {
     int ntx = 0, nty = 0;
     long long cols = 0, planes_per_cta = 0;
     int ctas = 0;
-    int zslab = 0;          // > 0: round-robin pieces of zslab planes (partial-sum kernel)
-    long long pieces = 0;
-    long long *starts = nullptr;   // device: cost-balanced ranges (zslab = 0), or none
+    int seg_off = 0;        // ints before the segments
+    void *segs = nullptr;   // partial-sum kernel, device: [first segment of each block | segments]
     bool ready = false;
 };
 
@@ -107,7 +106,8 @@ struct stencil_plan_s {
     cudaStream_t stream = nullptr;
     int device = 0, sms = 0;
     float *scratch = nullptr;
-    long long ld_scratch = 0;   // row pitch of the scratch grid (2D), floats
+    float *scratch2 = nullptr;  // second scratch grid, where the caller's rows are unaligned
+    long long ld_scratch = 0;   // row pitch of the scratch grids, floats
     size_t scratch_bytes = 0;
     int T = 1;
     // 2D
@@ -119,7 +119,8 @@ struct stencil_plan_s {
     double model = 0.0;   // calibrated model's prediction for this plan (1000 steps), GCell/s
     int tuned = 0;        // configuration taken from the tuning cache
     PassCfg2D traj;       // trajectory passes (stencil_run_trajectory)
-    float *src = nullptr;   // contracted float32 Hotspot 2D: the source map sdc*(p + amb*Rz)
+    float *src = nullptr;   // contracted float32 Hotspot 2D: the source map sdc*(p + amb*Rz);
+                            // Hotspot 3D, unaligned rows: the power map with padded rows
     long long ld_src = 0;   // its row pitch, floats
     int ntx_star = 0, nty_star = 0;   // star diffusion (rad > 1): tiles along x and y
     int nseg_star = 1, zseg_star = 0; // 3D star: z-segments per tile column, their length
@@ -242,49 +243,119 @@ double model_gcells_2d(const stencil_desc &d, int sms, const Cand2D &k, int bps,
     return r.gcells;
 }
 
-// 3D partial-sum kernel: the same restatement.  Issued work: 17.3 (Diffusion) and 19.7
-// (Hotspot) thread instructions per computed cell update including halos (ncu counts of the
-// 512^3 and 512^2 x 256 runs with 2 x 4 cells per thread at T = 4), x(0.85 + 0.6/T) for the
-// costlier first stage.  Issue efficiency 0.61 for one
-// 16-warp block per SM, x1.10 for two 8-warp blocks (they wait at fewer barriers together),
-// x0.80 for 32-warp blocks of 2 x 2 cells (twice the y exchange per cell).  Device memory: the
-// tiles read their halos again (the tile fit's read factor, ntx*bx*nty*by / (nx*ny)), at 62 %
-// of the measured copy bandwidth.  Calibrated on the 50-point sweep of bench.py --model-study
-// (measured / predicted per configuration).
-// 3D segments (tb3f): the z-slab length Z of round-robin (tile column, z-slab) pieces, or 0 for
-// contiguous (tile column, plane) ranges.  Pieces read the tiles' halo planes from L2 and cut
-// the pass's DRAM traffic to about the algorithmic bytes (ranges: 1.4-1.6x), which pays only
-// where the pass is memory-bound: measured on GB300, T = 1 (512^3 diffusion: 578 GCell/s with
-// pieces, 431 with ranges); from T = 2 on the kernel is issue-bound and the cost-balanced
-// ranges are faster (T = 3: 963 against 935).  So pieces for T = 1, when their rounds cost at
-// most 6 % more plane-times per block (planes plus T of pipeline fill per segment) than the
-// ranges; *cost receives the chosen mode's plane-times per block.
-int zslab_pick(long long cols, int nz, long long slots, int T, double *cost)
+// 3D partial-sum kernel: the same restatement.  Issue-equivalent work per computed cell update
+// including halos, by T: 16 / 13.5 / 11.2 / 13 operations (Diffusion, T = 1 .. 4; T = 4 spills
+// registers), 18.6 / 15.7 / 12.9 / 13.7 (Hotspot), at an issue efficiency of 0.61 for one 16-warp
+// block per SM, x1.04 for two 8-warp blocks, x0.80 for 32-warp blocks of 2 x 2 cells (twice the y
+// exchange per cell).  A pass costs 9 us besides (launch, first planes, drain).  Device memory:
+// with the columns streamed in step most halo re-reads hit L2: three tenths of the tile fit's
+// excess reads, at 90 % of the copy bandwidth.  Calibrated on GB300 over 512^3, 512^2 x 256,
+// 256^3, 300 x 200 x 400 and 187 x 141 x 93, both kinds, T = 2 .. 4, 64- and 32-row tiles.
+// 3D segments (tb3f): which planes of which tile columns each block streams.  A segment costs
+// w[col] per plane plus `fill` planes of pipeline fill, and the slowest block sets the pass time.
+// The tile columns overlap, so neighbouring columns should be at nearby planes at the same time:
+// then the halo cells a tile reads again (and the partial sectors of its rows) are still in L2.
+// So, level by level: with at least as many blocks as columns left, every column gets one block,
+// all from the same first plane, for as many planes as the budget allows, and what is left of the
+// columns goes to the blocks without work; with fewer blocks than columns, each block takes one
+// whole rest of a column, the costliest first, and goes on with the budget that leaves it.  The
+// budget is the smallest for which everything is dealt out (bisection).
+// Measured on GB300 against contiguous ranges of (column, plane) units balanced the same way,
+// where neighbours run at unrelated planes: see prepare3.
+struct Seg3 { int col, z0, z1, pad; };
+
+bool deal_segments(int nz, int slots, double fill, const std::vector<double> &w, double budget,
+                   std::vector<std::vector<Seg3>> *out)
 {
-    const long long total = cols * nz;
-    const long long ctas = std::min(slots, std::max<long long>(1, total / std::max(16, 8 * T)));
-    const double range_cost = (double)((total + ctas - 1) / ctas) + T;
-    double best = 0.0;
-    int best_z = 0;
-    for (int S = 1; S <= std::max(1, nz / (2 * T)); S++) {
-        const int Z = (nz + S - 1) / S;
-        const long long pieces = cols * ((nz + Z - 1) / Z);
-        const long long G = std::min(slots, pieces);
-        const double c = (double)((pieces + G - 1) / G) * (Z + T);
-        if (!best_z || c < best) {
-            best = c;
-            best_z = Z;
+    struct Rest { int col, z0; };
+    struct Block { double left; int id; };
+    std::vector<Rest> rest(w.size()), next;
+    for (size_t c = 0; c < w.size(); c++) rest[c] = Rest{(int)c, 0};
+    // blocks with work to take, the largest budget first, from `head` on; `spare`: those that have
+    // a segment and budget left, taken up when the others have run out
+    std::vector<Block> blocks(slots), spare;
+    for (int b = 0; b < slots; b++) blocks[b] = Block{budget, b};
+    size_t head = 0;
+    if (out) out->assign(slots, {});
+    while (!rest.empty()) {
+        if (head == blocks.size()) {
+            if (spare.empty()) return false;
+            std::sort(spare.begin(), spare.end(), [](const Block &a, const Block &b) {
+                return a.left != b.left ? a.left > b.left : a.id < b.id;
+            });
+            blocks.swap(spare);
+            spare.clear();
+            head = 0;
         }
+        const size_t avail = blocks.size() - head;
+        const bool whole = rest.size() > avail;   // fewer blocks than columns: whole rests
+        if (whole)
+            std::sort(rest.begin(), rest.end(), [&](const Rest &a, const Rest &b) {
+                const double ca = (nz - a.z0) * w[a.col], cb = (nz - b.z0) * w[b.col];
+                return ca != cb ? ca > cb : a.col < b.col;
+            });
+        next.clear();
+        for (size_t i = 0; i < rest.size(); i++) {
+            const Rest &q = rest[i];
+            if (i >= avail) {
+                next.push_back(q);
+                continue;
+            }
+            Block &b = blocks[head + i];
+            const int h = nz - q.z0;
+            const int take = std::max(1, (int)std::min<double>(h, std::floor((b.left - fill) / w[q.col])));
+            if (out) (*out)[b.id].push_back(Seg3{q.col, q.z0, q.z0 + take, 0});
+            if (take < h) {
+                next.push_back(Rest{q.col, q.z0 + take});
+            } else {
+                b.left -= fill + take * w[q.col];
+                if (b.left >= fill + 4) spare.push_back(b);
+            }
+        }
+        head += std::min(avail, rest.size());
+        if (whole)
+            std::sort(next.begin(), next.end(), [](const Rest &a, const Rest &b) { return a.col < b.col; });
+        rest.swap(next);
     }
-    if (T == 1 && best_z > 0 && best <= 1.06 * range_cost) {
-        if (cost) *cost = best;
-        return best_z;
-    }
-    if (cost) *cost = range_cost;
-    return 0;
+    return true;
 }
 
-double model_gcells_3d(const stencil_desc &d, int sms, int T, int VX, int VY, int NW)
+// The smallest budget for `slots` blocks (within tol), and with out != nullptr the segments per
+// block.
+double best_segments(int nz, int slots, double fill, const std::vector<double> &w, double tol,
+                     std::vector<std::vector<Seg3>> *out)
+{
+    double total = 0.0;
+    for (double x : w) total += x * nz;
+    double lo = total / slots, hi = lo + 3.0 * fill;
+    while (!deal_segments(nz, slots, fill, w, hi, nullptr)) hi *= 1.5;
+    for (int i = 0; i < 40 && hi - lo > tol; i++) {
+        const double mid = 0.5 * (lo + hi);
+        if (deal_segments(nz, slots, fill, w, mid, nullptr)) hi = mid;
+        else lo = mid;
+    }
+    if (out) deal_segments(nz, slots, fill, w, hi, out);
+    return hi;
+}
+
+// relative cost of a plane of each tile column (kWX3, kWY3: see prepare3)
+constexpr double kWX3 = 1.4, kWY3 = 1.2;
+
+std::vector<double> column_weights(int ntx, int nty)
+{
+    std::vector<double> w((size_t)ntx * nty, 1.0);
+    for (int ty = 0; ty < nty; ty++)
+        for (int tx = 0; tx < ntx; tx++) {
+            double &x = w[(size_t)ty * ntx + tx];
+            if (tx == 0 || tx == ntx - 1) x *= kWX3;
+            if (ty == 0 || ty == nty - 1) x *= kWY3;
+        }
+    return w;
+}
+
+// `bound`: an upper bound instead, with segments dealt at no loss (no bisection)
+double model_gcells_3d(const stencil_desc &d, int sms, int T, int VX, int VY, int NW,
+                       bool bound = false)
 {
     stencil_gpu_model_in m = {};
     m.ndim = 3;
@@ -304,23 +375,23 @@ double model_gcells_3d(const stencil_desc &d, int sms, int T, int VX, int VY, in
     if (cx < 1 || cy < 1) return 0.0;
     const long long cols = (long long)std::ceil(d.nx / cx) * (long long)std::ceil(d.ny / cy);
     double rf = std::ceil(d.nx / cx) * m.bx * std::ceil(d.ny / cy) * m.by / ((double)d.nx * d.ny);
-    // the segments prepare3 will take: z-slab pieces read their halos again from L2, not DRAM
+    // the segments prepare3 will take
     const long long slots = (long long)sms * (NW <= 8 ? 2 : 1);
-    double seg_cost = 0.0;
-    const bool pieces = zslab_pick(cols, d.nz, slots, T, &seg_cost) > 0;
-    if (pieces) rf = 1.0;
+    const double seg_cost =
+        bound ? 0.0
+              : best_segments(d.nz, (int)slots, 3.0 * T - 1,
+                              column_weights((int)std::ceil(d.nx / cx), (int)std::ceil(d.ny / cy)),
+                              0.02 * cols * d.nz / slots + 0.5, nullptr);
     const double alg = d.kind == ST_DIFFUSION ? 8.0 : 12.0;
     const double read = alg - 4.0;   // field (and power) in; the field out is written once
     m.bytes_per_cell = alg;
-    m.hbm_eff = 0.62 * alg / (read * rf + 4.0);
-    // stage 0 (three ring planes, their exchange) costs more than the partial-sum stages
-    // (recalibrated after interior tile columns dropped the clamp fix-ups: measured / model
-    // over the 3D configurations of the accuracy study was 1.11 (diffusion), 1.07 (Hotspot))
-    m.ops_per_cell = (d.kind == ST_DIFFUSION ? 16.0 : 18.6) * (0.85 + 0.6 / T);
-    m.issue_eff = 0.61 * (NW <= 8 ? 1.10 : NW >= 32 ? 0.80 : 1.0);
-    // plane-times per block beyond an even share of the planes (fill, round quantisation)
-    m.stream_overhead = pieces ? std::max(0.0, seg_cost * slots / ((double)cols * d.nz) - 1.0) : 0.04;
-    m.launch_s = 4e-6;
+    m.hbm_eff = 0.90 * alg / (read * (1.0 + 0.3 * (rf - 1.0)) + 4.0);
+    const double ops[2][5] = {{0, 16.0, 13.5, 11.2, 13.0}, {0, 18.6, 15.7, 12.9, 13.7}};
+    m.ops_per_cell = ops[d.kind == ST_DIFFUSION ? 0 : 1][std::min(std::max(T, 1), 4)];
+    m.issue_eff = 0.61 * (NW <= 8 ? 1.04 : NW >= 32 ? 0.80 : 1.0);
+    // plane-times per block beyond an even share of the planes (fill, edge columns)
+    m.stream_overhead = std::max(0.0, seg_cost * slots / ((double)cols * d.nz) - 1.0);
+    m.launch_s = 9e-6;
     stencil_gpu_model_out r;
     if (stencil_model_gpu(&m, &r) != ST_OK) return 0.0;
     return r.gcells;
@@ -567,44 +638,35 @@ int prepare3(stencil_plan_s *p, int Tk, PassCfg3D **out)
         c.planes_per_cta = (total + ctas - 1) / ctas;
         c.ctas = (int)((total + c.planes_per_cta - 1) / c.planes_per_cta);
         if (p->alg3) {
-            // or pieces (tile column, z-slab) dealt round-robin (zslab_pick): the blocks of a
-            // round stream neighbouring tile columns through the same planes together, so the
-            // halo cells a tile reads again come from L2 (with contiguous ranges the neighbours
-            // run far apart in z and every tile reads its halos from device memory: measured
-            // on 512^2 x 256 diffusion, T = 3, DRAM bytes per pass 751 MB with ranges, 504 MB
-            // with 52-plane pieces, 537 MB algorithmic).
-            const long long slots = (long long)p->sms * bps;
-            const int best_z = zslab_pick(c.cols, p->d.nz, slots, Tk, nullptr);
-            // a plane of a tile column at the x edge costs 1.2, at the y edge 1.1 (only those
-            // columns run the kernel instance with the clamp fix-ups; measured on GB300,
-            // weights swept 1.0-1.45, T = 3: 512^3 diffusion 923 -> 1027 GCell/s, 512^2 x 256
-            // Hotspot 752 -> 838)
-            const double wx = 1.2, wy = 1.1;
-            std::vector<double> w(c.cols, 1.0);
-            for (long long col = 0; col < c.cols; col++) {
-                const long long ty = col / c.ntx, tx = col - ty * c.ntx;
-                if (tx == 0 || tx == c.ntx - 1) w[col] *= wx;
-                if (ty == 0 || ty == c.nty - 1) w[col] *= wy;
+            // segments dealt to the blocks (best_segments): a plane of a tile column at the x
+            // edge costs 1.4, at the y edge 1.2 (only they run instances with the clamp fix-ups,
+            // and the barrier makes a block wait for its slowest warp; swept 1.0-1.4 on GB300,
+            // T = 3: 512^3 diffusion 1188 GCell/s at 1.1 / 1.05, 1318 at 1.4 / 1.2).  Dealt
+            // level by level against contiguous ranges balanced the same way: 512^2 x 256 Hotspot
+            // 940 -> 1044 GCell/s at T = 3, 611 -> 912 at T = 2 (DRAM reads of a 512^2 x 256
+            // diffusion pass 491 -> 302 MB); a plan of few columns is spread over more blocks
+            // (187 x 141 x 93 diffusion x 30: 427 -> 242 us)
+            const std::vector<double> w = column_weights(c.ntx, c.nty);
+            std::vector<std::vector<Seg3>> segs;
+            best_segments(p->d.nz, p->sms * bps, 3.0 * Tk - 1, w, 0.25, &segs);
+            while (segs.size() > 1 && segs.back().empty()) segs.pop_back();
+            c.ctas = (int)segs.size();
+            std::vector<int> host(((size_t)c.ctas + 1 + 3) / 4 * 4, 0);   // first[], 16-byte aligned end
+            c.seg_off = (int)host.size();
+            for (int i = 0, n = 0; i < c.ctas; i++) {
+                host[i] = n;
+                n += (int)segs[i].size();
+                host[i + 1] = n;
             }
-            if (best_z > 0) {
-                c.zslab = best_z;
-                c.pieces = c.cols * ((p->d.nz + best_z - 1) / best_z);
-                c.ctas = (int)std::min(slots, c.pieces);
-            } else {
-                // contiguous ranges balanced by cost: edge tile columns weigh more
-                std::vector<long long> st;
-                if (balanced_ranges(p->d.nz, (int)ctas, Tk, w, st) <
-                    even_ranges_cost(p->d.nz, c.planes_per_cta, Tk, w)) {
-                    e = stn::dev_malloc(&c.starts, st.size() * sizeof(long long));
-                    if (e == cudaSuccess)
-                        e = cudaMemcpy(c.starts, st.data(), st.size() * sizeof(long long), cudaMemcpyHostToDevice);
-                    if (e != cudaSuccess) {
-                        if (c.starts) stn::dev_free(c.starts);
-                        c.starts = nullptr;
-                        return map_cuda(e);
-                    }
-                    c.ctas = (int)ctas;
-                }
+            for (const auto &v : segs)
+                for (const Seg3 &q : v) host.insert(host.end(), {q.col, q.z0, q.z1, 0});
+            e = stn::dev_malloc(&c.segs, host.size() * sizeof(int));
+            if (e == cudaSuccess)
+                e = cudaMemcpy(c.segs, host.data(), host.size() * sizeof(int), cudaMemcpyHostToDevice);
+            if (e != cudaSuccess) {
+                if (c.segs) stn::dev_free(c.segs);
+                c.segs = nullptr;
+                return map_cuda(e);
             }
         }
         c.ready = true;
@@ -853,7 +915,7 @@ int run_pass_star3(stencil_plan_s *p, const float *src, float *dst, const float 
     a.err = p->err;
     CUtensorMap tm;
     std::memset(&tm, 0, sizeof(tm));
-    a.use_tma = tma3d_encode(&tm, src, p->d.nx, p->d.ny, p->d.nz, 64, 64) ? 1 : 0;
+    a.use_tma = tma3d_encode(&tm, src, p->d.nx, p->d.ny, p->d.nz, p->d.nx, 64, 64) ? 1 : 0;
     if (p->timing && p->ev_used + 2 > 2 * 1024) {
         const int rc = flush_timing(p);
         if (rc != ST_OK) return rc;
@@ -882,7 +944,7 @@ int run_pass_star(stencil_plan_s *p, const float *src, float *dst, const float *
     a.err = p->err;
     CUtensorMap tm;
     std::memset(&tm, 0, sizeof(tm));
-    a.use_tma = tma3d_encode(&tm, src, p->d.nx, p->d.ny, 1, 128, 128) ? 1 : 0;
+    a.use_tma = tma3d_encode(&tm, src, p->d.nx, p->d.ny, 1, p->d.nx, 128, 128) ? 1 : 0;
     if (p->timing && p->ev_used + 2 > 2 * 1024) {
         const int rc = flush_timing(p);
         if (rc != ST_OK) return rc;
@@ -893,8 +955,9 @@ int run_pass_star(stencil_plan_s *p, const float *src, float *dst, const float *
     return map_cuda(e);
 }
 
-int run_pass3(stencil_plan_s *p, const float *src, float *dst, const float *pw, const float *k,
-              int tsteps)
+// row pitches lds, ldd, ldp of the input, the output and the power map, in floats
+int run_pass3(stencil_plan_s *p, const float *src, long long lds, float *dst, long long ldd,
+              const float *pw, long long ldp, const float *k, int tsteps)
 {
     PassCfg3D *c = nullptr;
     int rc = prepare3(p, kernel_T_for(p, tsteps), &c);
@@ -912,20 +975,24 @@ int run_pass3(stencil_plan_s *p, const float *src, float *dst, const float *pw, 
     a.total_cols = c->cols;
     a.planes_per_cta = c->planes_per_cta;
     a.ctas = c->ctas;
-    a.zslab = c->zslab;
-    a.pieces = c->pieces;
-    a.starts = c->starts;
+    a.seg_first = static_cast<const int *>(c->segs);
+    a.segs = c->segs ? reinterpret_cast<const int4 *>(a.seg_first + c->seg_off) : nullptr;
     for (int i = 0; i < 9; i++) a.k[i] = i < ncoef(p->d) ? k[i] : 0.f;
-    a.vec = ((uintptr_t)src % 16 == 0) && ((uintptr_t)dst % 16 == 0) && (p->d.nx % 4 == 0);
-    a.vec_pw = pw && ((uintptr_t)pw % 16 == 0) && (p->d.nx % 4 == 0);
+    a.ld_in = lds;
+    a.ld_out = ldd;
+    a.ld_pw = ldp;
+    a.vec = ((uintptr_t)src % 16 == 0) && (lds % 4 == 0);
+    a.vec_out = ((uintptr_t)dst % 16 == 0) && (ldd % 4 == 0);
+    if (!p->alg3) a.vec = a.vec && a.vec_out;
+    a.vec_pw = pw && ((uintptr_t)pw % 16 == 0) && (ldp % 4 == 0);
     a.err = p->err;
     a.use_tma = 0;
     Tma3D tm;
     std::memset(&tm, 0, sizeof(tm));
     if (p->alg3 && a.vec) {
         const int bx = 32 * p->VX3, by = p->VY * p->NW;
-        bool ok = tma3d_encode(&tm.in, src, p->d.nx, p->d.ny, p->d.nz, bx, by);
-        if (ok && pw) ok = a.vec_pw && tma3d_encode(&tm.pw, pw, p->d.nx, p->d.ny, p->d.nz, bx, by);
+        bool ok = tma3d_encode(&tm.in, src, p->d.nx, p->d.ny, p->d.nz, lds, bx, by);
+        if (ok && pw) ok = a.vec_pw && tma3d_encode(&tm.pw, pw, p->d.nx, p->d.ny, p->d.nz, ldp, bx, by);
         a.use_tma = ok ? 1 : 0;
     }
     if (p->timing && p->ev_used + 2 > 2 * 1024) {
@@ -1081,6 +1148,7 @@ static int plan_create(stencil_plan *out, const stencil_desc *desc)
             }
             p->zseg_star = (int)((d.nz + nseg - 1) / nseg);
             p->nseg_star = (d.nz + p->zseg_star - 1) / p->zseg_star;
+            p->ld_scratch = d.nx;
             p->scratch_bytes = (size_t)cells_of(d) * sizeof(float);
         }
     } else if (d.rad > 1) {
@@ -1245,12 +1313,13 @@ static int plan_create(stencil_plan *out, const stencil_desc *desc)
         if (free_tile && !d.force_T && d.rad <= 1) {
             // nothing forced, contracted: the compiled partial-sum (tile, T) the calibrated
             // model rates best
-            const int shapes[][3] = {{64, 64, 8}, {64, 64, 4}, {128, 32, 8}, {64, 32, 8}};
+            const int shapes[][3] = {{64, 64, 8}, {64, 32, 8}, {128, 32, 8}, {64, 64, 4}};
             double best = -1.0;
             for (const auto &sh : shapes)
-                for (int t = 1; t <= 4; t++) {
+                for (int t : {3, 2, 4, 1}) {
                     const int vx = sh[0] / 32, vy = sh[2] / vx, nw = sh[1] / vy;
                     if (!tb3d_available(Shape3D{d.kind, 0, t, vy, nw, 1, vx})) continue;
+                    if (model_gcells_3d(d, p->sms, t, vx, vy, nw, true) <= best) continue;
                     const double g = model_gcells_3d(d, p->sms, t, vx, vy, nw);
                     if (g > best) {
                         best = g;
@@ -1276,10 +1345,24 @@ static int plan_create(stencil_plan *out, const stencil_desc *desc)
         if (p->T == 0 || (d.force_T && p->T != d.force_T)) rc = ST_ERR_UNSUPPORTED;
         PassCfg3D *c = nullptr;
         if (rc == ST_OK) rc = prepare3(p, p->T, &c);
-        p->scratch_bytes = (size_t)cells_of(d) * sizeof(float);
+        // the partial-sum kernel's scratch rows are padded to whole 16-byte chunks
+        p->ld_scratch = p->alg3 ? ((long long)d.nx + 3) / 4 * 4 : d.nx;
+        p->scratch_bytes = (size_t)p->ld_scratch * d.ny * d.nz * sizeof(float);
     }
+    // Contracted first-order plans on rows that are no whole 16-byte chunks (nx not a multiple of
+    // 4): the passes between the first and the last run between two padded scratch grids, so that
+    // only those two touch the caller's rows (staged and stored cell by cell)
+    const bool two = rc == ST_OK && d.nx % 4 != 0 && !d.exact && !p->res && !p->stor && d.rad <= 1 &&
+                     d.kind != ST_DIFFUSION_VAR && (d.ndim == 2 || p->alg3);
     if (rc == ST_OK && p->scratch_bytes) {
         e = stn::dev_malloc(&p->scratch, p->scratch_bytes);
+        if (e == cudaSuccess && two) e = stn::dev_malloc(&p->scratch2, p->scratch_bytes);
+        if (e != cudaSuccess) rc = map_cuda(e);
+        if (two) p->scratch_bytes *= 2;
+    }
+    if (two && rc == ST_OK && d.ndim == 3 && d.kind == ST_THERMAL) {
+        p->ld_src = p->ld_scratch;
+        e = stn::dev_malloc(&p->src, (size_t)p->ld_src * d.ny * d.nz * sizeof(float));
         if (e != cudaSuccess) rc = map_cuda(e);
     }
     if (rc == ST_OK && d.ndim == 2 && d.kind == ST_THERMAL && !d.exact && !p->stor) {
@@ -1384,9 +1467,21 @@ int stencil_run(stencil_plan p, const void *grid_in, void *grid_out, const void 
     // buffer of pass i: the caller's output when (passes-1-i) is even, else the scratch grid;
     // in place with an odd pass count, pass 0 cannot write the input it reads, so every pass
     // shifts by one and a final copy brings the scratch result to the output.
-    const bool shift = (in == out) && (passes % 2 == 1);
-    const long long ldo = d.nx, ldsc = d.ndim == 2 ? p->ld_scratch : d.nx;
-    if (p->src) {
+    // With two scratch grids the passes between the first and the last use only those.
+    const bool two = p->scratch2 != nullptr;
+    const bool shift = (in == out) && (two ? passes == 1 : passes % 2 == 1);
+    const long long ldo = d.nx, ldsc = p->ld_scratch;
+    long long ldp = d.nx;
+    if (p->src && d.ndim == 3) {
+        if (passes > 1) {   // padded rows: one copy instead of unaligned reads in every pass
+            e = cudaMemcpy2DAsync(p->src, (size_t)p->ld_src * sizeof(float), pw,
+                                  (size_t)d.nx * sizeof(float), (size_t)d.nx * sizeof(float),
+                                  (size_t)d.ny * d.nz, cudaMemcpyDeviceToDevice, p->stream);
+            if (e != cudaSuccess) return map_cuda(e);
+            pw = p->src;
+            ldp = p->ld_src;
+        }
+    } else if (p->src) {
         // contracted Hotspot 2D kernels stage sdc*(p + amb*Rz) (Table 2's source and ambient
         // terms folded into one map)
         e = hot_source(pw, d.nx, p->src, p->ld_src, d.nx, d.ny, coeffs[4], coeffs[3], coeffs[0],
@@ -1399,12 +1494,13 @@ int stencil_run(stencil_plan p, const void *grid_in, void *grid_out, const void 
     for (int i = 0; i < passes; i++) {
         const stn::NvtxRange r_pass("pass");
         const int ts = (i == passes - 1) ? last : T;
-        const bool to_out = shift ? ((passes - i) % 2 == 0) : ((passes - 1 - i) % 2 == 0);
-        float *dst = to_out ? out : p->scratch;
+        const bool to_out = two ? !shift && i == passes - 1
+                            : shift ? ((passes - i) % 2 == 0) : ((passes - 1 - i) % 2 == 0);
+        float *dst = to_out ? out : (two && i % 2) ? p->scratch2 : p->scratch;
         const long long ldd = to_out ? ldo : ldsc;
         int rc = d.rad > 1     ? run_pass_star(p, src, dst, coeffs, ts)
                  : d.ndim == 2 ? run_pass2(p, src, lds, dst, ldd, pw, coeffs, ts)
-                               : run_pass3(p, src, dst, pw, coeffs, ts);
+                               : run_pass3(p, src, lds, dst, ldd, pw, ldp, coeffs, ts);
         if (rc != ST_OK) {
             p->sticky = rc;
             return rc;
@@ -1413,10 +1509,10 @@ int stencil_run(stencil_plan p, const void *grid_in, void *grid_out, const void 
         lds = ldd;
     }
     if (shift) {
-        if (d.ndim == 2)
+        if (ldsc != d.nx)
             e = cudaMemcpy2DAsync(out, (size_t)d.nx * sizeof(float), p->scratch,
-                                  (size_t)p->ld_scratch * sizeof(float), (size_t)d.nx * sizeof(float),
-                                  d.ny, cudaMemcpyDeviceToDevice, p->stream);
+                                  (size_t)ldsc * sizeof(float), (size_t)d.nx * sizeof(float),
+                                  (size_t)d.ny * d.nz, cudaMemcpyDeviceToDevice, p->stream);
         else
             e = cudaMemcpyAsync(out, p->scratch, bytes, cudaMemcpyDeviceToDevice, p->stream);
         if (e != cudaSuccess) return map_cuda(e);
@@ -1591,6 +1687,7 @@ int stencil_plan_destroy(stencil_plan p)
     if (p->ev_used) cudaStreamSynchronize(p->stream);
     for (cudaEvent_t e : p->ev) cudaEventDestroy(e);
     if (p->scratch) stn::dev_free(p->scratch);
+    if (p->scratch2) stn::dev_free(p->scratch2);
     for (int b = 0; b < 2; b++) {
         if (p->q[b]) stn::dev_free(p->q[b]);
         if (p->qm[b]) stn::dev_free(p->qm[b]);
@@ -1604,7 +1701,7 @@ int stencil_plan_destroy(stencil_plan p)
     for (PassCfg2D &c : p->cfg2)
         if (c.starts) stn::dev_free(c.starts);
     for (PassCfg3D &c : p->cfg3)
-        if (c.starts) stn::dev_free(c.starts);
+        if (c.segs) stn::dev_free(c.segs);
     delete p;
     return ST_OK;
 }

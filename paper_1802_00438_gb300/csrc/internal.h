@@ -191,12 +191,16 @@ struct Pass3D {
     long long total_cols;  // ntx * nty tile columns (each streamed along z)
     long long planes_per_cta;
     int ctas;
-    int zslab;             // partial-sum kernel: > 0 = pieces of zslab planes, round-robin
-    long long pieces;      // total_cols * ceil(nz / zslab)
-    const long long *starts;   // partial-sum kernel, zslab = 0: block b takes units
-                               // [starts[b], starts[b+1]) (nullptr: planes_per_cta each)
+    // partial-sum kernel: block b streams segments seg_first[b] .. seg_first[b+1]-1, each
+    // (tile column, first plane, end plane, 0)
+    const int *seg_first;
+    const int4 *segs;
     float k[9];
-    int vec;               // 1: rows start on 16-byte boundaries
+    long long ld_in, ld_out, ld_pw;   // row pitches in floats (planes are ny rows); the
+                                      // three-plane-window kernel takes dense grids (nx)
+    int vec;               // 1: input rows start on 16-byte boundaries (three-plane-window kernel:
+                           // output rows too)
+    int vec_out;           // 1: output rows start on 16-byte boundaries
     int vec_pw;            // 1: the power map's rows start on 16-byte boundaries
     int use_tma;           // partial-sum kernel: stage planes with tensor-map bulk copies
     int *err;              // device flag: a bounded wait gave up (set to 1)
@@ -217,9 +221,11 @@ int tb3d_halo(const Shape3D &s);
 size_t tb3d_smem_bytes(const Shape3D &s);
 cudaError_t tb3d_prepare(const Shape3D &s, int *blocks_per_sm);
 cudaError_t tb3d_launch(const Shape3D &s, const Pass3D &p, const Tma3D &t, cudaStream_t st);
-// encode the tensor map of a (nx, ny, nz) float32 grid with a (bx, by, 1) box; false if the
-// driver entry point or the encoding is unavailable
-bool tma3d_encode(CUtensorMap *m, const float *base, int nx, int ny, int nz, int bx, int by);
+// encode the tensor map of a (nx, ny, nz) float32 grid, rows ld floats apart, with a
+// (bx, by, 1) box; false if rows are not on 16-byte boundaries or the driver entry point or the
+// encoding is unavailable
+bool tma3d_encode(CUtensorMap *m, const float *base, int nx, int ny, int nz, long long ld, int bx,
+                  int by);
 
 // Resident tiles (res2d.cu): the whole 2D grid held on chip by nbx x nby co-resident blocks
 // for a run of `steps` steps, halos exchanged through L2 every T steps (an epoch).

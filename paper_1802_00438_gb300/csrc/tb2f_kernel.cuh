@@ -818,8 +818,10 @@ __global__ void __launch_bounds__(32) k_tb2f(const Pass2D p)
         for (int j = 0; j < V / 2; j++) A[s][j] = B[s][j] = make_float2(0.f, 0.f);
     long long f, fend;
     if (p.starts) {
-        f = __ldg(p.starts + blockIdx.x);
-        fend = __ldg(p.starts + blockIdx.x + 1);
+        // (a broadcast, so that the compiler knows the bounds, and what follows from them, to be
+        // uniform across the warp and keeps it in uniform registers)
+        f = __shfl_sync(0xffffffffu, __ldg(p.starts + blockIdx.x), 0);
+        fend = __shfl_sync(0xffffffffu, __ldg(p.starts + blockIdx.x + 1), 0);
     } else {
         f = (long long)blockIdx.x * p.rows_per_cta;
         fend = min(f + p.rows_per_cta, p.total_rows);

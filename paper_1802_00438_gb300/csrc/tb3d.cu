@@ -89,12 +89,13 @@ EncodeTiledFn encode_fn()
 }
 }  // namespace
 
-bool tma3d_encode(CUtensorMap *m, const float *base, int nx, int ny, int nz, int bx, int by)
+bool tma3d_encode(CUtensorMap *m, const float *base, int nx, int ny, int nz, long long ld, int bx,
+                  int by)
 {
     EncodeTiledFn fn = encode_fn();
-    if (!fn || !base || (uintptr_t)base % 16 != 0 || nx % 4 != 0) return false;
+    if (!fn || !base || (uintptr_t)base % 16 != 0 || ld % 4 != 0 || ld < nx) return false;
     const cuuint64_t dim[3] = {(cuuint64_t)nx, (cuuint64_t)ny, (cuuint64_t)nz};
-    const cuuint64_t stride[2] = {(cuuint64_t)nx * 4, (cuuint64_t)nx * ny * 4};
+    const cuuint64_t stride[2] = {(cuuint64_t)ld * 4, (cuuint64_t)ld * ny * 4};
     const cuuint32_t box[3] = {(cuuint32_t)bx, (cuuint32_t)by, 1};
     const cuuint32_t estr[3] = {1, 1, 1};
     // out-of-bound cells of a box arrive as zeros (FLOAT_OOB_FILL_NONE)

@@ -1,30 +1,43 @@
 // 3D temporally-blocked Jacobi sweep, contracted arithmetic, partial sums along z.
 //
 // Method (arXiv 1802.00438): 2D spatial blocking in x and y with streaming along z (Sec. 3.1),
-// overlapped tiles with halos of width >= rad*T (Eq. 2), a chain of T stages where stage t
-// computes time step t one plane behind stage t-1 (Sec. 3.2), redundant halo computation with
-// only the compute block written (Sec. 3.2), trailing stages forwarding when a pass fuses fewer
-// than T steps (Sec. 3.2), clamped boundaries at every stage (Sec. 5.1).
+// overlapped tiles with halos of width >= rad*T (Eq. 2), a chain of T stages where stage s
+// computes time step s+1 (Sec. 3.2), redundant halo computation with only the compute block
+// written (Sec. 3.2), trailing stages forwarding when a pass fuses fewer than T steps (Sec. 3.2),
+// clamped boundaries at every stage (Sec. 5.1).
 //
 // GPU mapping: tile 32*VX x NW*VY cells incl. halos; a thread owns VX adjacent x cells of VY
 // consecutive rows, a warp spans the tile's width, warps are stacked along y.
-//   Stage 0 evaluates plane z-1 directly from a cp.async ring of input planes in shared memory.
-//   Stages 1..T-1 consume the plane the previous stage has just produced, in the same z
-//   iteration, and keep only two partial sums per cell instead of a three-plane window: when
-//   plane z of its input arrives, a stage
+//   A stage keeps two partial sums per cell instead of a three-plane window: when plane z of its
+//   input (time s) arrives it
 //     finishes output plane z-1:   out = P + ca*d
 //     starts   output plane z:     P   = Q + cc*d + cw*w + ce*e + cs*s + cn*n (+ sdc*p(z))
 //     starts   output plane z+1:   Q   = cb*d (+ ca*amb)
-//   The rows above and below a warp's rows come from its neighbour warps through a small
-//   shared-memory exchange (one barrier per stage and plane); x neighbours are warp shuffles.
+//   Stage s works two planes behind stage s-1: the plane a stage emits in one iteration is the
+//   next stage's input in the next one.  So the T stages of an iteration are independent of each
+//   other (their shuffles, loads and multiply-adds interleave), and the rows above and below a
+//   warp's rows, which come from its neighbour warps through a shared-memory exchange
+//   (alternating buffers), need ONE barrier per plane for all stages together instead of one
+//   per stage; a segment pays T-1 more iterations to drain.
+//   Arithmetic is on packed float32 pairs (fma.rn.f32x2): a packed operation holds the FMA pipe
+//   for two cycles but takes one issue slot, and issue is what bounds these kernels.  A pair is
+//   cells p and p + VX/2 of a row (VX = 2: the two adjacent cells): its west and east neighbours
+//   are the pairs p-1 and p+1, only the outermost pairs mix halves; its y and z neighbours are
+//   pairs as they lie, and with VX = 2 loads, stores and the exchange move whole pairs.
 //   Clamped z boundaries: at z = 0 the missing plane z-1 is plane 0 itself (Q is started from
-//   d before it is used), and the missing plane nz is plane nz-1: a stage that reaches the
-//   virtual plane nz finishes plane nz-1 from the repeated input and then repeats that output
-//   so that the next stage sees the same clamp.
-//   Power (Hotspot 3D) is staged with the field: a second cp.async ring holds the power planes
-//   of every stage's current plane, so each power value is read from HBM once per pass.
-//   Ring slots advance with the z iteration as rolling indices (no integer division in the
-//   steady state); shared memory is addressed with 32-bit shared-window addresses.
+//   d before it is used); on arrival of plane nz-1 a stage completes P with ca*d (the missing
+//   plane nz is plane nz-1), and emits it unchanged one iteration later.
+//   Tile columns of one pass are streamed in step (see best_segments in api.cu).
+//   Measured (GB300), kernel with one barrier per stage and scalar arithmetic -> this one: 512^3
+//   diffusion 1022 -> 1330 GCell/s, 512^2 x 256 Hotspot 837 -> 1033, 187 x 141 x 93 diffusion 172
+//   -> 304.  What bounds it now (ncu, 512^2 x 256, T = 3): issue 57 % active with 275
+//   instructions per thread and plane (115 of them multiply-adds, the other half shuffles,
+//   exchange, ring and store addressing), FMA pipe 41 %, shared memory 50 %, DRAM 3.2 TB/s; the
+//   warps run the shuffle phase and the multiply-add phase of a plane together.  Tried and not
+//   kept: neighbour flags instead of the barrier (1054 against 1265 at the time: polling costs
+//   more than the barrier's wait), 16 cells per thread in 8 warps (1172 against 1287).
+//   Input planes arrive in a shared-memory ring, PF planes ahead; every stage reads its power
+//   plane from a second ring (Hotspot 3D), so each value is read from HBM once per pass.
 #pragma once
 #include <type_traits>
 #include "common.cuh"
@@ -37,32 +50,41 @@ struct TB3F {
     static constexpr int NT = 32 * NW;
     static constexpr int BX = 32 * VX;
     static constexpr int BY = NW * VY;
+    static constexpr int H = VX / 2;             // pairs per row of a thread
     static constexpr int HX = (T + 3) / 4 * 4;   // 16-byte aligned tile origins
     static constexpr int HY = T;
     static constexpr int CX = BX - 2 * HX;
     static constexpr int CY = BY - 2 * HY;
-    static constexpr int NS = T > 1 ? T - 1 : 1;
     static constexpr int PLANE = BX * BY;
     static constexpr uint32_t PLANE_B = 4u * PLANE;
-    static constexpr size_t XCH = (size_t)NS * NW * 2 * BX;   // [stage][warp][top/bottom][BX]
-    // shared memory with PF planes in flight past the newest read: field ring of planes z-1,
-    // z, z+1 and PF more; power ring of planes z-max(T-1,1) .. z+PF (stage 0 reads plane z-1
-    // also when T = 1); exchange; one mbarrier per field slot (tensor-map staging)
-    static constexpr size_t smem_for(int pf)
+    static constexpr uint32_t ROWB = 4u * BX;
+    // exchange of stages 1 .. T-1: [buffer][stage][2*NW + 2 rows], warp w's top row at 2w + 1,
+    // its bottom row at 2w + 2 (the outermost rows are never written: they only feed halo rows)
+    static constexpr uint32_t XROWS = 2 * NW + 2;
+    static constexpr uint32_t XSTAGE = XROWS * ROWB;
+    static constexpr uint32_t XBUF = (T - 1) * XSTAGE;
+    // power planes an iteration reads: stage s reads plane Z0 - 2s
+    static constexpr int PWIN = 2 * T - 1;
+    // shared memory with PF planes in flight and xb exchange buffers: one row of padding at
+    // either end (a tile's first row looks one row up, its last row one row down), the field
+    // ring, the power ring, the exchange, one mbarrier per field slot
+    static constexpr size_t smem_for(int pf, int xb)
     {
-        return sizeof(float) * ((size_t)((pf + 3) + (KIND == KTHERM ? (T > 1 ? T : 2) + pf : 0)) *
-                                    PLANE + XCH) + 8 * (pf + 3);
+        return 2 * ROWB + (size_t)((pf + 1) + (KIND == KTHERM ? PWIN + pf : 0)) * PLANE_B +
+               (size_t)xb * XBUF + 8 * (pf + 1);
     }
     // blocks of up to 8 warps run two per SM, larger ones one
     static constexpr int MINB = NT <= 256 ? 2 : 1;
-    // the deepest prefetch (2..5 planes) whose shared memory fits MINB blocks per SM (1 KiB of
-    // each block's share is reserved by the hardware)
+    // (1 KiB of each block's share is reserved by the hardware)
     static constexpr size_t BUDGET = MINB == 2 ? 113 * 1024 : 227 * 1024;
-    static constexpr int PF = smem_for(5) <= BUDGET ? 5 : smem_for(4) <= BUDGET ? 4
-                            : smem_for(3) <= BUDGET ? 3 : 2;
-    static constexpr int NBF = PF + 3;
-    static constexpr int NBP = KIND == KTHERM ? (T > 1 ? T : 2) + PF : 0;
-    static constexpr size_t SMEM = smem_for(PF);
+    // alternating exchange buffers where they fit with at least one plane in flight, else one
+    // buffer and a second barrier per plane; then the deepest prefetch (up to 4 planes) that fits
+    static constexpr int XB = smem_for(1, 2) <= BUDGET ? 2 : 1;
+    static constexpr int PF = smem_for(4, XB) <= BUDGET ? 4 : smem_for(3, XB) <= BUDGET ? 3
+                            : smem_for(2, XB) <= BUDGET ? 2 : 1;
+    static constexpr int NBF = PF + 1;
+    static constexpr int NBP = KIND == KTHERM ? PWIN + PF : 0;
+    static constexpr size_t SMEM = smem_for(PF, XB);
     static_assert(CX > 0 && CY > 0, "tile smaller than its halos");
     static_assert(VX == 2 || VX == 4, "cells per lane");
     static_assert(VX * VY <= 32, "store mask");
@@ -75,11 +97,12 @@ struct CtxF3 {
     float *__restrict__ out;
     const float *__restrict__ pw;
     int nx, ny, nz, tsteps, vec, vec_pw;
-    long long plane;       // nx * ny
+    long long ld_in, ld_out, ld_pw;           // row pitches, floats
+    long long plane_in, plane_out, plane_pw;  // plane pitches, floats
     int x0, y0;            // tile origin
     int gx, gy;            // my first cell
     int z_start, last_plane, z0, z1;
-    bool edge_x, edge_y;   // warp touches a domain edge in x / in y
+    bool edge_y;           // warp touches a domain edge in y
     bool lx0;              // my cell 0 is x = 0
     unsigned rxm;          // bit j: my cell j is x = nx-1 (a mask, not an index: a compare of
                            // the index per cell would become an indexed store to memory)
@@ -87,45 +110,59 @@ struct CtxF3 {
     unsigned st_mask;      // bit (k*VX + j): my cell (row k, x j) is stored
     unsigned st_rows;      // bit k: my row k is stored whole
     bool st_fast;          // vector stores: every row whole or empty, aligned rows
-    long long st_off;      // gy * nx + gx
+    long long st_off;      // gy * ld_out + gx
     int tid, lane, wid;
-    float k[9];
-    float ca_amb;
 };
 
-template <int VX>
-struct VecF;
-template <>
-struct VecF<2> {
-    float v[2];
-};
-template <>
-struct VecF<4> {
-    float v[4];
+// Coefficients as pairs of equal values, the operands of the packed float32 operations.
+struct Coef3 {
+    float2 cc, cw, ce, cs, cn, cb, ca, sdc, ca_amb;
 };
 
+// a thread's row of VX cells as pairs: (x, y) of v[p] are cells p and p + VX/2
 template <int VX>
-__device__ __forceinline__ VecF<VX> ldsv(uint32_t a)
+__device__ __forceinline__ void lds_pairs(uint32_t a, float2 (&v)[VX / 2])
 {
-    VecF<VX> r;
-    if constexpr (VX == 2)
-        asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];\n" : "=f"(r.v[0]), "=f"(r.v[1]) : "r"(a));
-    else
+    if constexpr (VX == 2) {
+        asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];\n" : "=f"(v[0].x), "=f"(v[0].y) : "r"(a));
+    } else {
         asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];\n"
-                     : "=f"(r.v[0]), "=f"(r.v[1]), "=f"(r.v[2]), "=f"(r.v[3])
+                     : "=f"(v[0].x), "=f"(v[1].x), "=f"(v[0].y), "=f"(v[1].y)
                      : "r"(a));
-    return r;
+    }
+}
+
+// exchange rows stay in pair order
+template <int VX>
+__device__ __forceinline__ void lds_xch(uint32_t a, float2 (&v)[VX / 2])
+{
+#pragma unroll
+    for (int p = 0; p < VX / 2; p++)
+        asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];\n"
+                     : "=f"(v[p].x), "=f"(v[p].y)
+                     : "r"(a + 256u * p));
 }
 
 template <int VX>
-__device__ __forceinline__ void stsv(uint32_t a, const float *x)
+__device__ __forceinline__ void sts_xch(uint32_t a, const float2 (&v)[VX / 2])
 {
-    if constexpr (VX == 2)
-        asm volatile("st.shared.v2.f32 [%0], {%1, %2};\n" ::"r"(a), "f"(x[0]), "f"(x[1]) : "memory");
-    else
-        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"r"(a), "f"(x[0]), "f"(x[1]),
-                     "f"(x[2]), "f"(x[3])
+#pragma unroll
+    for (int p = 0; p < VX / 2; p++)
+        asm volatile("st.shared.v2.f32 [%0], {%1, %2};\n" ::"r"(a + 256u * p), "f"(v[p].x), "f"(v[p].y)
                      : "memory");
+}
+
+template <int H>
+__device__ __forceinline__ float cell3(const float2 (&v)[H], int j)
+{
+    return j < H ? v[j < H ? j : 0].x : v[j < H ? 0 : j - H].y;
+}
+
+template <int H>
+__device__ __forceinline__ void set_cell3(float2 (&v)[H], int j, float x)
+{
+    if (j < H) v[j < H ? j : 0].x = x;
+    else v[j < H ? 0 : j - H].y = x;
 }
 
 __device__ __forceinline__ void cpa16(uint32_t dst, const void *src, int nbytes)
@@ -182,10 +219,11 @@ __device__ __forceinline__ void tma_plane(uint32_t dst, const CUtensorMap *m, in
         : "memory");
 }
 
-// Stage the tile's window of one plane (z-plane base `src`) into the slot at `dst`; cells
-// outside the domain arrive as zeros.
+// Stage the tile's window of one plane (z-plane base `src`, rows ld apart) into the slot at
+// `dst` by per-thread copies; cells outside the domain arrive as zeros.
 template <int BX, int BY, int NT>
-__device__ __forceinline__ void tbf3_load(const CtxF3 &c, const float *src, int vec, uint32_t dst)
+__device__ __forceinline__ void tbf3_load(const CtxF3 &c, const float *src, long long ld, int vec,
+                                          uint32_t dst)
 {
     constexpr int CH = BX / 4;
     constexpr int NCH = CH * BY;
@@ -197,7 +235,7 @@ __device__ __forceinline__ void tbf3_load(const CtxF3 &c, const float *src, int 
             const int y = c.y0 + row, x = c.x0 + 4 * ch;
             const uint32_t d = dst + 4u * (row * BX + 4 * ch);
             const bool yok = (y >= 0 && y < c.ny);
-            const float *rs = src + (long long)(yok ? y : 0) * c.nx;
+            const float *rs = src + (long long)(yok ? y : 0) * ld;
             if (vec) {
                 const int nb = (yok && x >= 0 && x < c.nx) ? min(16, 4 * (c.nx - x)) : 0;
                 cpa16(d, nb ? rs + x : src, nb);
@@ -213,103 +251,93 @@ __device__ __forceinline__ void tbf3_load(const CtxF3 &c, const float *src, int 
     }
 }
 
-// Neighbours of my cells in a plane held as m[VY][VX]: w/e inside my cells or by shuffle,
-// n/s from my rows or the rows of the warps above (nt) and below (sb).
-// Clamped domain edges are applied to the plane, not to the neighbour arrays: in a warp that
-// touches an edge, the out-of-domain cell next to each edge cell (a ghost: its own value is
-// never used) takes the edge cell's value, inside my cells (m, in place) or in the value that
-// arrives from another lane or warp (wl, er, nt, sb).  The neighbour arrays stay pure renames of
-// m, so the common path keeps no second copy of them.
-template <int VX, int VY, bool EDGE>
-__device__ __forceinline__ void nbf3(const CtxF3 &c, float (&m)[VY][VX], float (&nt)[VX],
-                                     float (&sb)[VX], float (&w)[VY][VX], float (&e)[VY][VX],
-                                     float (&n)[VY][VX], float (&s)[VY][VX])
+// Clamped x and y edges of a plane d with its outer rows nt and sb and the values wl, er from the
+// neighbour lanes, in a warp that touches an edge: the out-of-domain cell next to each edge cell
+// (a ghost: its own value is never used) takes the edge cell's value, inside my cells (d, in
+// place) or in the value that arrives from another lane or warp.  The neighbours stay pure
+// renames of d, so the common path keeps no second copy of them.
+// (every index stays in range even in code the unrolling discards: an out-of-range constant
+// index, even in a dead branch, makes the compiler keep the array in memory)
+// Which edges an instance handles (a tile column runs one that covers what it touches).
+enum : int {
+    E3X = 1,   // x = 0 or x = nx-1
+    E3Y = 2,   // y = 0 or y = ny-1
+};
+
+template <int VX, int VY, int EDGE>
+__device__ __forceinline__ void edge3(const CtxF3 &c, float2 (&d)[VY][VX / 2], float2 (&nt)[VX / 2],
+                                      float2 (&sb)[VX / 2], float (&wl)[VY], float (&er)[VY])
 {
-    float wl[VY], er[VY];
-#pragma unroll
-    for (int k = 0; k < VY; k++) {
-        wl[k] = __shfl_sync(0xffffffffu, m[k][VX - 1], (c.lane + 31) & 31);
-        er[k] = __shfl_sync(0xffffffffu, m[k][0], (c.lane + 1) & 31);
-    }
-    if (EDGE && c.edge_y) {
+    constexpr int H = VX / 2;
+    if ((EDGE & E3Y) && c.edge_y) {
         // y = 0 at my row k: ghost row k-1 (or the row above, nt) := row k; likewise below
 #pragma unroll
-        for (int j = 0; j < VX; j++) {
-            nt[j] = (c.ym0 & 1u) ? m[0][j] : nt[j];
-            sb[j] = ((c.ymn >> (VY - 1)) & 1u) ? m[VY - 1][j] : sb[j];
+        for (int p = 0; p < H; p++) {
+            nt[p].x = (c.ym0 & 1u) ? d[0][p].x : nt[p].x;
+            nt[p].y = (c.ym0 & 1u) ? d[0][p].y : nt[p].y;
+            sb[p].x = ((c.ymn >> (VY - 1)) & 1u) ? d[VY - 1][p].x : sb[p].x;
+            sb[p].y = ((c.ymn >> (VY - 1)) & 1u) ? d[VY - 1][p].y : sb[p].y;
         }
 #pragma unroll
-        for (int k = 1; k < VY; k++)
+        for (int k = 1; k < VY; k++) {
+            const bool g = (c.ym0 >> k) & 1u;
 #pragma unroll
-            for (int j = 0; j < VX; j++) m[k - 1][j] = ((c.ym0 >> k) & 1u) ? m[k][j] : m[k - 1][j];
+            for (int p = 0; p < H; p++) {
+                d[k - 1][p].x = g ? d[k][p].x : d[k - 1][p].x;
+                d[k - 1][p].y = g ? d[k][p].y : d[k - 1][p].y;
+            }
+        }
 #pragma unroll
-        for (int k = 0; k < VY - 1; k++)
+        for (int k = 0; k < VY - 1; k++) {
+            const bool g = (c.ymn >> k) & 1u;
 #pragma unroll
-            for (int j = 0; j < VX; j++) m[k + 1][j] = ((c.ymn >> k) & 1u) ? m[k][j] : m[k + 1][j];
+            for (int p = 0; p < H; p++) {
+                d[k + 1][p].x = g ? d[k][p].x : d[k + 1][p].x;
+                d[k + 1][p].y = g ? d[k][p].y : d[k + 1][p].y;
+            }
+        }
     }
-    if (EDGE && c.edge_x) {
+    if (EDGE & E3X) {
         // x = 0 is always my cell 0 (tile origins are multiples of 4); x = nx-1 is my cell j
 #pragma unroll
         for (int k = 0; k < VY; k++) {
-            wl[k] = c.lx0 ? m[k][0] : wl[k];
-            er[k] = ((c.rxm >> (VX - 1)) & 1u) ? m[k][VX - 1] : er[k];
+            wl[k] = c.lx0 ? d[k][0].x : wl[k];
+            er[k] = ((c.rxm >> (VX - 1)) & 1u) ? d[k][H - 1].y : er[k];
 #pragma unroll
-            for (int j = 1; j < VX; j++) m[k][j] = ((c.rxm >> (j - 1)) & 1u) ? m[k][j - 1] : m[k][j];
+            for (int j = 1; j < VX; j++) {
+                const float e = cell3(d[k], j - 1), own = cell3(d[k], j);
+                set_cell3(d[k], j, ((c.rxm >> (j - 1)) & 1u) ? e : own);
+            }
         }
     }
-    // (every index below stays in range even in code the unrolling discards: an out-of-range
-    // constant index, even in a dead branch, makes the compiler keep the array in memory)
-#pragma unroll
-    for (int k = 0; k < VY; k++) {
-        w[k][0] = wl[k];
-        e[k][VX - 1] = er[k];
-#pragma unroll
-        for (int j = 1; j < VX; j++) w[k][j] = m[k][j - 1];
-#pragma unroll
-        for (int j = 0; j < VX - 1; j++) e[k][j] = m[k][j + 1];
-    }
-#pragma unroll
-    for (int j = 0; j < VX; j++) {
-        n[0][j] = nt[j];
-        s[VY - 1][j] = sb[j];
-    }
-#pragma unroll
-    for (int k = 1; k < VY; k++)
-#pragma unroll
-        for (int j = 0; j < VX; j++) n[k][j] = m[k - 1][j];
-#pragma unroll
-    for (int k = 0; k < VY - 1; k++)
-#pragma unroll
-        for (int j = 0; j < VX; j++) s[k][j] = m[k + 1][j];
 }
 
+// my cells of the compute block; dst: my first cell of the plane
 template <int VX, int VY>
-__device__ __forceinline__ void tbf3_store(const CtxF3 &c, int z, const float (&v)[VY][VX])
+__device__ __forceinline__ void tbf3_store(const CtxF3 &c, float *dst, const float2 (&v)[VY][VX / 2])
 {
-    float *dst = c.out + (long long)z * c.plane + c.st_off;
     if (c.st_fast) {
         // every row of mine is stored whole or not at all, with aligned vector stores
 #pragma unroll
         for (int k = 0; k < VY; k++) {
-            float *d = dst + (long long)k * c.nx;
             if ((c.st_rows >> k) & 1u) {
-                if constexpr (VX == 2) *reinterpret_cast<float2 *>(d) = make_float2(v[k][0], v[k][1]);
-                else *reinterpret_cast<float4 *>(d) = make_float4(v[k][0], v[k][1], v[k][2], v[k][3]);
+                if constexpr (VX == 2)
+                    *reinterpret_cast<float2 *>(dst) = v[k][0];
+                else
+                    *reinterpret_cast<float4 *>(dst) =
+                        make_float4(v[k][0].x, v[k][VX / 2 - 1].x, v[k][0].y, v[k][VX / 2 - 1].y);
             }
+            dst += c.ld_out;
         }
     } else {
 #pragma unroll
-        for (int k = 0; k < VY; k++)
+        for (int k = 0; k < VY; k++) {
 #pragma unroll
             for (int j = 0; j < VX; j++)
-                if ((c.st_mask >> (VX * k + j)) & 1u) dst[(long long)k * c.nx + j] = v[k][j];
+                if ((c.st_mask >> (VX * k + j)) & 1u) dst[j] = cell3(v[k], j);
+            dst += c.ld_out;
+        }
     }
-}
-
-template <int N>
-__device__ __forceinline__ int slot_of(int rel)   // rel >= -2N
-{
-    return (rel + 2 * N) % N;
 }
 
 template <int N>
@@ -319,203 +347,126 @@ __device__ __forceinline__ int slot_back(int s, int k)   // (s - k) mod N for 0 
     return r < 0 ? r + N : r;
 }
 
-// Ring slots of the current iteration: field plane Z0 and power plane Z0-1.
-struct Slots3 {
-    int f0;
-    int p1;
-};
-
-template <int KIND>
-__device__ __forceinline__ float upd3f(const CtxF3 &c, float m, float w, float e, float s,
-                                       float n, float b, float a, float p)
-{
-    if (KIND == KDIFF) return diff7<false>(m, w, e, s, n, b, a, c.k);
-    else return hot3<false>(m, w, e, s, n, b, a, p, c.k, c.ca_amb);
-}
-
-template <int KIND, int T, int VX, int VY, int NW, bool SPECIAL, bool EDGE>
-__device__ __forceinline__ void tbf3_iter(const CtxF3 &c, uint32_t sring, uint32_t spw,
-                                          uint32_t sxch, const Slots3 &sl,
-                                          const float (&P)[TB3F<KIND, T, VX, VY, NW>::NS][VY][VX],
-                                          const float (&Q)[TB3F<KIND, T, VX, VY, NW>::NS][VY][VX],
-                                          float (&Pn)[TB3F<KIND, T, VX, VY, NW>::NS][VY][VX],
-                                          float (&Qn)[TB3F<KIND, T, VX, VY, NW>::NS][VY][VX], int i)
+// One iteration: stage s receives plane Z0 - 2s of time s (stage 0 from the ring slot at `field`,
+// the others in D[s-1]) and emits plane Z0 - 2s - 1 of time s+1 into D[s], the last stage into
+// the output (dst: my first cell there).  p0: ring slot of power plane Z0; xr / xw: exchange
+// buffers read and written.
+template <int KIND, int T, int VX, int VY, int NW, bool SPECIAL, int EDGE>
+__device__ __forceinline__ void tbf3_iter(const CtxF3 &c, const Coef3 &k, uint32_t field,
+                                          uint32_t spw, int p0, uint32_t xr, uint32_t xw, float *dst,
+                                          float2 (&P)[T][VY][VX / 2], float2 (&Q)[T][VY][VX / 2],
+                                          float2 (&D)[T][VY][VX / 2], int Z0)
 {
     using C = TB3F<KIND, T, VX, VY, NW>;
-    const int Z0 = c.z_start + i;   // newest plane in the ring
-    const float cc = c.k[0], cw = c.k[1], ce = c.k[2], cs = c.k[3], cn = c.k[4], cb = c.k[5],
-                ca = c.k[6];
-    const uint32_t own = 4u * (c.wid * VY * C::BX + VX * c.lane);   // my row 0, cell 0
-    float d[VY][VX];
-
-    // ---- stage 0: plane R = Z0 - 1 from the ring ------------------------------------------
-    {
-        int fu, fm, fd, pm;
-        if (SPECIAL) {
-            const int R = min(Z0 - 1, c.nz - 1);   // past the bottom: repeat plane nz-1
-            fu = slot_of<C::NBF>(max(R - 1, 0) - c.z_start);
-            fm = slot_of<C::NBF>(R - c.z_start);
-            fd = slot_of<C::NBF>(min(R + 1, c.nz - 1) - c.z_start);
-            pm = KIND == KTHERM ? slot_of<C::NBP ? C::NBP : 1>(max(R, 0) - c.z_start) : 0;
+    constexpr int H = VX / 2;
+    const uint32_t own = C::ROWB * (c.wid * VY) + 4u * VX * c.lane;   // my row 0, cell 0 of a plane
+    const uint32_t xo = C::ROWB * (2 * c.wid + 1) + 8u * c.lane;      // my top row in the exchange
+    float2 xn[T][H], xs[T][H];
+    if constexpr (C::XB == 1 && T > 1) {   // one buffer: every read before the first write
+#pragma unroll
+        for (int s = 1; s < T; s++) {
+            lds_xch<VX>(xr + (s - 1) * C::XSTAGE + xo - C::ROWB, xn[s]);
+            lds_xch<VX>(xr + (s - 1) * C::XSTAGE + xo + 2 * C::ROWB, xs[s]);
+        }
+        __syncthreads();
+    }
+    float2 res[VY][H];   // the last stage's plane
+#pragma unroll
+    for (int s = T - 1; s >= 0; s--) {
+        const int zc = Z0 - 2 * s;   // the plane that arrives
+        float2 d[VY][H], nt[H], sb[H], o[VY][H];
+        if (s == 0) {
+#pragma unroll
+            for (int r = 0; r < VY; r++) lds_pairs<VX>(field + own + r * C::ROWB, d[r]);
         } else {
-            fd = sl.f0;
-            fm = slot_back<C::NBF>(fd, 1);
-            fu = slot_back<C::NBF>(fd, 2);
-            pm = sl.p1;
+#pragma unroll
+            for (int r = 0; r < VY; r++)
+#pragma unroll
+                for (int p = 0; p < H; p++) d[r][p] = D[s > 0 ? s - 1 : 0][r][p];
         }
-        const uint32_t au = sring + fu * C::PLANE_B + own;
-        const uint32_t am = sring + fm * C::PLANE_B + own;
-        const uint32_t ad = sring + fd * C::PLANE_B + own;
-        float u[VY][VX], m[VY][VX], a[VY][VX], w[VY][VX], e[VY][VX], n[VY][VX], s[VY][VX];
-        float p[VY][VX];
+        if (SPECIAL && s >= c.tsteps) {
+            // forwarding stage: one plane of delay, no arithmetic
 #pragma unroll
-        for (int k = 0; k < VY; k++) {
-            const VecF<VX> x = ldsv<VX>(au + 4u * k * C::BX);
-            const VecF<VX> y = ldsv<VX>(am + 4u * k * C::BX);
-            const VecF<VX> z = ldsv<VX>(ad + 4u * k * C::BX);
+            for (int r = 0; r < VY; r++)
 #pragma unroll
-            for (int j = 0; j < VX; j++) {
-                u[k][j] = x.v[j];
-                m[k][j] = y.v[j];
-                a[k][j] = z.v[j];
-            }
-        }
-        float nt[VX], sb[VX];
-        {
-            const int up = c.wid > 0 ? -1 : 0, dn = c.wid < NW - 1 ? VY : VY - 1;
-            const VecF<VX> x = ldsv<VX>(am + 4 * up * C::BX);
-            const VecF<VX> y = ldsv<VX>(am + 4 * dn * C::BX);
+                for (int p = 0; p < H; p++) {
+                    o[r][p] = P[s][r][p];
+                    P[s][r][p] = d[r][p];
+                }
+        } else {
+            if (s == 0) {
+                lds_pairs<VX>(field + own - C::ROWB, nt);
+                lds_pairs<VX>(field + own + VY * C::ROWB, sb);
+            } else if constexpr (C::XB == 1) {
 #pragma unroll
-            for (int j = 0; j < VX; j++) {
-                nt[j] = x.v[j];
-                sb[j] = y.v[j];
-            }
-        }
-        nbf3<VX, VY, EDGE>(c, m, nt, sb, w, e, n, s);
-        if (KIND == KTHERM) {
-            const uint32_t ap = spw + pm * C::PLANE_B + own;
-#pragma unroll
-            for (int k = 0; k < VY; k++) {
-                const VecF<VX> x = ldsv<VX>(ap + 4u * k * C::BX);
-#pragma unroll
-                for (int j = 0; j < VX; j++) p[k][j] = x.v[j];
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < VY; k++)
-#pragma unroll
-            for (int j = 0; j < VX; j++)
-                d[k][j] = upd3f<KIND>(c, m[k][j], w[k][j], e[k][j], s[k][j], n[k][j], u[k][j],
-                                      a[k][j], KIND == KTHERM ? p[k][j] : 0.f);
-    }
-    if constexpr (T == 1) {
-        const int R = Z0 - 1;
-        if (R >= c.z0 && R < c.z1) tbf3_store<VX, VY>(c, R, d);
-    } else {
-        constexpr uint32_t XS = 4u * NW * 2 * C::BX;   // bytes per stage in the exchange
-        const uint32_t xo = 4u * VX * c.lane;
-        const int wt = c.wid > 0 ? c.wid - 1 : 0;   // warp above (tile edge: any in-bounds row)
-        const int wb = c.wid < NW - 1 ? c.wid + 1 : NW - 1;
-#pragma unroll
-        for (int st = 1; st < T; st++) {
-            const int zc = Z0 - st;   // plane of d (output of stage st-1)
-            float o[VY][VX];
-            if (SPECIAL && st >= c.tsteps) {
-                // forwarding stage: one plane of delay, no arithmetic
-#pragma unroll
-                for (int k = 0; k < VY; k++)
-#pragma unroll
-                    for (int j = 0; j < VX; j++) {
-                        o[k][j] = Q[st - 1][k][j];
-                        Qn[st - 1][k][j] = d[k][j];
-                        Pn[st - 1][k][j] = P[st - 1][k][j];
-                    }
+                for (int p = 0; p < H; p++) {
+                    nt[p] = xn[s][p];
+                    sb[p] = xs[s][p];
+                }
             } else {
-                const uint32_t xw = sxch + (st - 1) * XS + xo;
-                stsv<VX>(xw + 4u * (c.wid * 2 + 0) * C::BX, d[0]);
-                stsv<VX>(xw + 4u * (c.wid * 2 + 1) * C::BX, d[VY - 1]);
-                __syncthreads();
-                float nt[VX], sb[VX];
-                {
-                    const VecF<VX> x = ldsv<VX>(xw + 4u * (wt * 2 + 1) * C::BX);
-                    const VecF<VX> y = ldsv<VX>(xw + 4u * (wb * 2 + 0) * C::BX);
-#pragma unroll
-                    for (int j = 0; j < VX; j++) {
-                        nt[j] = x.v[j];
-                        sb[j] = y.v[j];
-                    }
-                }
-                float w[VY][VX], e[VY][VX], n[VY][VX], s[VY][VX], p[VY][VX];
-                nbf3<VX, VY, EDGE>(c, d, nt, sb, w, e, n, s);
-                if (KIND == KTHERM) {
-                    int ps;
-                    if (SPECIAL)
-                        ps = slot_of<C::NBP ? C::NBP : 1>(min(max(zc, 0), c.nz - 1) - c.z_start);
-                    else
-                        ps = slot_back<C::NBP ? C::NBP : 1>(sl.p1, st - 1);
-                    const uint32_t ap = spw + ps * C::PLANE_B + own;
-#pragma unroll
-                    for (int k = 0; k < VY; k++) {
-                        const VecF<VX> x = ldsv<VX>(ap + 4u * k * C::BX);
-#pragma unroll
-                        for (int j = 0; j < VX; j++) p[k][j] = x.v[j];
-                    }
-                }
-                const float(&Ps)[VY][VX] = P[st - 1];
-                const float(&Qs)[VY][VX] = Q[st - 1];
-                float(&Pw)[VY][VX] = Pn[st - 1];
-                float(&Qw)[VY][VX] = Qn[st - 1];
-                if (!SPECIAL || zc < c.nz) {
-                    const bool first = SPECIAL && zc == 0;   // clamp: plane -1 is plane 0
-#pragma unroll
-                    for (int k = 0; k < VY; k++)
-#pragma unroll
-                        for (int j = 0; j < VX; j++) {
-                            const float dv = d[k][j];
-                            float qn;
-                            if (KIND == KTHERM) qn = __fmaf_rn(cb, dv, c.ca_amb);
-                            else qn = __fmul_rn(cb, dv);
-                            const float qi = first ? qn : Qs[k][j];
-                            o[k][j] = __fmaf_rn(ca, dv, Ps[k][j]);
-                            float r = qi;
-                            if (KIND == KTHERM) r = __fmaf_rn(c.k[7], p[k][j], r);
-                            r = __fmaf_rn(cc, dv, r);
-                            r = __fmaf_rn(cn, n[k][j], r);
-                            r = __fmaf_rn(cs, s[k][j], r);
-                            r = __fmaf_rn(ce, e[k][j], r);
-                            r = __fmaf_rn(cw, w[k][j], r);
-                            Pw[k][j] = r;
-                            Qw[k][j] = qn;
-                        }
-                } else if (zc == c.nz) {
-                    // virtual plane nz (= plane nz-1): finish plane nz-1 and keep it
-#pragma unroll
-                    for (int k = 0; k < VY; k++)
-#pragma unroll
-                        for (int j = 0; j < VX; j++) {
-                            o[k][j] = __fmaf_rn(ca, d[k][j], Ps[k][j]);
-                            Pw[k][j] = o[k][j];
-                            Qw[k][j] = Qs[k][j];
-                        }
-                } else {
-#pragma unroll
-                    for (int k = 0; k < VY; k++)
-#pragma unroll
-                        for (int j = 0; j < VX; j++) {
-                            o[k][j] = Ps[k][j];
-                            Pw[k][j] = Ps[k][j];
-                            Qw[k][j] = Qs[k][j];
-                        }
-                }
+                lds_xch<VX>(xr + (s - 1) * C::XSTAGE + xo - C::ROWB, nt);
+                lds_xch<VX>(xr + (s - 1) * C::XSTAGE + xo + 2 * C::ROWB, sb);
             }
+            // (before the shuffles: the power value is the first term after the pipeline's own --
+            // it is small, and added after the large terms it would round by their ulp)
+            float2 pv[VY][H];
+            if (KIND == KTHERM) {
+                const uint32_t ap = spw + slot_back<C::NBP ? C::NBP : 1>(p0, 2 * s) * C::PLANE_B + own;
 #pragma unroll
-            for (int k = 0; k < VY; k++)
+                for (int r = 0; r < VY; r++) lds_pairs<VX>(ap + r * C::ROWB, pv[r]);
+            }
+            float wl[VY], er[VY];
 #pragma unroll
-                for (int j = 0; j < VX; j++) d[k][j] = o[k][j];
+            for (int r = 0; r < VY; r++) {
+                wl[r] = __shfl_sync(0xffffffffu, d[r][H - 1].y, (c.lane + 31) & 31);
+                er[r] = __shfl_sync(0xffffffffu, d[r][0].x, (c.lane + 1) & 31);
+            }
+            if (EDGE) edge3<VX, VY, EDGE>(c, d, nt, sb, wl, er);
+            const bool first = SPECIAL && zc == 0;          // clamp: plane -1 is plane 0
+            const bool last = SPECIAL && zc == c.nz - 1;    // clamp: plane nz is plane nz-1
+            const bool past = SPECIAL && zc == c.nz;        // plane nz-1 is complete
+            // term by term over all the thread's pairs: consecutive operations are independent
+            // (a chain per cell would wait out the latency of each of its links)
+#define STN_PAIRS                                                                                  \
+    _Pragma("unroll") for (int r = 0; r < VY; r++) _Pragma("unroll") for (int p = 0; p < H; p++)
+            float2 t[VY][H];
+            if (first) {   // Q of plane 0: plane -1 is plane 0
+                STN_PAIRS Q[s][r][p] = KIND == KTHERM ? __ffma2_rn(k.cb, d[r][p], k.ca_amb) : __fmul2_rn(k.cb, d[r][p]);
+            }
+            STN_PAIRS o[r][p] = past ? P[s][r][p] : __ffma2_rn(k.ca, d[r][p], P[s][r][p]);
+            STN_PAIRS t[r][p] = KIND == KTHERM ? __ffma2_rn(k.sdc, pv[r][p], Q[s][r][p]) : Q[s][r][p];
+            STN_PAIRS t[r][p] = __ffma2_rn(k.cc, d[r][p], t[r][p]);
+            STN_PAIRS Q[s][r][p] = KIND == KTHERM ? __ffma2_rn(k.cb, d[r][p], k.ca_amb) : __fmul2_rn(k.cb, d[r][p]);
+            STN_PAIRS t[r][p] = __ffma2_rn(k.cn, r > 0 ? d[r > 0 ? r - 1 : 0][p] : nt[p], t[r][p]);
+            STN_PAIRS t[r][p] = __ffma2_rn(k.cs, r < VY - 1 ? d[r < VY - 1 ? r + 1 : r][p] : sb[p], t[r][p]);
+            // the outermost pairs take one half from a neighbour lane: their halves are added one
+            // by one (building the pair would cost as many register moves)
+            STN_PAIRS t[r][p] = p == H - 1
+                ? make_float2(__fmaf_rn(k.ce.x, d[r][0].y, t[r][p].x), __fmaf_rn(k.ce.x, er[r], t[r][p].y))
+                : __ffma2_rn(k.ce, d[r][p < H - 1 ? p + 1 : p], t[r][p]);
+            STN_PAIRS t[r][p] = p == 0
+                ? make_float2(__fmaf_rn(k.cw.x, wl[r], t[r][p].x), __fmaf_rn(k.cw.x, d[r][H - 1].x, t[r][p].y))
+                : __ffma2_rn(k.cw, d[r][p > 0 ? p - 1 : 0], t[r][p]);
+            if (last) STN_PAIRS t[r][p] = __ffma2_rn(k.ca, d[r][p], t[r][p]);
+            STN_PAIRS P[s][r][p] = t[r][p];
+#undef STN_PAIRS
         }
-        const int R = Z0 - T;
-        if (R >= c.z0 && R < c.z1) tbf3_store<VX, VY>(c, R, d);
+        if (s == T - 1) {
+#pragma unroll
+            for (int r = 0; r < VY; r++)
+#pragma unroll
+                for (int p = 0; p < H; p++) res[r][p] = o[r][p];
+        } else {
+#pragma unroll
+            for (int r = 0; r < VY; r++)
+#pragma unroll
+                for (int p = 0; p < H; p++) D[s][r][p] = o[r][p];
+            sts_xch<VX>(xw + s * C::XSTAGE + xo, o[0]);
+            sts_xch<VX>(xw + s * C::XSTAGE + xo + C::ROWB, o[VY - 1]);
+        }
     }
+    const int R = Z0 - 2 * T + 1;
+    if (R >= c.z0 && R < c.z1) tbf3_store<VX, VY>(c, dst, res);
 }
 
 template <int KIND, int T, int VX, int VY, int NW>
@@ -525,10 +476,10 @@ __global__ void __launch_bounds__(32 * NW, (TB3F<KIND, T, VX, VY, NW>::MINB))
 {
     using C = TB3F<KIND, T, VX, VY, NW>;
     extern __shared__ __align__(128) float smem[];
-    const uint32_t sring = smem_u32(smem);
+    const uint32_t sring = smem_u32(smem) + C::ROWB;
     const uint32_t spw = sring + C::NBF * C::PLANE_B;
     const uint32_t sxch = spw + C::NBP * C::PLANE_B;
-    const uint32_t sbar = sxch + (uint32_t)(4 * C::XCH);   // NBF mbarriers, 8 bytes each
+    const uint32_t sbar = sxch + C::XB * C::XBUF;   // NBF mbarriers, 8 bytes each
     const bool tma = p.use_tma != 0;
     if (tma) {
         if (threadIdx.x == 0) {
@@ -538,8 +489,8 @@ __global__ void __launch_bounds__(32 * NW, (TB3F<KIND, T, VX, VY, NW>::MINB))
         }
         __syncthreads();
     }
-    unsigned phase = 0;     // bit b: parity of the next completion of barrier b
-    unsigned pending = 0;   // bit b: a copy on barrier b has not been waited for
+    uint32_t f0 = 0, fpar = 0;   // field slot of the next plane to arrive, its parity
+    bool bad = false;       // a bounded wait of mine gave up: no further copies, no further waits
     CtxF3 c;
     c.in = p.in;
     c.out = p.out;
@@ -547,54 +498,47 @@ __global__ void __launch_bounds__(32 * NW, (TB3F<KIND, T, VX, VY, NW>::MINB))
     c.nx = p.nx;
     c.ny = p.ny;
     c.nz = p.nz;
-    c.plane = (long long)p.nx * p.ny;
+    c.ld_in = p.ld_in;
+    c.ld_out = p.ld_out;
+    c.ld_pw = p.ld_pw;
+    c.plane_in = p.ld_in * p.ny;
+    c.plane_out = p.ld_out * p.ny;
+    c.plane_pw = p.ld_pw * p.ny;
     c.tsteps = p.tsteps;
     c.vec = p.vec;
     c.vec_pw = p.vec_pw;
     c.tid = threadIdx.x;
     c.lane = threadIdx.x & 31;
-    c.wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int j = 0; j < 9; j++) c.k[j] = p.k[j];
-    c.ca_amb = (KIND == KTHERM) ? __fmul_rn(p.k[6], p.k[8]) : 0.f;
+    c.wid = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);
+    Coef3 k;
+    auto pair = [&](int i) { return make_float2(p.k[i], p.k[i]); };
+    k.cc = pair(0);
+    k.cw = pair(1);
+    k.ce = pair(2);
+    k.cs = pair(3);
+    k.cn = pair(4);
+    k.cb = pair(5);
+    k.ca = pair(6);
+    k.sdc = pair(7);
+    const float ca_amb = KIND == KTHERM ? __fmul_rn(p.k[6], p.k[8]) : 0.f;
+    k.ca_amb = make_float2(ca_amb, ca_amb);
 
-    float PA[C::NS][VY][VX], QA[C::NS][VY][VX], PB[C::NS][VY][VX], QB[C::NS][VY][VX];
+    float2 P[T][VY][C::H], Q[T][VY][C::H], D[T][VY][C::H];
 #pragma unroll
-    for (int s = 0; s < C::NS; s++)
+    for (int s = 0; s < T; s++)
 #pragma unroll
-        for (int k = 0; k < VY; k++)
+        for (int r = 0; r < VY; r++)
 #pragma unroll
-            for (int j = 0; j < VX; j++) PA[s][k][j] = QA[s][k][j] = PB[s][k][j] = QB[s][k][j] = 0.f;
+            for (int q = 0; q < C::H; q++) P[s][r][q] = Q[s][r][q] = D[s][r][q] = make_float2(0.f, 0.f);
 
-    // segments: zslab > 0 -- pieces (tile column, z-slab), taken round-robin, so that the
-    // blocks of one round stream neighbouring tile columns through the same z-planes together
-    // and the halo one of them re-reads is still in L2; else a contiguous range of
-    // (tile column, plane) units per block, balanced by cost on the host
-    long long f = (long long)blockIdx.x * p.planes_per_cta, pc = blockIdx.x;
-    const long long total = p.total_cols * p.nz;
-    long long fend = min(f + p.planes_per_cta, total);
-    if (p.starts) {   // cost-balanced ranges
-        f = __ldg(p.starts + blockIdx.x);
-        fend = __ldg(p.starts + blockIdx.x + 1);
-    }
-    for (;;) {
-        long long col;
-        int z0, z1;
-        if (p.zslab > 0) {
-            if (pc >= p.pieces) break;
-            const long long sl = pc / p.total_cols;
-            col = pc - sl * p.total_cols;
-            z0 = (int)(sl * p.zslab);
-            z1 = min(p.nz, z0 + p.zslab);
-            pc += gridDim.x;
-        } else {
-            if (f >= fend) break;
-            col = f / p.nz;
-            z0 = (int)(f - col * p.nz);
-            z1 = (int)min((long long)p.nz, (long long)z0 + (fend - f));
-            f += z1 - z0;
-        }
-        const int ty = (int)(col / p.ntx), tx = (int)(col - (long long)ty * p.ntx);
+    // (broadcasts, so that the compiler knows the segment's bounds to be uniform across the warp
+    // and keeps them, and what follows from them, in uniform registers)
+    const int si_end = __shfl_sync(0xffffffffu, __ldg(p.seg_first + blockIdx.x + 1), 0);
+    for (int si = __shfl_sync(0xffffffffu, __ldg(p.seg_first + blockIdx.x), 0); si < si_end; si++) {
+        const int4 seg = __ldg(p.segs + si);
+        const int col = __shfl_sync(0xffffffffu, seg.x, 0);
+        const int z0 = __shfl_sync(0xffffffffu, seg.y, 0), z1 = __shfl_sync(0xffffffffu, seg.z, 0);
+        const int ty = col / p.ntx, tx = col - ty * p.ntx;
 
         c.z0 = z0;
         c.z1 = z1;
@@ -611,7 +555,6 @@ __global__ void __launch_bounds__(32 * NW, (TB3F<KIND, T, VX, VY, NW>::MINB))
         const int kyn = (c.gy <= c.ny - 1 && c.ny - 1 < c.gy + VY) ? (c.ny - 1 - c.gy) : -1;
         c.ym0 = ky0 >= 0 ? (1u << ky0) : 0u;
         c.ymn = kyn >= 0 ? (1u << kyn) : 0u;
-        c.edge_x = __any_sync(0xffffffffu, c.lx0 || rxj >= 0);
         c.edge_y = __any_sync(0xffffffffu, ky0 >= 0 || kyn >= 0);
         {
             const int xl = max(c.x0 + C::HX, 0), xh = min(c.x0 + C::HX + C::CX, c.nx);
@@ -627,7 +570,7 @@ __global__ void __launch_bounds__(32 * NW, (TB3F<KIND, T, VX, VY, NW>::MINB))
             c.st_mask = msk;
             constexpr unsigned ALL = (1u << VX) - 1u;
             unsigned rows = 0;
-            bool fast = c.vec != 0;
+            bool fast = p.vec_out != 0;
 #pragma unroll
             for (int k = 0; k < VY; k++) {
                 const unsigned b = (msk >> (VX * k)) & ALL;
@@ -636,126 +579,108 @@ __global__ void __launch_bounds__(32 * NW, (TB3F<KIND, T, VX, VY, NW>::MINB))
             }
             c.st_rows = rows;
             c.st_fast = fast;
-            c.st_off = (long long)c.gy * c.nx + c.gx;
+            c.st_off = (long long)c.gy * c.ld_out + c.gx;
         }
-        const int n_it = z1 + T - c.z_start;
-        const int bot_i = c.nz - c.z_start;
+        const int n_it = z1 + 2 * T - 1 - c.z_start;   // the last stage emits plane z1-1 last
+        const int bot_i = c.nz - 1 - c.z_start;   // stage 0 meets plane nz-1 first
         const bool top = (c.z_start == 0);
         const bool partial = (c.tsteps < T);
 
-        // load plane z into field slot `fs` (and power slot `ps`), on barrier fs when staged
-        // by tensor-map copies (one elected thread), else by per-thread cp.async (one group)
-        auto load = [&](int z, int fs, int ps) {
-            if (z <= c.last_plane) {
-                if (tma) {
-                    if (threadIdx.x == 0) {
-                        const uint32_t bar = sbar + 8u * fs;
-                        mbar_expect_tx(bar, (KIND == KTHERM ? 2u : 1u) * C::PLANE_B);
-                        tma_plane(sring + fs * C::PLANE_B, &tin, c.x0, c.y0, z, bar);
-                        if (KIND == KTHERM) tma_plane(spw + ps * C::PLANE_B, &tpw, c.x0, c.y0, z, bar);
-                    }
-                    pending |= 1u << fs;
-                } else {
-                    tbf3_load<C::BX, C::BY, C::NT>(c, c.in + (long long)z * c.plane, c.vec,
-                                                   sring + fs * C::PLANE_B);
-                    if (KIND == KTHERM)
-                        tbf3_load<C::BX, C::BY, C::NT>(c, c.pw + (long long)z * c.plane,
-                                                       c.vec_pw, spw + ps * C::PLANE_B);
-                }
-            }
-            if (!tma) cp_async_commit();
-        };
-        // on a failed wait: flag it, give the copies in flight a bounded chance to land, leave
-        auto bail = [&]() {
-            if (threadIdx.x == 0) atomicExch(p.err, 1);
-            for (int b = 0; b < C::NBF; b++)
-                if ((pending >> b) & 1u) (void)mbar_wait_bounded(sbar + 8u * b, (phase >> b) & 1u);
-        };
-#pragma unroll 1
-        for (int j = 0; j < C::PF; j++) load(c.z_start + j, j, KIND == KTHERM ? j : 0);
-        Slots3 sl;
-        sl.f0 = 0;
-        sl.p1 = KIND == KTHERM ? C::NBP - 1 : 0;
-        int lf = C::PF, lp = KIND == KTHERM ? C::PF : 0;   // slots the next loads fill
-        // wait for plane z_start + i, then refill the slot last read one iteration ago (plane
-        // z-1 of stage 0; for power, plane z-T+1 of stage T-1) with plane z_start + i + PF
-        auto prologue = [&](int i) -> bool {
-            bool bad = false;
+        // queue plane z into field slot `fs` (and power slot `ps`): by tensor-map copies on
+        // barrier fs (one elected thread), else by per-thread cp.async (one group)
+        auto load = [&](int z, uint32_t fs, uint32_t ps) {
             if (tma) {
-                const int b = sl.f0;
-                if ((pending >> b) & 1u) {
-                    bad = !mbar_wait_bounded(sbar + 8u * b, (phase >> b) & 1u);
-                    phase ^= 1u << b;
-                    pending &= ~(1u << b);
+                if (threadIdx.x == 0 && z <= c.last_plane && !bad) {
+                    const uint32_t bar = sbar + 8u * fs;
+                    mbar_expect_tx(bar, (KIND == KTHERM ? 2u : 1u) * C::PLANE_B);
+                    tma_plane(sring + fs * C::PLANE_B, &tin, c.x0, c.y0, z, bar);
+                    if (KIND == KTHERM) tma_plane(spw + ps * C::PLANE_B, &tpw, c.x0, c.y0, z, bar);
                 }
             } else {
-                cp_async_wait<C::PF - 1>();
-            }
-            if (__syncthreads_or(bad)) return false;
-            // the slot refilled below was read through the generic proxy before the barrier
-            if (tma && threadIdx.x == 0) asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-            load(c.z_start + i + C::PF, lf, lp);
-            return true;
-        };
-        auto advance = [&]() {
-            sl.f0 = sl.f0 + 1 == C::NBF ? 0 : sl.f0 + 1;
-            lf = lf + 1 == C::NBF ? 0 : lf + 1;
-            if (KIND == KTHERM) {
-                sl.p1 = sl.p1 + 1 == C::NBP ? 0 : sl.p1 + 1;
-                lp = lp + 1 == C::NBP ? 0 : lp + 1;
+                if (z <= c.last_plane) {
+                    tbf3_load<C::BX, C::BY, C::NT>(c, c.in + (long long)z * c.plane_in, c.ld_in, c.vec,
+                                                   sring + fs * C::PLANE_B);
+                    if (KIND == KTHERM)
+                        tbf3_load<C::BX, C::BY, C::NT>(c, c.pw + (long long)z * c.plane_pw, c.ld_pw,
+                                                       c.vec_pw, spw + ps * C::PLANE_B);
+                }
+                cp_async_commit();
             }
         };
-        auto special = [&](int i) { return partial || (top && i <= T) || i >= bot_i; };
-        auto copy_back = [&]() {
-#pragma unroll
-            for (int s = 0; s < C::NS; s++)
-#pragma unroll
-                for (int k = 0; k < VY; k++)
-#pragma unroll
-                    for (int j = 0; j < VX; j++) {
-                        PA[s][k][j] = PB[s][k][j];
-                        QA[s][k][j] = QB[s][k][j];
-                    }
+        // the field ring goes on where the previous segment left it (slot f0 with parity fpar
+        // takes this segment's first plane); slots advance with the planes that are loaded
+        {
+            uint32_t fs = f0;
+#pragma unroll 1
+            for (int j = 0; j < C::PF; j++) {
+                load(c.z_start + j, fs, KIND == KTHERM ? j : 0);
+                fs = fs + 1 == C::NBF ? 0 : fs + 1;
+            }
+        }
+        uint32_t p0 = 0;                                         // slot of power plane Z0
+        uint32_t xr = sxch, xw = sxch + (C::XB - 1) * C::XBUF;   // exchange read / written
+        float *dst = c.out + c.st_off + ((long long)c.z_start - (2 * T - 1)) * c.plane_out;
+        if (!tma) cp_async_wait<C::PF - 1>();
+        __syncthreads();
+        // one plane
+        auto step = [&](auto special_tag, auto edge_tag, int i) {
+            const int Z0 = c.z_start + i;
+            // the slot refilled here was last read in the previous iteration, before its barrier
+            load(Z0 + C::PF, f0 == 0 ? C::NBF - 1 : f0 - 1,
+                 KIND == KTHERM ? (p0 + C::PF >= C::NBP ? p0 + C::PF - C::NBP : p0 + C::PF) : 0);
+            const bool in = Z0 <= c.last_plane;
+            if (tma && in && !bad && !mbar_wait_bounded(sbar + 8u * f0, fpar)) {
+                bad = true;   // flag it and carry on: every later wait and copy is skipped
+                atomicExch(p.err, 1);
+            }
+            tbf3_iter<KIND, T, VX, VY, NW, decltype(special_tag)::value, decltype(edge_tag)::value>(
+                c, k, sring + f0 * C::PLANE_B, spw, p0, xr, xw, dst, P, Q, D, Z0);
+            dst += c.plane_out;
+            if (in) {
+                f0++;
+                if (f0 == C::NBF) {
+                    f0 = 0;
+                    fpar ^= 1u;
+                }
+            }
+            if (KIND == KTHERM) p0 = p0 + 1 == C::NBP ? 0 : p0 + 1;
+            const uint32_t t = xr;
+            xr = xw;
+            xw = t;
+            if (!tma) cp_async_wait<C::PF - 1>();   // (plane Z0 + 1, made visible by the barrier)
+            __syncthreads();
         };
-        // The partial sums alternate between two register sets (A -> B, then B -> A) so that
-        // no iteration copies them; the rare special iterations run A -> B and copy back.
-        // Tile columns away from the x and y domain edges run an instance without the clamp
-        // fix-ups: their in-place updates of the plane otherwise cost register copies on every
-        // path.  Returns false when a wait gave up.
-        auto run = [&](auto edge_tag) -> bool {
-            constexpr bool EDGE = decltype(edge_tag)::value;
+        // the planes that need z-boundary handling (the first and last of the grid, and all of a
+        // pass that forwards trailing stages) run in loops of their own: a loop that chose per
+        // plane would have to merge the partial sums of both bodies, with register copies, in
+        // every iteration
+        const int i_a = partial ? n_it : (top ? min(2 * T - 1, n_it) : 0);
+        const int i_b = partial ? n_it : max(i_a, min(n_it, bot_i));
+        // A tile column runs the instance that handles the edges it touches (interior ones none):
+        // the fix-ups' in-place updates of the plane otherwise cost register copies on every path.
+        auto run = [&](auto edge_tag) {
             int i = 0;
 #pragma unroll 1
-            while (i < n_it) {
-                if (!prologue(i)) return false;
-                if (special(i)) {
-                    tbf3_iter<KIND, T, VX, VY, NW, true, EDGE>(c, sring, spw, sxch, sl, PA, QA, PB, QB, i);
-                    advance();
-                    copy_back();
-                    ++i;
-                    continue;
-                }
-                tbf3_iter<KIND, T, VX, VY, NW, false, EDGE>(c, sring, spw, sxch, sl, PA, QA, PB, QB, i);
-                advance();
-                ++i;
-                if (i < n_it && !special(i)) {
-                    if (!prologue(i)) return false;
-                    tbf3_iter<KIND, T, VX, VY, NW, false, EDGE>(c, sring, spw, sxch, sl, PB, QB, PA, QA, i);
-                    advance();
-                    ++i;
-                } else {
-                    copy_back();
-                }
-            }
-            return true;
+            for (; i < i_a; i++) step(std::true_type{}, edge_tag, i);
+#pragma unroll 1
+            for (; i < i_b; i++) step(std::false_type{}, edge_tag, i);
+#pragma unroll 1
+            for (; i < n_it; i++) step(std::true_type{}, edge_tag, i);
         };
-        const bool edge = __syncthreads_or(c.edge_x || c.edge_y) != 0;
-        if (!(edge ? run(std::true_type{}) : run(std::false_type{}))) {
-            bail();
+        const int touch = (c.x0 <= 0 || c.x0 + C::BX >= c.nx ? E3X : 0) |
+                          (c.y0 <= 0 || c.y0 + C::BY >= c.ny ? E3Y : 0);   // block-uniform
+        if (touch == 0) run(std::integral_constant<int, 0>{});
+        else if (touch == E3Y) run(std::integral_constant<int, E3Y>{});
+        else run(std::integral_constant<int, E3X | E3Y>{});
+        if (!tma) cp_async_wait<0>();
+        if (__syncthreads_or(bad)) {
+            // give whatever may still be in flight a bounded chance to land, then leave
+            for (int b = 0; b < C::NBF; b++) {
+                (void)mbar_wait_bounded(sbar + 8u * b, 0);
+                (void)mbar_wait_bounded(sbar + 8u * b, 1);
+            }
             return;
         }
-        if (!tma) cp_async_wait<0>();
-        __syncthreads();
     }
 }
 

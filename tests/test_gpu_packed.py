@@ -40,3 +40,22 @@ def test_widths_16bit(eng, orc, kind, storage):  # noqa: F811
         plan.close()
         o = orc.run(kind, w.u0, w.coef, 19, w.power, dtype=np.float64)
         assert np.linalg.norm(g - o) <= 1e-2 * np.linalg.norm(o), nx
+
+
+# 3D segments (which planes of which tile columns a block streams): fewer columns than blocks with
+# long and short z, about as many, more columns than blocks, one plane, one column; odd widths
+# run between padded scratch grids
+SHAPES_SEG = [(60, 50, 301), (131, 127, 61), (187, 141, 33), (400, 300, 9), (733, 700, 5), (300, 200, 1),
+              (9, 7, 130), (1300, 61, 11)]
+
+
+@pytest.mark.parametrize("kind", [0, 1])
+@pytest.mark.parametrize("T,by", [(3, 64), (2, 32)])
+def test_segments_3d(eng, orc, kind, T, by):  # noqa: F811
+    for n, (nx, ny, nz) in enumerate(SHAPES_SEG):
+        w = synth.make(kind, 3, nx, ny, nz, seed=8500 + 7 * n + kind)
+        steps = T if n % 2 else 2 * T + 1
+        g, info = gpu_run(eng, w, steps, T=T, vec=8, bx=64, by=by)
+        assert (info["T"], info["by"]) == (T, by)
+        o = orc.run(kind, w.u0, w.coef, steps, w.power)
+        assert max_rel(g, o) <= TOL, (nx, ny, nz, steps, max_rel(g, o))
