@@ -26,68 +26,10 @@ struct PassCfg2D {
     int ntx = 0;
     long long total = 0, rows_per_cta = 0;
     int ctas = 0;
-    long long *starts = nullptr;   // device: cost-balanced ranges (contracted kernel), or none
+    int seg_off = 0;        // ints before the segments
+    void *segs = nullptr;   // contracted kernel, device: [first segment of each block | segments]
     bool ready = false;
 };
-
-// Ranges of (tile column, row or plane) units, one per block, balanced by cost rather than by
-// count: a segment streams 2T rows (planes) of pipeline fill besides its own (Sec. 3.2), so a
-// block whose range crosses a tile column pays the fill twice, and a unit of an edge tile column
-// costs more (its warps run the clamp selects): w[col] per unit.  The slowest block sets the
-// pass time.  Greedy cut at the mean cost.  Returns the ranges' largest cost and fills starts
-// (ctas + 1 entries).
-double balanced_ranges(long long len, int ctas, int fill, const std::vector<double> &w,
-                       std::vector<long long> &st)
-{
-    const long long ncol = (long long)w.size(), total = ncol * len;
-    double weighted = 0.0;
-    for (double x : w) weighted += x * len;
-    const double target = (weighted + (double)fill * (ctas + ncol - 1)) / ctas;
-    st.assign(ctas + 1, total);
-    long long u = 0;
-    for (int b = 0; b < ctas; b++) {
-        st[b] = u;
-        double cost = 0.0;
-        while (u < total) {
-            const long long col = u / len, col_end = (col + 1) * len;
-            const double room = target - cost - fill;
-            if (room < w[col] && cost > 0.0) break;
-            const long long take = std::min<long long>(col_end - u, std::max<long long>(1, (long long)std::ceil(room / w[col])));
-            cost += fill + w[col] * (double)take;
-            u += take;
-            if (cost >= target) break;
-        }
-    }
-    double worst = 0.0;
-    for (int b = 0; b < ctas; b++) {   // the last block also takes whatever is left
-        double c = 0.0;
-        for (long long x = st[b]; x < st[b + 1];) {
-            const long long e = std::min(st[b + 1], (x / len + 1) * len);
-            c += fill + w[x / len] * (double)(e - x);
-            x = e;
-        }
-        worst = std::max(worst, c);
-    }
-    return worst;
-}
-
-// the largest cost of ranges of `per` units each (same costs)
-double even_ranges_cost(long long len, long long per, int fill, const std::vector<double> &w)
-{
-    const long long total = (long long)w.size() * len;
-    double worst = 0.0;
-    for (long long a = 0; a < total; a += per) {
-        const long long e = std::min(total, a + per);
-        double c = 0.0;
-        for (long long x = a; x < e;) {
-            const long long f = std::min(e, (x / len + 1) * len);
-            c += fill + w[x / len] * (double)(f - x);
-            x = f;
-        }
-        worst = std::max(worst, c);
-    }
-    return worst;
-}
 
 struct PassCfg3D {
     Shape3D shape;
@@ -189,37 +131,47 @@ bool available(const stencil_plan_s *p, int T)
 
 // ---- parameter choice seeded by the GPU restatement of the paper's model (Eqs. 3-9) -------
 //
-// Calibration (GB300 ncu counts of the contracted 2D kernels): each stage issues its Table 2
-// operations (5 Diffusion, 9 Hotspot per cell) plus ~4 per thread (2 shuffles, power loads,
-// addressing), each row ~100 more per thread (waits, copies, ring and pointer updates); issue
-// efficiency grows with resident warps (0.69 at 8, 0.77 at 12 per SM); a hot loop beyond ~12 KB
-// of code loses issue rate in proportion (instruction-cache misses); these kernels reach ~62 %
-// of the measured copy bandwidth when they are memory-bound; every row segment streams 2T rows
-// more than it stores, which dominates on small grids cut into many short segments.  With these factors the model
-// ranks the compiled variants as measured on 16384^2 grids at T in {4, 6, 8, 12}.
+// Calibration of the contracted 2D kernels (GB300): a pass takes a * (cell steps computed, fill
+// included) / (SMs * 128 lanes * clock) + b, per compiled (kind, T, V, variant) with a in cycles
+// per lane and cell step and b what a pass costs besides (launch, first rows, drain: the fewer
+// warps share a scheduler the more).  Fitted on 16384^2 and 3000 x 2000; within 5 % on 8000^2 and
+// 4096^2, 10 % on 1600^2, 25 % on 1000 x 600.
+struct Cal2D { int kind, T, V, W; double a, b_us; };
+const Cal2D kCal2D[] = {
+    {0, 4, 4, 1, 12.6, 6.6},  {0, 8, 4, 1, 10.2, 6.5},  {0, 12, 4, 1, 9.8, 13.1}, {0, 4, 8, 1, 12.0, 6.4},
+    {0, 6, 8, 1, 10.5, 9.1},  {0, 8, 8, 1, 8.4, 16.5},  {0, 8, 8, 0, 9.5, 8.9},   {0, 12, 4, 0, 9.9, 8.8},
+    {1, 4, 4, 1, 22.4, 2.0},  {1, 8, 4, 1, 12.2, 9.4},  {1, 12, 4, 1, 11.7, 18.9}, {1, 4, 8, 1, 20.0, 5.4},
+    {1, 6, 8, 1, 13.5, 12.4}, {1, 8, 8, 1, 11.5, 24.7}, {1, 8, 8, 0, 11.9, 11.4}, {1, 12, 4, 0, 12.3, 12.8},
+};
+
 struct Cand2D { int T, V, W; };
+
+// 2D: rows of fill a segment costs, per fused step (2T rows with the idle stages skipped)
+constexpr double kFill2 = 1.25;
+// 2D: relative cost of a row of an edge tile column (see segments_2d)
+constexpr double kEdge2 = 1.05, kGhost2 = 1.45;
+// 2D: how far the oldest (youngest) block of a scheduler is ahead (behind): see segments_2d
+constexpr double kAhead2 = 0.04;
+// 2D: rows a segment that starts or ends at the grid's top or bottom costs besides, per fused step
+// (8 and 4 cells per thread)
+constexpr double kTop2V8 = 3.0, kTop2V4 = 1.5;
 
 // seg_rows = 0: the plan's own launch geometry; > 0: a batch launch, whose segments hold about
 // seg_rows rows across all its grids and whose launch cost the grids share
 double model_gcells_2d(const stencil_desc &d, int sms, const Cand2D &k, int bps, int steps,
                        int seg_rows = 0)
 {
-    const bool swap = k.W == 1;
-    const double fp = d.kind == ST_DIFFUSION ? 5.0 : 6.0;   // Hotspot: the expanded weights
-    const double ops = fp + 4.0 / k.V + 100.0 / (k.T * k.V);
-    const double code_kb = (swap ? 2.0 : 1.0) * k.T * (k.V * fp + 6.0) * 16.0 / 1024.0;
-    // the launch geometry of prepare2: one-warp blocks over (tile column, row) units in
-    // segments of at least 4 rows; each segment streams 2T extra rows (Sec. 3.2's pipeline
-    // fill and drain), and a small grid leaves SMs with fewer resident warps
+    double ops = 14.0 + 32.0 / k.T, fixed = 8e-6;   // forced (T, V) without a calibration
+    for (const Cal2D &c : kCal2D)
+        if (c.kind == d.kind && c.T == k.T && c.V == k.V && c.W == k.W) {
+            ops = c.a;
+            fixed = c.b_us * 1e-6;
+        }
+    // one-warp blocks, as many as are resident, over the rows of every tile column
     const int halo = (k.T + k.V - 1) / k.V * k.V;   // tb2d_halo
     const long long cx = 32LL * k.V - 2 * halo;
-    const long long units = (d.nx + cx - 1) / cx * (long long)d.ny;
-    const long long ctas = std::min<long long>((long long)sms * bps, std::max<long long>(1, units / 4));
-    const double rows_per_cta = seg_rows > 0 ? seg_rows : (double)units / ctas;
-    const int warps = seg_rows > 0 ? std::min(bps, 16)
-                                   : (int)std::min<long long>(std::min(bps, 16), (ctas + sms - 1) / sms);
-    double eff = std::min(0.85, 0.45 + 0.027 * warps);
-    if (code_kb > 12.0) eff *= 12.0 / code_kb;
+    const double units = (double)((d.nx + cx - 1) / cx) * d.ny;
+    const double rows = seg_rows > 0 ? seg_rows : std::max(1.0, units / ((double)sms * bps));
     stencil_gpu_model_in m = {};
     m.ndim = 2;
     m.nx = d.nx;
@@ -234,10 +186,10 @@ double model_gcells_2d(const stencil_desc &d, int sms, const Cand2D &k, int bps,
     m.hbm_gbs = 6800.0;
     m.bytes_per_cell = d.kind == ST_DIFFUSION ? 8.0 : 12.0;
     m.ops_per_cell = ops;
-    m.issue_eff = eff;
-    m.hbm_eff = 0.62;
-    m.stream_overhead = 2.0 * k.T / rows_per_cta;
-    m.launch_s = seg_rows > 0 ? 0.0 : 4e-6;
+    m.issue_eff = 1.0;
+    m.hbm_eff = 0.90;
+    m.stream_overhead = kFill2 * k.T / rows;
+    m.launch_s = seg_rows > 0 ? 0.0 : fixed;
     stencil_gpu_model_out r;
     if (stencil_model_gpu(&m, &r) != ST_OK) return 0.0;
     return r.gcells;
@@ -251,8 +203,10 @@ double model_gcells_2d(const stencil_desc &d, int sms, const Cand2D &k, int bps,
 // with the columns streamed in step most halo re-reads hit L2: three tenths of the tile fit's
 // excess reads, at 90 % of the copy bandwidth.  Calibrated on GB300 over 512^3, 512^2 x 256,
 // 256^3, 300 x 200 x 400 and 187 x 141 x 93, both kinds, T = 2 .. 4, 64- and 32-row tiles.
-// 3D segments (tb3f): which planes of which tile columns each block streams.  A segment costs
-// w[col] per plane plus `fill` planes of pipeline fill, and the slowest block sets the pass time.
+// Segments of the contracted passes: which planes (2D: rows) of which tile columns each block
+// streams.  A segment costs w[col] per plane plus `fill` planes of pipeline fill, plus `edge` at
+// the first and the last plane of the grid (boundary handling), and the slowest block sets the
+// pass time.
 // The tile columns overlap, so neighbouring columns should be at nearby planes at the same time:
 // then the halo cells a tile reads again (and the partial sectors of its rows) are still in L2.
 // So, level by level: with at least as many blocks as columns left, every column gets one block,
@@ -261,10 +215,12 @@ double model_gcells_2d(const stencil_desc &d, int sms, const Cand2D &k, int bps,
 // whole rest of a column, the costliest first, and goes on with the budget that leaves it.  The
 // budget is the smallest for which everything is dealt out (bisection).
 // Measured on GB300 against contiguous ranges of (column, plane) units balanced the same way,
-// where neighbours run at unrelated planes: see prepare3.
+// where neighbours run at unrelated planes: see prepare3 and segments_2d.
 struct Seg3 { int col, z0, z1, pad; };
 
-bool deal_segments(int nz, int slots, double fill, const std::vector<double> &w, double budget,
+// speed: each block's share of the budget (empty: all alike)
+bool deal_segments(int nz, int slots, double fill, double edge, const std::vector<double> &w,
+                   const std::vector<double> &speed, double budget,
                    std::vector<std::vector<Seg3>> *out)
 {
     struct Rest { int col, z0; };
@@ -274,7 +230,7 @@ bool deal_segments(int nz, int slots, double fill, const std::vector<double> &w,
     // blocks with work to take, the largest budget first, from `head` on; `spare`: those that have
     // a segment and budget left, taken up when the others have run out
     std::vector<Block> blocks(slots), spare;
-    for (int b = 0; b < slots; b++) blocks[b] = Block{budget, b};
+    for (int b = 0; b < slots; b++) blocks[b] = Block{speed.empty() ? budget : budget * speed[b], b};
     size_t head = 0;
     if (out) out->assign(slots, {});
     while (!rest.empty()) {
@@ -303,12 +259,16 @@ bool deal_segments(int nz, int slots, double fill, const std::vector<double> &w,
             }
             Block &b = blocks[head + i];
             const int h = nz - q.z0;
-            const int take = std::max(1, (int)std::min<double>(h, std::floor((b.left - fill) / w[q.col])));
+            const double fixed = fill + (q.z0 == 0 ? edge : 0.0);
+            int take = std::max(1, (int)std::min<double>(h, std::floor((b.left - fixed) / w[q.col])));
+            // a segment that reaches the end pays `edge` too; one that cannot, leaves a rest
+            if (take == h && take > 1 && fixed + edge + h * w[q.col] > b.left)
+                take = std::max(1, std::min(h - 1, (int)std::floor((b.left - fixed - edge) / w[q.col])));
             if (out) (*out)[b.id].push_back(Seg3{q.col, q.z0, q.z0 + take, 0});
             if (take < h) {
                 next.push_back(Rest{q.col, q.z0 + take});
             } else {
-                b.left -= fill + take * w[q.col];
+                b.left -= fixed + edge + take * w[q.col];
                 if (b.left >= fill + 4) spare.push_back(b);
             }
         }
@@ -322,19 +282,20 @@ bool deal_segments(int nz, int slots, double fill, const std::vector<double> &w,
 
 // The smallest budget for `slots` blocks (within tol), and with out != nullptr the segments per
 // block.
-double best_segments(int nz, int slots, double fill, const std::vector<double> &w, double tol,
+double best_segments(int nz, int slots, double fill, double edge, const std::vector<double> &w,
+                     const std::vector<double> &speed, double tol,
                      std::vector<std::vector<Seg3>> *out)
 {
     double total = 0.0;
     for (double x : w) total += x * nz;
-    double lo = total / slots, hi = lo + 3.0 * fill;
-    while (!deal_segments(nz, slots, fill, w, hi, nullptr)) hi *= 1.5;
+    double lo = std::max(total / slots, fill + 4.0), hi = lo + 3.0 * fill + edge;
+    while (!deal_segments(nz, slots, fill, edge, w, speed, hi, nullptr)) hi *= 1.5;
     for (int i = 0; i < 40 && hi - lo > tol; i++) {
         const double mid = 0.5 * (lo + hi);
-        if (deal_segments(nz, slots, fill, w, mid, nullptr)) hi = mid;
+        if (deal_segments(nz, slots, fill, edge, w, speed, mid, nullptr)) hi = mid;
         else lo = mid;
     }
-    if (out) deal_segments(nz, slots, fill, w, hi, out);
+    if (out) deal_segments(nz, slots, fill, edge, w, speed, hi, out);
     return hi;
 }
 
@@ -379,8 +340,8 @@ double model_gcells_3d(const stencil_desc &d, int sms, int T, int VX, int VY, in
     const long long slots = (long long)sms * (NW <= 8 ? 2 : 1);
     const double seg_cost =
         bound ? 0.0
-              : best_segments(d.nz, (int)slots, 3.0 * T - 1,
-                              column_weights((int)std::ceil(d.nx / cx), (int)std::ceil(d.ny / cy)),
+              : best_segments(d.nz, (int)slots, 3.0 * T - 1, 0.0,
+                              column_weights((int)std::ceil(d.nx / cx), (int)std::ceil(d.ny / cy)), {},
                               0.02 * cols * d.nz / slots + 0.5, nullptr);
     const double alg = d.kind == ST_DIFFUSION ? 8.0 : 12.0;
     const double read = alg - 4.0;   // field (and power) in; the field out is written once
@@ -538,6 +499,54 @@ int kernel_T_for(const stencil_plan_s *p, int want)
     return best;
 }
 
+// Dealt segments on the device, [first segment of each block | segments], and their block count.
+int upload_segments(std::vector<std::vector<Seg3>> &segs, int *ctas, int *seg_off, void **dev)
+{
+    while (segs.size() > 1 && segs.back().empty()) segs.pop_back();
+    *ctas = (int)segs.size();
+    std::vector<int> host((segs.size() + 1 + 3) / 4 * 4, 0);   // (the segments start 16-byte aligned)
+    *seg_off = (int)host.size();
+    for (size_t i = 0; i < segs.size(); i++) host[i + 1] = host[i] + (int)segs[i].size();
+    for (const auto &v : segs)
+        for (const Seg3 &q : v) host.insert(host.end(), {q.col, q.z0, q.z1, 0});
+    cudaError_t e = stn::dev_malloc(dev, host.size() * sizeof(int));
+    if (e == cudaSuccess) e = cudaMemcpy(*dev, host.data(), host.size() * sizeof(int), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+        if (*dev) stn::dev_free(*dev);
+        *dev = nullptr;
+    }
+    return map_cuda(e);
+}
+
+// Segments of a contracted 2D pass: rows of tile columns dealt like the planes of the 3D passes
+// (best_segments), so that neighbouring columns stream the same rows at the same time and share
+// their halo cells, and the partial sectors of their rows, in L2.  A segment's fill is 2T rows of
+// which the idle stages are skipped.  A row of a tile column whose edge lies on a lane boundary
+// (x = 0 always, x = nx-1 when nx is a multiple of the cells per thread) costs kEdge2, one whose
+// last column lies inside a lane kGhost2 (its warps run a clamp select per cell), and a segment
+// that starts at the top or ends at the bottom kTop2 T rows more (special rows run a loop with
+// boundary tests).  Measured on GB300 against contiguous ranges balanced the same way: 12000^2
+// diffusion 4001 -> 4184 GCell/s, 16384^2 4114 -> 4247, Hotspot 3058 -> 3107, 8192^2 Hotspot 2645
+// -> 2761 (T = 8, 8 cells per thread); DRAM reads of a 16384^2 diffusion pass 1.31 -> 1.10 GB.
+int segments_2d(stencil_plan_s *p, int bps, PassCfg2D *c)
+{
+    std::vector<double> w(c->ntx, 1.0);
+    w.front() = kEdge2;
+    w.back() = p->d.nx % c->shape.V == 0 ? kEdge2 : kGhost2;
+    std::vector<std::vector<Seg3>> segs;
+    // A scheduler issues from its oldest ready warp first, so of the one-warp blocks that share one
+    // the first to arrive (blocks arrive in order, one per SM and round, four rounds per warp
+    // rank) runs ahead of the others (equal shares, 12000^2 diffusion: the first half of the
+    // blocks took 204 us, the second 265; ahead by 0 / 0.05 / 0.1 / 0.15, 16384^2 diffusion:
+    // 4071 / 4160 / 3986 / 3814 GCell/s)
+    const int slots = p->sms * bps, ranks = (bps + 3) / 4;
+    std::vector<double> speed(slots, 1.0);
+    for (int b = 0; b < slots && ranks > 1; b++)
+        speed[b] = 1.0 + kAhead2 * (1.0 - 2.0 * (b / p->sms / 4) / (ranks - 1));
+    best_segments(p->d.ny, slots, kFill2 * c->shape.T, (c->shape.V == 8 ? kTop2V8 : kTop2V4) * c->shape.T, w, speed, 0.5, &segs);
+    return upload_segments(segs, &c->ctas, &c->seg_off, &c->segs);
+}
+
 int prepare2(stencil_plan_s *p, int Tk, PassCfg2D **out)
 {
     if ((int)p->cfg2.size() <= Tk) p->cfg2.resize(Tk + 1);
@@ -560,26 +569,8 @@ int prepare2(stencil_plan_s *p, int Tk, PassCfg2D **out)
         c.rows_per_cta = (c.total + ctas - 1) / ctas;
         c.ctas = (int)((c.total + c.rows_per_cta - 1) / c.rows_per_cta);
         if (!c.shape.exact && c.shape.kind != ST_DIFFUSION_VAR) {
-            // contracted kernel: cost-balanced ranges where they shorten the longest block
-            std::vector<long long> st;
-            const int fill = 2 * Tk;
-            // a row of an edge tile column costs 1.25: its warps run the clamp selects
-            // (measured on GB300 with the edge weight swept 1.0-1.4: 16384^2 Hotspot 2684 ->
-            // 2948 GCell/s, diffusion 3337 -> 3753, flat between 1.2 and 1.4)
-            std::vector<double> w(c.ntx, 1.0);
-            w.front() = w.back() = 1.25;
-            if (balanced_ranges(p->d.ny, (int)ctas, fill, w, st) <
-                even_ranges_cost(p->d.ny, c.rows_per_cta, fill, w)) {
-                e = stn::dev_malloc(&c.starts, st.size() * sizeof(long long));
-                if (e == cudaSuccess)
-                    e = cudaMemcpy(c.starts, st.data(), st.size() * sizeof(long long), cudaMemcpyHostToDevice);
-                if (e != cudaSuccess) {
-                    if (c.starts) stn::dev_free(c.starts);
-                    c.starts = nullptr;
-                    return map_cuda(e);
-                }
-                c.ctas = (int)ctas;
-            }
+            const int rc = segments_2d(p, bps, &c);
+            if (rc != ST_OK) return rc;
         }
         c.ready = true;
     }
@@ -605,10 +596,8 @@ int prepare_traj(stencil_plan_s *p, PassCfg2D **out)
         const int cx = tb2d_tile_width(c.shape) - 2 * tb2d_halo(c.shape);
         c.ntx = (p->d.nx + cx - 1) / cx;
         c.total = (long long)c.ntx * p->d.ny;
-        const long long ctas = std::min<long long>((long long)p->sms * bps,
-                                                   std::max<long long>(1, c.total / 4));
-        c.rows_per_cta = (c.total + ctas - 1) / ctas;
-        c.ctas = (int)((c.total + c.rows_per_cta - 1) / c.rows_per_cta);
+        const int rc = segments_2d(p, bps, &c);
+        if (rc != ST_OK) return rc;
         c.ready = true;
     }
     *out = &c;
@@ -648,26 +637,9 @@ int prepare3(stencil_plan_s *p, int Tk, PassCfg3D **out)
             // (187 x 141 x 93 diffusion x 30: 427 -> 242 us)
             const std::vector<double> w = column_weights(c.ntx, c.nty);
             std::vector<std::vector<Seg3>> segs;
-            best_segments(p->d.nz, p->sms * bps, 3.0 * Tk - 1, w, 0.25, &segs);
-            while (segs.size() > 1 && segs.back().empty()) segs.pop_back();
-            c.ctas = (int)segs.size();
-            std::vector<int> host(((size_t)c.ctas + 1 + 3) / 4 * 4, 0);   // first[], 16-byte aligned end
-            c.seg_off = (int)host.size();
-            for (int i = 0, n = 0; i < c.ctas; i++) {
-                host[i] = n;
-                n += (int)segs[i].size();
-                host[i + 1] = n;
-            }
-            for (const auto &v : segs)
-                for (const Seg3 &q : v) host.insert(host.end(), {q.col, q.z0, q.z1, 0});
-            e = stn::dev_malloc(&c.segs, host.size() * sizeof(int));
-            if (e == cudaSuccess)
-                e = cudaMemcpy(c.segs, host.data(), host.size() * sizeof(int), cudaMemcpyHostToDevice);
-            if (e != cudaSuccess) {
-                if (c.segs) stn::dev_free(c.segs);
-                c.segs = nullptr;
-                return map_cuda(e);
-            }
+            best_segments(p->d.nz, p->sms * bps, 3.0 * Tk - 1, 0.0, w, {}, 0.25, &segs);
+            const int rc = upload_segments(segs, &c.ctas, &c.seg_off, &c.segs);
+            if (rc != ST_OK) return rc;
         }
         c.ready = true;
     }
@@ -767,7 +739,8 @@ int run_pass2(stencil_plan_s *p, const float *src, long long lds, float *dst, lo
     a.ntx = c->ntx;
     a.total_rows = c->total;
     a.rows_per_cta = c->rows_per_cta;
-    a.starts = c->starts;
+    a.seg_first = static_cast<const int *>(c->segs);
+    a.segs = c->segs ? reinterpret_cast<const int4 *>(a.seg_first + c->seg_off) : nullptr;
     a.ctas = c->ctas;
     for (int i = 0; i < 5; i++) a.k[i] = a.kf[i] = k[i];
     a.kf[5] = k[0] * k[2];    // Hotspot: sdc * Ry, rounded once (float32)
@@ -876,7 +849,8 @@ int run_pass2q(stencil_plan_s *p, int src, int dst, const float *k, int tsteps)
     a.ntx = c->ntx;
     a.total_rows = c->total;
     a.rows_per_cta = c->rows_per_cta;
-    a.starts = c->starts;
+    a.seg_first = static_cast<const int *>(c->segs);
+    a.segs = c->segs ? reinterpret_cast<const int4 *>(a.seg_first + c->seg_off) : nullptr;
     a.ctas = c->ctas;
     for (int i = 0; i < 5; i++) a.k[i] = a.kf[i] = k[i];
     a.kf[5] = k[0] * k[2];
@@ -1699,7 +1673,8 @@ int stencil_plan_destroy(stencil_plan p)
     if (p->res_xg) stn::dev_free(p->res_xg);
     if (p->res_flags) stn::dev_free(p->res_flags);
     for (PassCfg2D &c : p->cfg2)
-        if (c.starts) stn::dev_free(c.starts);
+        if (c.segs) stn::dev_free(c.segs);
+    if (p->traj.segs) stn::dev_free(p->traj.segs);
     for (PassCfg3D &c : p->cfg3)
         if (c.segs) stn::dev_free(c.segs);
     delete p;

@@ -20,8 +20,10 @@ struct Pass2D {
     int ntx;               // tiles along x
     long long total_rows;  // ntx * ny: the (tile column, row) pairs of the pass
     long long rows_per_cta;
-    const long long *starts;   // contracted kernel: block b takes pairs [starts[b], starts[b+1])
-                               // (nullptr: rows_per_cta pairs each)
+    // contracted kernel: block b streams segments seg_first[b] .. seg_first[b+1]-1, each (tile
+    // column, first row, end row, 0); nullptr: rows_per_cta pairs each
+    const int *seg_first;
+    const int4 *segs;
     int ctas;
     float k[5];
     // contracted kernel's coefficients, derived on the host from k: diffusion cc, cw, ce, cs, cn;

@@ -35,8 +35,9 @@
 // source map, read again by every stage, is stored in pair order (src_pos), so that a 16-byte
 // load yields two pairs.  Stage 0 keeps partial rows like the others: it reads one ring row per
 // iteration (the direct form read three, and would have to pair each).
-// Measured (GB300), before -> after: 16384^2 Hotspot 2928 -> 3045 GCell/s, diffusion 3753 ->
-// 4132, 8192^2 Hotspot with bf16 storage 2032 -> 2430, 3001 x 2003 Hotspot 1053 -> 1248.
+// Measured (GB300), scalar kernel on even ranges -> this one on dealt segments: 16384^2 Hotspot
+// 2928 -> 3118 GCell/s, diffusion 3753 -> 4244, 8192^2 Hotspot with bf16 storage 2032 -> 2630,
+// 3001 x 2003 Hotspot 1053 -> 1466, 3000 x 2000 diffusion 1900.
 // What bounds it now (ncu, 6144^2): Hotspot FMA pipe 58 % busy, issue 57 %, shared memory 64 %
 // (every stage reads its source row), two warps per scheduler; diffusion 58 / 52 / 30 %.
 //
@@ -50,6 +51,8 @@
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
+
+#include <type_traits>
 
 #include "tb2d_kernel.cuh"
 
@@ -204,7 +207,8 @@ struct CtxF {
     int y_start, last_row, s0, s1;
     unsigned lmask, rmask;
     int st_lo, st_hi;
-    bool st_full, st_any, edge;
+    bool st_full, st_any;
+    int edge;              // clamped x edges of my tile: 0 none, 1 lane-aligned ones, 2 any
     int vec_in, vec_out, vec_pw;
     int lane;
     uint32_t oq[2];        // byte offsets in a ring row of my cells' 16-byte chunks
@@ -258,12 +262,14 @@ __device__ __forceinline__ float cell(const float2 (&v)[H], int j)
 // x = nx-1 the ghost cell to its right takes the edge cell's value (a ghost's own value is
 // never used), or e_in when the edge is the lane's last cell; x = 0 is always a lane's cell 0
 // (tile origins are multiples of V), whose west value is its own.
-template <int V>
+// GHOST = false: for warps whose only edges are x = 0 and an x = nx-1 on a lane's last cell.
+template <int V, bool GHOST>
 __device__ __forceinline__ void edge_fix(const CtxF &c, float2 (&d)[V / 2], float &w_in, float &e_in)
 {
     constexpr int H = V / 2;
     e_in = ((c.rmask >> (V - 1)) & 1u) ? d[H - 1].y : e_in;
     w_in = (c.lmask & 1u) ? d[0].x : w_in;
+    if (!GHOST) return;
 #pragma unroll
     for (int j = V - 2; j >= 0; j--) {
         const bool g = (c.rmask >> j) & 1u;
@@ -325,7 +331,7 @@ __device__ __forceinline__ void stf(const CtxF &c, const CoefF &k, int y, bool f
     // pairs take a value from the neighbour lane and one across the halves
     float w_in = __shfl_sync(0xffffffffu, d[H - 1].y, (c.lane + 31) & 31);
     float e_in = __shfl_sync(0xffffffffu, d[0].x, (c.lane + 1) & 31);
-    if (ED) edge_fix<V>(c, d, w_in, e_in);
+    if (ED) edge_fix<V, MODE != MODE_EDGE>(c, d, w_in, e_in);
     float2(&Pn)[H] = SWAP ? Xq : Xp;   // where row y's P goes
     float2(&Qn)[H] = SWAP ? Xp : Xq;   // where row y+1's Q goes
 #pragma unroll
@@ -430,6 +436,10 @@ __device__ __forceinline__ void tbf_iter(const CtxF &c, const CoefF &k,
     float2 d[V / 2];
 #pragma unroll
     for (int s = 0; s < T; s++) {
+        // pipeline fill of a segment that starts inside the grid: stage s gets its first valid
+        // row at i = 2s (row y_start + s), before that it and the stages behind it have nothing
+        // to do
+        if (MODE == MODE_HEAD && i < 2 * s) break;
 #pragma unroll
         for (int j = 0; j < V / 2; j++) d[j] = out[j];
         stf<KIND, V, MODE, SWAP, STOR>(c, k, R0 - s, s >= c.tsteps, PH == 0 ? A[s] : B[s],
@@ -636,10 +646,9 @@ __device__ __forceinline__ void tbf_step_rt(const CtxF &c, const CoefF &k,
     else tbf_step<KIND, T, V, MODE, 0, SWAP, STOR>(c, k, A, B, i, r);
 }
 
-// Work units [f, fend) of one grid's pass: unit f = (tile column f / ny, row f % ny); a block
-// walks them as segments of consecutive rows of one tile column.
+// Rows [s0, s1) of tile column tx of one grid's pass.
 template <int KIND, int T, int V, bool SWAP, int STOR>
-__device__ __forceinline__ void tbf_range(const Pass2D &p, long long f, const long long fend,
+__device__ __forceinline__ void tbf_segment(const Pass2D &p, const int tx, const int s0, const int s1,
                                           float2 (&A)[TB2F<KIND, T, V>::NS][V / 2],
                                           float2 (&B)[TB2F<KIND, T, V>::NS][V / 2], float *smem)
 {
@@ -687,12 +696,7 @@ __device__ __forceinline__ void tbf_range(const Pass2D &p, long long f, const lo
     c.st_states = p.states;
     c.st_stride = p.state_stride;
 
-    while (f < fend) {
-        const int tx = (int)(f / p.ny);
-        const int s0 = (int)(f - (long long)tx * p.ny);
-        const int s1 = (int)min((long long)p.ny, (long long)s0 + (fend - f));
-        f += s1 - s0;
-
+    {
         c.s0 = s0;
         c.s1 = s1;
         c.x0 = tx * C::CX - C::H;
@@ -704,7 +708,8 @@ __device__ __forceinline__ void tbf_range(const Pass2D &p, long long f, const lo
             const int rcl = (c.xt <= c.nx - 1 && c.nx - 1 < c.xt + V) ? (c.nx - 1 - c.xt) : -1;
             c.lmask = lcl >= 0 ? (1u << lcl) : 0u;
             c.rmask = rcl >= 0 ? (1u << rcl) : 0u;
-            c.edge = __any_sync(0xffffffffu, lcl >= 0 || rcl >= 0);
+            c.edge = __any_sync(0xffffffffu, rcl >= 0 && rcl < V - 1) ? 2
+                     : __any_sync(0xffffffffu, lcl >= 0 || rcl >= 0) ? 1 : 0;
         }
         {
             const int lo = max(c.x0 + C::H, 0), hi = min(c.x0 + C::H + C::CX, c.nx);
@@ -760,6 +765,9 @@ __device__ __forceinline__ void tbf_range(const Pass2D &p, long long f, const lo
             tbf_decode_ring<V, STOR>(c, c.sRP + C::PF * C::RAWB, c.sP, c.sP + C::NBP * C::ROWB);
         }
 
+        // the fill rows of a segment inside the grid run a loop that skips the idle stages (T^2 of
+        // the segment's (rows + 2T) T stage rows, a fifth of them on a 3001 x 2003 grid, whose
+        // blocks have 30 rows each: with the dealt segments 692 -> 622 us for 150 steps);
         // rows that need boundary handling: the grid's top rows (for every stage), its bottom
         // rows, and every row of a pass that forwards trailing stages
         const bool partial = (c.tsteps < T);
@@ -767,37 +775,32 @@ __device__ __forceinline__ void tbf_range(const Pass2D &p, long long f, const lo
         // (stage s meets row 0 at i = s when the segment starts at the top, and rows ny-1 / ny
         // from i = ny-1 - y_start on)
         const int i_b = partial ? n_it : max(i_a, min(n_it, c.ny - 1 - c.y_start));
+        const int i_h = (partial || c.y_start == 0) ? 0 : min(2 * T - 2, i_b);
         int i = 0;
 #pragma unroll 1
         for (; i < i_a; i++) tbf_step_rt<KIND, T, V, MODE_SPECIAL, SWAP, STOR>(c, k, A, B, i, r);
-        if (SWAP) {
-            if (i < i_b && (i & 1)) {
-                if (c.edge) tbf_step<KIND, T, V, MODE_EDGE, 1, SWAP, STOR>(c, k, A, B, i, r);
-                else tbf_step<KIND, T, V, MODE_PLAIN, 1, SWAP, STOR>(c, k, A, B, i, r);
-                i++;
-            }
-            if (c.edge) {
 #pragma unroll 1
-                for (; i + 1 < i_b; i += 2) {
-                    tbf_step<KIND, T, V, MODE_EDGE, 0, SWAP, STOR>(c, k, A, B, i, r);
-                    tbf_step<KIND, T, V, MODE_EDGE, 1, SWAP, STOR>(c, k, A, B, i + 1, r);
-                }
-            } else {
-#pragma unroll 1
-                for (; i + 1 < i_b; i += 2) {
-                    tbf_step<KIND, T, V, MODE_PLAIN, 0, SWAP, STOR>(c, k, A, B, i, r);
-                    tbf_step<KIND, T, V, MODE_PLAIN, 1, SWAP, STOR>(c, k, A, B, i + 1, r);
-                }
-            }
-        } else {
-            if (c.edge) {
-#pragma unroll 1
-                for (; i < i_b; i++) tbf_step<KIND, T, V, MODE_EDGE, 0, SWAP, STOR>(c, k, A, B, i, r);
-            } else {
-#pragma unroll 1
-                for (; i < i_b; i++) tbf_step<KIND, T, V, MODE_PLAIN, 0, SWAP, STOR>(c, k, A, B, i, r);
-            }
+        for (; i < i_h; i++) tbf_step_rt<KIND, T, V, MODE_HEAD, SWAP, STOR>(c, k, A, B, i, r);
+        if (SWAP && i < i_b && (i & 1)) {
+            tbf_step<KIND, T, V, MODE_GHOST, 1, SWAP, STOR>(c, k, A, B, i, r);
+            i++;
         }
+        auto rows = [&](auto mode) {
+            constexpr int M = decltype(mode)::value;
+            if (SWAP) {
+#pragma unroll 1
+                for (; i + 1 < i_b; i += 2) {
+                    tbf_step<KIND, T, V, M, 0, SWAP, STOR>(c, k, A, B, i, r);
+                    tbf_step<KIND, T, V, M, 1, SWAP, STOR>(c, k, A, B, i + 1, r);
+                }
+            } else {
+#pragma unroll 1
+                for (; i < i_b; i++) tbf_step<KIND, T, V, M, 0, SWAP, STOR>(c, k, A, B, i, r);
+            }
+        };
+        if (c.edge == 0) rows(std::integral_constant<int, MODE_PLAIN>{});
+        else if (c.edge == 1) rows(std::integral_constant<int, MODE_EDGE>{});
+        else rows(std::integral_constant<int, MODE_GHOST>{});
 #pragma unroll 1
         for (; i < n_it; i++) tbf_step_rt<KIND, T, V, MODE_SPECIAL, SWAP, STOR>(c, k, A, B, i, r);
         cp_async_wait<0>();
@@ -816,17 +819,32 @@ __global__ void __launch_bounds__(32) k_tb2f(const Pass2D p)
     for (int s = 0; s < C::NS; s++)
 #pragma unroll
         for (int j = 0; j < V / 2; j++) A[s][j] = B[s][j] = make_float2(0.f, 0.f);
-    long long f, fend;
-    if (p.starts) {
-        // (a broadcast, so that the compiler knows the bounds, and what follows from them, to be
-        // uniform across the warp and keeps it in uniform registers)
-        f = __shfl_sync(0xffffffffu, __ldg(p.starts + blockIdx.x), 0);
-        fend = __shfl_sync(0xffffffffu, __ldg(p.starts + blockIdx.x + 1), 0);
-    } else {
-        f = (long long)blockIdx.x * p.rows_per_cta;
-        fend = min(f + p.rows_per_cta, p.total_rows);
+    // segments from the plan's list, or (no list) an even share of the (tile column, row) units.
+    // The bounds are broadcast so that the compiler knows them, and what follows from them, to
+    // be uniform across the warp and keeps it in uniform registers.
+    const bool listed = p.segs != nullptr;
+    long long f = listed ? __ldg(p.seg_first + blockIdx.x) : (long long)blockIdx.x * p.rows_per_cta;
+    const long long fend = listed ? __ldg(p.seg_first + blockIdx.x + 1)
+                                  : min(f + p.rows_per_cta, p.total_rows);
+#pragma unroll 1
+    while (__shfl_sync(0xffffffffu, f < fend ? 1 : 0, 0)) {
+        int tx, s0, s1;
+        if (listed) {
+            const int4 q = __ldg(p.segs + f);
+            tx = q.x;
+            s0 = q.y;
+            s1 = q.z;
+            f++;
+        } else {
+            tx = (int)(f / p.ny);
+            s0 = (int)(f - (long long)tx * p.ny);
+            s1 = (int)min((long long)p.ny, s0 + (fend - f));
+            f += s1 - s0;
+        }
+        tbf_segment<KIND, T, V, SWAP, STOR>(p, __shfl_sync(0xffffffffu, tx, 0),
+                                            __shfl_sync(0xffffffffu, s0, 0),
+                                            __shfl_sync(0xffffffffu, s1, 0), A, B, smem);
     }
-    tbf_range<KIND, T, V, SWAP, STOR>(p, f, fend, A, B, smem);
 }
 
 }  // namespace stn

@@ -159,10 +159,11 @@ __global__ void __launch_bounds__(32, 12) k_tb2f_queue(const QueueBatch2D q)
             }
         } else if (w.k < G.P) {
             const Pass2D &p = q.passes[G.pass_base + w.k];
-            const long long lo = (long long)w.tx * G.ny + r0;
-            const long long hi = lo + (r1 - r0);
-            if (G.kind == KDIFF) tbf_range<KDIFF, T, V, SW, STOR_F32>(p, lo, hi, A, B, smem);
-            else tbf_range<KTHERM, T, V, SW, STOR_SRC>(p, lo, hi, A, B, smem);
+            // (broadcasts: uniform registers, see k_tb2f)
+            const int tx = __shfl_sync(0xffffffffu, w.tx, 0);
+            const int lo = __shfl_sync(0xffffffffu, r0, 0), hi = __shfl_sync(0xffffffffu, r1, 0);
+            if (G.kind == KDIFF) tbf_segment<KDIFF, T, V, SW, STOR_F32>(p, tx, lo, hi, A, B, smem);
+            else tbf_segment<KTHERM, T, V, SW, STOR_SRC>(p, tx, lo, hi, A, B, smem);
         } else {
             for (int y = r0; y < r1; y++) {
                 const float *s = G.copy_from + (long long)y * G.ld_copy;
