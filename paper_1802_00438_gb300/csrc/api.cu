@@ -66,6 +66,7 @@ struct stencil_plan_s {
     long long ld_src = 0;   // its row pitch, floats
     int ntx_star = 0, nty_star = 0;   // star diffusion (rad > 1): tiles along x and y
     int nseg_star = 1, zseg_star = 0; // 3D star: z-segments per tile column, their length
+    int star_rows = 0;                // 2D star streamed by one-warp blocks (contracted, radius 2)
     std::vector<PassCfg3D> cfg3;
     // timing
     bool timing = false;
@@ -528,11 +529,12 @@ int upload_segments(std::vector<std::vector<Seg3>> &segs, int *ctas, int *seg_of
 // boundary tests).  Measured on GB300 against contiguous ranges balanced the same way: 12000^2
 // diffusion 4001 -> 4184 GCell/s, 16384^2 4114 -> 4247, Hotspot 3058 -> 3107, 8192^2 Hotspot 2645
 // -> 2761 (T = 8, 8 cells per thread); DRAM reads of a 16384^2 diffusion pass 1.31 -> 1.10 GB.
-int segments_2d(stencil_plan_s *p, int bps, PassCfg2D *c)
+// halo: rows per side a segment streams besides its own (R T); V: cells per thread.
+int segments_2d(stencil_plan_s *p, int bps, int halo, int V, PassCfg2D *c)
 {
     std::vector<double> w(c->ntx, 1.0);
     w.front() = kEdge2;
-    w.back() = p->d.nx % c->shape.V == 0 ? kEdge2 : kGhost2;
+    w.back() = p->d.nx % V == 0 ? kEdge2 : kGhost2;
     std::vector<std::vector<Seg3>> segs;
     // A scheduler issues from its oldest ready warp first, so of the one-warp blocks that share one
     // the first to arrive (blocks arrive in order, one per SM and round, four rounds per warp
@@ -543,7 +545,7 @@ int segments_2d(stencil_plan_s *p, int bps, PassCfg2D *c)
     std::vector<double> speed(slots, 1.0);
     for (int b = 0; b < slots && ranks > 1; b++)
         speed[b] = 1.0 + kAhead2 * (1.0 - 2.0 * (b / p->sms / 4) / (ranks - 1));
-    best_segments(p->d.ny, slots, kFill2 * c->shape.T, (c->shape.V == 8 ? kTop2V8 : kTop2V4) * c->shape.T, w, speed, 0.5, &segs);
+    best_segments(p->d.ny, slots, kFill2 * halo, (V == 8 ? kTop2V8 : kTop2V4) * halo, w, speed, 0.5, &segs);
     return upload_segments(segs, &c->ctas, &c->seg_off, &c->segs);
 }
 
@@ -569,7 +571,7 @@ int prepare2(stencil_plan_s *p, int Tk, PassCfg2D **out)
         c.rows_per_cta = (c.total + ctas - 1) / ctas;
         c.ctas = (int)((c.total + c.rows_per_cta - 1) / c.rows_per_cta);
         if (!c.shape.exact && c.shape.kind != ST_DIFFUSION_VAR) {
-            const int rc = segments_2d(p, bps, &c);
+            const int rc = segments_2d(p, bps, c.shape.T, c.shape.V, &c);
             if (rc != ST_OK) return rc;
         }
         c.ready = true;
@@ -596,7 +598,26 @@ int prepare_traj(stencil_plan_s *p, PassCfg2D **out)
         const int cx = tb2d_tile_width(c.shape) - 2 * tb2d_halo(c.shape);
         c.ntx = (p->d.nx + cx - 1) / cx;
         c.total = (long long)c.ntx * p->d.ny;
-        const int rc = segments_2d(p, bps, &c);
+        const int rc = segments_2d(p, bps, c.shape.T, c.shape.V, &c);
+        if (rc != ST_OK) return rc;
+        c.ready = true;
+    }
+    *out = &c;
+    return ST_OK;
+}
+
+// The streamed radius-2 star: T = 1, 2 or 4 steps fused.
+int prepare_star2f(stencil_plan_s *p, int Tk, PassCfg2D **out)
+{
+    if ((int)p->cfg2.size() <= Tk) p->cfg2.resize(Tk + 1);
+    PassCfg2D &c = p->cfg2[Tk];
+    if (!c.ready) {
+        int bps = 0;
+        const cudaError_t e = star2f_prepare(Tk, &bps);
+        if (e != cudaSuccess) return map_cuda(e);
+        if (bps < 1) return ST_ERR_UNSUPPORTED;
+        c.ntx = (p->d.nx + star2f_compute_width() - 1) / star2f_compute_width();
+        const int rc = segments_2d(p, bps, 2 * Tk, 8, &c);
         if (rc != ST_OK) return rc;
         c.ready = true;
     }
@@ -900,8 +921,42 @@ int run_pass_star3(stencil_plan_s *p, const float *src, float *dst, const float 
     return map_cuda(e);
 }
 
-int run_pass_star(stencil_plan_s *p, const float *src, float *dst, const float *k, int tsteps)
+int run_pass_star2f(stencil_plan_s *p, const float *src, long long lds, float *dst, long long ldd,
+                    const float *k, int tsteps)
 {
+    PassCfg2D *c = nullptr;
+    int rc = prepare_star2f(p, tsteps <= 1 ? 1 : tsteps <= 2 ? 2 : 4, &c);
+    if (rc != ST_OK) return rc;
+    Pass2D a = {};
+    a.in = src;
+    a.out = dst;
+    a.ld_in = lds;
+    a.ld_out = ldd;
+    a.nx = p->d.nx;
+    a.ny = p->d.ny;
+    a.tsteps = tsteps;
+    a.ntx = c->ntx;
+    a.seg_first = static_cast<const int *>(c->segs);
+    a.segs = reinterpret_cast<const int4 *>(a.seg_first + c->seg_off);
+    a.ctas = c->ctas;
+    a.vec_in = ((uintptr_t)src % 16 == 0) && (lds % 4 == 0);
+    a.vec_out = ((uintptr_t)dst % 16 == 0) && (ldd % 4 == 0);
+    StarCoef2 ks;
+    for (int i = 0; i < 9; i++) ks.k[i] = k[i];
+    if (p->timing && p->ev_used + 2 > 2 * 1024) {
+        rc = flush_timing(p);
+        if (rc != ST_OK) return rc;
+    }
+    cudaError_t e = record(p, true);
+    if (e == cudaSuccess) e = star2f_launch(tsteps <= 1 ? 1 : tsteps <= 2 ? 2 : 4, a, ks, p->stream);
+    if (e == cudaSuccess) e = record(p, false);
+    return map_cuda(e);
+}
+
+int run_pass_star(stencil_plan_s *p, const float *src, long long lds, float *dst, long long ldd,
+                  const float *k, int tsteps)
+{
+    if (p->star_rows) return run_pass_star2f(p, src, lds, dst, ldd, k, tsteps);
     if (p->d.ndim == 3) return run_pass_star3(p, src, dst, k, tsteps);
     PassStar2D a = {};
     a.in = src;
@@ -1136,12 +1191,26 @@ static int plan_create(stencil_plan *out, const stencil_desc *desc)
                 if (cx > 0 && cy > 0 && cx * cy >= 0.7 * 128 * 128) T = t;
             }
         }
-        if (!star2d_available(d.rad, d.exact, T)) rc = ST_ERR_UNSUPPORTED;
-        if (rc == ST_OK) {
+        // contracted, radius 2, no tile asked for: streamed by one-warp blocks, T = 4 unless forced
+        // (8192^2 x 64: 2411 us; T = 2 3227 us, tiles 4026 us)
+        if (d.rad == 2 && !d.exact && !d.force_bx && !d.force_by && !d.force_vec &&
+            (T == 1 || T == 2 || T == 4)) {
+            PassCfg2D *c = nullptr;
+            rc = prepare_star2f(p, T, &c);
+            if (rc == ST_OK) {
+                p->star_rows = 1;
+                p->T = T;
+                p->ld_scratch = ((long long)d.nx + 31) / 32 * 32;
+                p->scratch_bytes = (size_t)p->ld_scratch * d.ny * sizeof(float);
+            }
+        } else if (!star2d_available(d.rad, d.exact, T)) {
+            rc = ST_ERR_UNSUPPORTED;
+        }
+        if (rc == ST_OK && !p->star_rows) {
             e = star2d_prepare(d.rad, d.exact, T);
             if (e != cudaSuccess) rc = map_cuda(e);
         }
-        if (rc == ST_OK) {
+        if (rc == ST_OK && !p->star_rows) {
             p->T = T;
             const int cx = 128 - 2 * star2d_halo_x(d.rad, T), cy = 128 - 2 * star2d_halo_y(d.rad, T);
             p->ntx_star = (d.nx + cx - 1) / cx;
@@ -1326,8 +1395,9 @@ static int plan_create(stencil_plan *out, const stencil_desc *desc)
     // Contracted first-order plans on rows that are no whole 16-byte chunks (nx not a multiple of
     // 4): the passes between the first and the last run between two padded scratch grids, so that
     // only those two touch the caller's rows (staged and stored cell by cell)
-    const bool two = rc == ST_OK && d.nx % 4 != 0 && !d.exact && !p->res && !p->stor && d.rad <= 1 &&
-                     d.kind != ST_DIFFUSION_VAR && (d.ndim == 2 || p->alg3);
+    const bool two = rc == ST_OK && d.nx % 4 != 0 && !d.exact && !p->res && !p->stor &&
+                     (d.rad <= 1 || p->star_rows) && d.kind != ST_DIFFUSION_VAR &&
+                     (d.ndim == 2 || p->alg3);
     if (rc == ST_OK && p->scratch_bytes) {
         e = stn::dev_malloc(&p->scratch, p->scratch_bytes);
         if (e == cudaSuccess && two) e = stn::dev_malloc(&p->scratch2, p->scratch_bytes);
@@ -1472,7 +1542,7 @@ int stencil_run(stencil_plan p, const void *grid_in, void *grid_out, const void 
                             : shift ? ((passes - i) % 2 == 0) : ((passes - 1 - i) % 2 == 0);
         float *dst = to_out ? out : (two && i % 2) ? p->scratch2 : p->scratch;
         const long long ldd = to_out ? ldo : ldsc;
-        int rc = d.rad > 1     ? run_pass_star(p, src, dst, coeffs, ts)
+        int rc = d.rad > 1     ? run_pass_star(p, src, lds, dst, ldd, coeffs, ts)
                  : d.ndim == 2 ? run_pass2(p, src, lds, dst, ldd, pw, coeffs, ts)
                                : run_pass3(p, src, lds, dst, ldd, pw, ldp, coeffs, ts);
         if (rc != ST_OK) {
@@ -1599,6 +1669,17 @@ int stencil_plan_get_info(stencil_plan p, stencil_plan_info *info)
         info->warps = 8;
         info->ctas = p->ntx_star * p->nty_star * p->nseg_star;
         info->kernel_id = 6;
+    } else if (p->star_rows) {
+        PassCfg2D *c = nullptr;
+        const int rc = prepare_star2f(p, p->T, &c);
+        if (rc != ST_OK) return rc;
+        info->bx = star2f_tile_width();
+        info->by = 0;
+        info->halo = (star2f_tile_width() - star2f_compute_width()) / 2;
+        info->vec = 8;
+        info->warps = 1;
+        info->ctas = c->ctas;
+        info->kernel_id = 8;
     } else if (p->d.rad > 1) {
         info->bx = 128;
         info->by = 128;

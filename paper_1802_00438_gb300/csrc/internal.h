@@ -162,6 +162,16 @@ cudaError_t star2d_prepare(int R, int exact, int T);
 cudaError_t star2d_launch(int R, int exact, int T, const PassStar2D &p, const CUtensorMap &tin,
                           cudaStream_t st);
 
+// One pass of the contracted radius-2 star in 2D streamed by one-warp blocks (star2f.cu), T in
+// {1, 2, 4}; of Pass2D it uses the grids, their pitches and alignment, tsteps and the segments.
+struct StarCoef2 {
+    float k[9];                // cc, then w, e, s, n at distance 1 and at distance 2
+};
+int star2f_tile_width();       // cells per tile incl. halos
+int star2f_compute_width();
+cudaError_t star2f_prepare(int T, int *blocks_per_sm);
+cudaError_t star2f_launch(int T, const Pass2D &p, const StarCoef2 &k, cudaStream_t st);
+
 // One pass of the 3D star diffusion of radius R (star3d.cu): one block per (tile, z-segment).
 struct PassStar3D {
     const float *in;

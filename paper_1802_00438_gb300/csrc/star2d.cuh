@@ -1,4 +1,5 @@
-// Star diffusion of radius R in 2D (4R+1 points): combined spatial and temporal blocking with
+// Star diffusion of radius R in 2D (4R+1 points), in shared-memory tiles (exact plans, radii 3 and
+// 4, forced tiles; contracted plans of radius 2 stream rows instead, star2f.cu): combined spatial and temporal blocking with
 // halos of width R*T (arXiv 1802.00438, Eqs. 1-2 with rad = R > 1, the paper's named
 // extension to higher-order stencils; Sec. 3.2's fused steps; Sec. 5.1's clamped boundary).
 //

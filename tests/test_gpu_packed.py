@@ -59,3 +59,19 @@ def test_segments_3d(eng, orc, kind, T, by):  # noqa: F811
         assert (info["T"], info["by"]) == (T, by)
         o = orc.run(kind, w.u0, w.coef, steps, w.power)
         assert max_rel(g, o) <= TOL, (nx, ny, nz, steps, max_rel(g, o))
+
+
+@pytest.mark.parametrize("T", [1, 2, 4])
+def test_star_rows(eng, orc, T):  # noqa: F811
+    """The streamed radius-2 star: the clamp reaches two cells, so a width may end on a lane's last
+    cell or on one of the next lane's first two; heights around the fill of a segment."""
+    import torch
+    for n, nx in enumerate([1, 2, 7, 8, 9, 10, 239, 240, 241, 242, 247, 248, 249, 490]):
+        for ny in (1, 2, 3, 19 + n % 5, 70):
+            w = synth.make_star(2, 2, nx, ny, seed=8700 + 7 * n + ny)
+            u = torch.from_numpy(w.u0).cuda()
+            plan = eng.Plan(0, 2, nx, ny, rad=2, force_T=T)
+            steps = 2 * T + 1 + n % 2
+            g = plan.run(u, torch.full_like(u, float("nan")), w.coef, steps).cpu().numpy()
+            plan.close()
+            assert max_rel(g, orc.run_star(2, w.u0, w.coef, steps)) <= TOL, (nx, ny, steps)
