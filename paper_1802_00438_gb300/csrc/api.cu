@@ -570,7 +570,7 @@ int prepare2(stencil_plan_s *p, int Tk, PassCfg2D **out)
                                              std::max<long long>(1, c.total / min_rows));
         c.rows_per_cta = (c.total + ctas - 1) / ctas;
         c.ctas = (int)((c.total + c.rows_per_cta - 1) / c.rows_per_cta);
-        if (!c.shape.exact && c.shape.kind != ST_DIFFUSION_VAR) {
+        if (tb2d_segments(c.shape)) {
             const int rc = segments_2d(p, bps, c.shape.T, c.shape.V, &c);
             if (rc != ST_OK) return rc;
         }
@@ -1396,8 +1396,7 @@ static int plan_create(stencil_plan *out, const stencil_desc *desc)
     // 4): the passes between the first and the last run between two padded scratch grids, so that
     // only those two touch the caller's rows (staged and stored cell by cell)
     const bool two = rc == ST_OK && d.nx % 4 != 0 && !d.exact && !p->res && !p->stor &&
-                     (d.rad <= 1 || p->star_rows) && d.kind != ST_DIFFUSION_VAR &&
-                     (d.ndim == 2 || p->alg3);
+                     (d.rad <= 1 || p->star_rows) && (d.ndim == 2 || p->alg3);
     if (rc == ST_OK && p->scratch_bytes) {
         e = stn::dev_malloc(&p->scratch, p->scratch_bytes);
         if (e == cudaSuccess && two) e = stn::dev_malloc(&p->scratch2, p->scratch_bytes);

@@ -134,6 +134,7 @@ cudaError_t hot_source(const float *p, long long ld_p, float *dst, long long ld_
                        float amb, float rz, float sdc, int V, cudaStream_t st);
 
 bool tb2d_available(const Shape2D &s);
+bool tb2d_segments(const Shape2D &s);    // the kernel streams dealt segments (Pass2D::segs)
 int tb2d_block_threads(const Shape2D &s);
 int tb2d_tile_width(const Shape2D &s);   // cells per tile incl. halos
 int tb2d_halo(const Shape2D &s);

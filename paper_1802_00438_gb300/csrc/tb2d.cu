@@ -16,6 +16,11 @@ static const Tb2dEntry *tb2d_find(const Shape2D &s)
     return nullptr;
 }
 
+bool tb2d_segments(const Shape2D &s)
+{
+    return !s.exact && (s.kind != KVDIFF || (s.W == 1 && (s.T == 2 || s.T == 4)));
+}
+
 bool tb2d_available(const Shape2D &s) { return tb2d_find(s) != nullptr; }
 int tb2d_block_threads(const Shape2D &s) { return 32 * (s.W > 0 ? s.W : 1); }   // W <= 0: one warp
 int tb2d_tile_width(const Shape2D &s) { return 32 * s.V * (s.W > 0 ? s.W : 1); }
