@@ -139,10 +139,10 @@ bool available(const stencil_plan_s *p, int T)
 // 4096^2, 10 % on 1600^2, 25 % on 1000 x 600.
 struct Cal2D { int kind, T, V, W; double a, b_us; };
 const Cal2D kCal2D[] = {
-    {0, 4, 4, 1, 12.6, 6.6},  {0, 8, 4, 1, 10.2, 6.5},  {0, 12, 4, 1, 9.8, 13.1}, {0, 4, 8, 1, 12.0, 6.4},
-    {0, 6, 8, 1, 10.5, 9.1},  {0, 8, 8, 1, 8.4, 16.5},  {0, 8, 8, 0, 9.5, 8.9},   {0, 12, 4, 0, 9.9, 8.8},
-    {1, 4, 4, 1, 22.4, 2.0},  {1, 8, 4, 1, 12.2, 9.4},  {1, 12, 4, 1, 11.7, 18.9}, {1, 4, 8, 1, 20.0, 5.4},
-    {1, 6, 8, 1, 13.5, 12.4}, {1, 8, 8, 1, 11.5, 24.7}, {1, 8, 8, 0, 11.9, 11.4}, {1, 12, 4, 0, 12.3, 12.8},
+    {0, 4, 4, 1, 13.1, 4.7},  {0, 8, 4, 1, 9.7, 7.5},   {0, 12, 4, 1, 9.7, 13.4},  {0, 4, 8, 1, 12.1, 6.2},
+    {0, 6, 8, 1, 10.5, 7.2},  {0, 8, 8, 1, 8.1, 11.7},  {0, 8, 8, 0, 9.4, 9.0},    {0, 12, 4, 0, 9.9, 8.8},
+    {1, 4, 4, 1, 22.7, 1.7},  {1, 8, 4, 1, 11.8, 8.3},  {1, 12, 4, 1, 11.3, 22.8}, {1, 4, 8, 1, 20.5, 3.4},
+    {1, 6, 8, 1, 13.4, 10.1}, {1, 8, 8, 1, 11.4, 19.8}, {1, 8, 8, 0, 11.9, 11.4},  {1, 12, 4, 0, 12.3, 12.8},
 };
 
 struct Cand2D { int T, V, W; };
@@ -1192,7 +1192,7 @@ static int plan_create(stencil_plan *out, const stencil_desc *desc)
             }
         }
         // contracted, radius 2, no tile asked for: streamed by one-warp blocks, T = 4 unless forced
-        // (8192^2 x 64: 2411 us; T = 2 3227 us, tiles 4026 us)
+        // (8192^2 x 64: 2327 us; T = 2 3227 us, tiles 4026 us)
         if (d.rad == 2 && !d.exact && !d.force_bx && !d.force_by && !d.force_vec &&
             (T == 1 || T == 2 || T == 4)) {
             PassCfg2D *c = nullptr;
@@ -1249,11 +1249,23 @@ static int plan_create(stencil_plan *out, const stencil_desc *desc)
             if (!d.exact && d.partial_rows == 1) p->W = 0;   // partial rows updated in place
             if (!d.exact && d.partial_rows == 2) p->W = 1;   // two alternating sets of partial rows
             if (p->stor && !d.force_T && !d.force_vec && !d.force_bx && !d.partial_rows) {
-                // 16-bit storage, nothing forced: T = 8, 8 cells per lane, rows in place (measured
-                // on 16384^2: Hotspot 1990 GCell/s against 1802 for V = 4 two-row; diffusion 2720
-                // against 2380 for V = 8 two-row)
+                // 16-bit storage, nothing forced: T = 8 with 8 cells per lane, rows in place, or,
+                // where a block has few rows, 4 cells per lane (three warps per scheduler).  The
+                // line is the float32 kernels' (their model): measured on GB300, 8192^2 Hotspot
+                // bf16 x 200 5241 against 6171 us, 3000 x 2000 887 against 846, 1100 x 6000 x 100
+                // 611 against 521
+                int b8 = 0, b4 = 0;
+                const Shape2D s8{d.kind, 0, 8, 8, 0, shape_stor(p)}, s4{d.kind, 0, 8, 4, 1, shape_stor(p)};
                 p->V = 8;
                 p->W = 0;
+                if (tb2d_available(s4) && tb2d_prepare(s8, &b8) == cudaSuccess &&
+                    tb2d_prepare(s4, &b4) == cudaSuccess && b8 > 0 && b4 > 0 &&
+                    model_gcells_2d(d, p->sms, Cand2D{8, 4, 1}, b4, 1000) >
+                        1.08 * model_gcells_2d(d, p->sms, Cand2D{8, 8, 0}, b8, 1000)) {
+                    p->V = 4;
+                    p->W = 1;
+                }
+                (void)cudaGetLastError();
             }
             if (!d.exact && !var && !p->stor && !d.force_T && !d.force_vec && !d.force_bx && !d.partial_rows) {
                 // contracted, nothing forced: the compiled (T, V, variant) the model rates best

@@ -20,7 +20,7 @@
 // (2304 of its cycles per 128 x 128 step); here a row crosses shared memory once per pass, the
 // neighbours of a stage come from registers and four shuffles per 8 cells, and the halo wastes
 // 16 of 256 cells instead of 16 of 128 in both directions.  Measured on GB300 (T = 4), tiles ->
-// here: 8192^2 x 64 steps 4026 -> 2411 us, 8191^2 5919 -> 2523, 4096^2 1244 -> 776, 2048^2 637 ->
+// here: 8192^2 x 64 steps 4026 -> 2327 us, 8191^2 5919 -> 2523, 4096^2 1244 -> 741, 2048^2 637 ->
 // 340, 1024^2 310 -> 242, 512^2 x 32 143 -> 112: faster over the whole range, so contracted plans
 // of radius 2 run this unless a tile is asked for.  It is bound by issue and latency with two
 // warps per scheduler, like the first-order kernel.
@@ -217,19 +217,23 @@ __global__ void __launch_bounds__(32) k_star2f(const Pass2D p, const StarCoef2 k
         const int i_b = partial ? n_it : max(i_a, min(n_it, c.ny - 1 - c.y_start));
         const int i_h = (partial || c.y_start == 0) ? 0 : min(4 * T - 4, i_b);
         int i = 0;
-#pragma unroll 1
-        for (; i < i_a; i++) star_row<T, MODE_SPECIAL>(c, k, A, i, r);
+        // (one body for the special rows of the top and the bottom: cold code, see tb2f_kernel.cuh)
 #pragma unroll 1
         for (; i < i_h; i++) star_row<T, MODE_HEAD>(c, k, A, i, r);
-        auto rows = [&](auto mode) {
 #pragma unroll 1
-            for (; i < i_b; i++) star_row<T, decltype(mode)::value>(c, k, A, i, r);
-        };
-        if (c.edge == 0) rows(std::integral_constant<int, MODE_PLAIN>{});
-        else if (c.edge == 1) rows(std::integral_constant<int, MODE_EDGE>{});
-        else rows(std::integral_constant<int, MODE_GHOST>{});
+        for (int part = 0; part < 2; part++) {
+            const int end = part == 0 ? i_a : n_it;
 #pragma unroll 1
-        for (; i < n_it; i++) star_row<T, MODE_SPECIAL>(c, k, A, i, r);
+            for (; i < end; i++) star_row<T, MODE_SPECIAL>(c, k, A, i, r);
+            if (part == 1) break;
+            auto rows = [&](auto mode) {
+#pragma unroll 1
+                for (; i < i_b; i++) star_row<T, decltype(mode)::value>(c, k, A, i, r);
+            };
+            if (c.edge == 0) rows(std::integral_constant<int, MODE_PLAIN>{});
+            else if (c.edge == 1) rows(std::integral_constant<int, MODE_EDGE>{});
+            else rows(std::integral_constant<int, MODE_GHOST>{});
+        }
         cp_async_wait<0>();
         __syncwarp();
     }

@@ -36,8 +36,8 @@
 // load yields two pairs.  Stage 0 keeps partial rows like the others: it reads one ring row per
 // iteration (the direct form read three, and would have to pair each).
 // Measured (GB300), scalar kernel on even ranges -> this one on dealt segments: 16384^2 Hotspot
-// 2928 -> 3118 GCell/s, diffusion 3753 -> 4244, 8192^2 Hotspot with bf16 storage 2032 -> 2630,
-// 3001 x 2003 Hotspot 1053 -> 1466, 3000 x 2000 diffusion 1900.
+// 2928 -> 3200 GCell/s, diffusion 3753 -> 4466, 8192^2 Hotspot with bf16 storage 2032 -> 2580,
+// 3001 x 2003 Hotspot 1053 -> 1545, 3000 x 2000 diffusion 1907.
 // What bounds it now (ncu, 6144^2): Hotspot FMA pipe 58 % busy, issue 57 %, shared memory 64 %
 // (every stage reads its source row), two warps per scheduler; diffusion 58 / 52 / 30 %.
 //
@@ -637,15 +637,6 @@ __device__ __forceinline__ void tbf_step(const CtxF &c, const CoefF &k,
     if (C::Q16) r.rr = (r.rr + 1 == C::NBR) ? 0 : r.rr + 1;
 }
 
-template <int KIND, int T, int V, int MODE, bool SWAP, int STOR>
-__device__ __forceinline__ void tbf_step_rt(const CtxF &c, const CoefF &k,
-                                            float2 (&A)[TB2F<KIND, T, V>::NS][V / 2],
-                                            float2 (&B)[TB2F<KIND, T, V>::NS][V / 2], int i, RowF &r)
-{
-    if (SWAP && (i & 1)) tbf_step<KIND, T, V, MODE, 1, SWAP, STOR>(c, k, A, B, i, r);
-    else tbf_step<KIND, T, V, MODE, 0, SWAP, STOR>(c, k, A, B, i, r);
-}
-
 // Rows [s0, s1) of tile column tx of one grid's pass.
 template <int KIND, int T, int V, bool SWAP, int STOR>
 __device__ __forceinline__ void tbf_segment(const Pass2D &p, const int tx, const int s0, const int s1,
@@ -777,32 +768,50 @@ __device__ __forceinline__ void tbf_segment(const Pass2D &p, const int tx, const
         const int i_b = partial ? n_it : max(i_a, min(n_it, c.ny - 1 - c.y_start));
         const int i_h = (partial || c.y_start == 0) ? 0 : min(2 * T - 2, i_b);
         int i = 0;
+        // Every loop but the two of ordinary rows has one body, with the partial rows updated in
+        // place: these bodies are cold code that every block fetches anew (a body per array phase
+        // cost a pass several us: see kCal2D in api.cu).  With float32 rows and two sets of
+        // partial rows the special rows of the top and the bottom share theirs, too (16384^2
+        // diffusion 4253 -> 4469 GCell/s); the other instances are faster with one each (8192^2
+        // bf16 Hotspot 5397 -> 5225 us for 200 steps).
+        constexpr bool kShare = SWAP && !C::Q16;
 #pragma unroll 1
-        for (; i < i_a; i++) tbf_step_rt<KIND, T, V, MODE_SPECIAL, SWAP, STOR>(c, k, A, B, i, r);
+        for (; i < i_h; i++) tbf_step<KIND, T, V, MODE_HEAD, 0, false, STOR>(c, k, A, B, i, r);
+        auto special = [&](int end) {
 #pragma unroll 1
-        for (; i < i_h; i++) tbf_step_rt<KIND, T, V, MODE_HEAD, SWAP, STOR>(c, k, A, B, i, r);
-        if (SWAP && i < i_b && (i & 1)) {
-            tbf_step<KIND, T, V, MODE_GHOST, 1, SWAP, STOR>(c, k, A, B, i, r);
-            i++;
-        }
-        auto rows = [&](auto mode) {
-            constexpr int M = decltype(mode)::value;
-            if (SWAP) {
-#pragma unroll 1
-                for (; i + 1 < i_b; i += 2) {
-                    tbf_step<KIND, T, V, M, 0, SWAP, STOR>(c, k, A, B, i, r);
-                    tbf_step<KIND, T, V, M, 1, SWAP, STOR>(c, k, A, B, i + 1, r);
-                }
-            } else {
-#pragma unroll 1
-                for (; i < i_b; i++) tbf_step<KIND, T, V, M, 0, SWAP, STOR>(c, k, A, B, i, r);
-            }
+            for (; i < end; i++) tbf_step<KIND, T, V, MODE_SPECIAL, 0, false, STOR>(c, k, A, B, i, r);
         };
-        if (c.edge == 0) rows(std::integral_constant<int, MODE_PLAIN>{});
-        else if (c.edge == 1) rows(std::integral_constant<int, MODE_EDGE>{});
-        else rows(std::integral_constant<int, MODE_GHOST>{});
+        auto ordinary = [&]() {
+            auto rows = [&](auto mode) {
+                constexpr int M = decltype(mode)::value;
+                if constexpr (SWAP) {
 #pragma unroll 1
-        for (; i < n_it; i++) tbf_step_rt<KIND, T, V, MODE_SPECIAL, SWAP, STOR>(c, k, A, B, i, r);
+                    for (; i + 1 < i_b; i += 2) {
+                        tbf_step<KIND, T, V, M, 0, true, STOR>(c, k, A, B, i, r);
+                        tbf_step<KIND, T, V, M, 1, true, STOR>(c, k, A, B, i + 1, r);
+                    }
+                } else {
+#pragma unroll 1
+                    for (; i < i_b; i++) tbf_step<KIND, T, V, M, 0, false, STOR>(c, k, A, B, i, r);
+                }
+            };
+            if (c.edge == 0) rows(std::integral_constant<int, MODE_PLAIN>{});
+            else if (c.edge == 1) rows(std::integral_constant<int, MODE_EDGE>{});
+#pragma unroll 1
+            for (; i < i_b; i++) tbf_step<KIND, T, V, MODE_GHOST, 0, false, STOR>(c, k, A, B, i, r);
+        };
+        if constexpr (kShare) {
+#pragma unroll 1
+            for (int part = 0; part < 2; part++) {   // one copy of the special body for both ends
+                special(part == 0 ? i_a : n_it);
+                if (part == 1) break;
+                ordinary();
+            }
+        } else {
+            special(i_a);
+            ordinary();
+            special(n_it);
+        }
         cp_async_wait<0>();
         __syncwarp();
     }
