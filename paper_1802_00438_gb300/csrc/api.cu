@@ -549,6 +549,15 @@ int segments_2d(stencil_plan_s *p, int bps, int halo, int V, PassCfg2D *c)
     return upload_segments(segs, &c->ctas, &c->seg_off, &c->segs);
 }
 
+// A remainder pass (fewer steps than the plan's T) gets its own shorter kernel, whose segments are
+// allocated on its first use.  Where that cannot be done - the stream is being captured, or no
+// memory is left - the plan's own kernel runs the fewer steps instead.
+bool capturing(const stencil_plan_s *p)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(p->stream, &st) == cudaSuccess && st != cudaStreamCaptureStatusNone;
+}
+
 int prepare2(stencil_plan_s *p, int Tk, PassCfg2D **out)
 {
     if ((int)p->cfg2.size() <= Tk) p->cfg2.resize(Tk + 1);
@@ -556,6 +565,7 @@ int prepare2(stencil_plan_s *p, int Tk, PassCfg2D **out)
     if (!c.ready) {
         c.shape = Shape2D{p->d.kind, p->d.exact ? 1 : 0, Tk, p->V, p->W, shape_stor(p)};
         if (!tb2d_available(c.shape)) return ST_ERR_UNSUPPORTED;
+        if (Tk < p->T && tb2d_segments(c.shape) && capturing(p)) return prepare2(p, p->T, out);
         int bps = 0;
         cudaError_t e = tb2d_prepare(c.shape, &bps);
         if (e != cudaSuccess) return map_cuda(e);
@@ -572,6 +582,10 @@ int prepare2(stencil_plan_s *p, int Tk, PassCfg2D **out)
         c.ctas = (int)((c.total + c.rows_per_cta - 1) / c.rows_per_cta);
         if (tb2d_segments(c.shape)) {
             const int rc = segments_2d(p, bps, c.shape.T, c.shape.V, &c);
+            if (rc == ST_ERR_OOM && Tk < p->T) {
+                (void)cudaGetLastError();
+                return prepare2(p, p->T, out);
+            }
             if (rc != ST_OK) return rc;
         }
         c.ready = true;
@@ -598,8 +612,12 @@ int prepare_traj(stencil_plan_s *p, PassCfg2D **out)
         const int cx = tb2d_tile_width(c.shape) - 2 * tb2d_halo(c.shape);
         c.ntx = (p->d.nx + cx - 1) / cx;
         c.total = (long long)c.ntx * p->d.ny;
-        const int rc = segments_2d(p, bps, c.shape.T, c.shape.V, &c);
-        if (rc != ST_OK) return rc;
+        // even shares: these passes wait for their writes (every fused step goes to memory), and
+        // nothing is allocated on the first call
+        const long long ctas = std::min<long long>((long long)p->sms * bps,
+                                                   std::max<long long>(1, c.total / 4));
+        c.rows_per_cta = (c.total + ctas - 1) / ctas;
+        c.ctas = (int)((c.total + c.rows_per_cta - 1) / c.rows_per_cta);
         c.ready = true;
     }
     *out = &c;
@@ -632,6 +650,7 @@ int prepare3(stencil_plan_s *p, int Tk, PassCfg3D **out)
     if (!c.ready) {
         c.shape = Shape3D{p->d.kind, p->d.exact ? 1 : 0, Tk, p->VY, p->NW, p->alg3, p->VX3};
         if (!tb3d_available(c.shape)) return ST_ERR_UNSUPPORTED;
+        if (Tk < p->T && p->alg3 && capturing(p)) return prepare3(p, p->T, out);
         int bps = 0;
         cudaError_t e = tb3d_prepare(c.shape, &bps);
         if (e != cudaSuccess) return map_cuda(e);
@@ -660,6 +679,10 @@ int prepare3(stencil_plan_s *p, int Tk, PassCfg3D **out)
             std::vector<std::vector<Seg3>> segs;
             best_segments(p->d.nz, p->sms * bps, 3.0 * Tk - 1, 0.0, w, {}, 0.25, &segs);
             const int rc = upload_segments(segs, &c.ctas, &c.seg_off, &c.segs);
+            if (rc == ST_ERR_OOM && Tk < p->T) {
+                (void)cudaGetLastError();
+                return prepare3(p, p->T, out);
+            }
             if (rc != ST_OK) return rc;
         }
         c.ready = true;
@@ -1196,7 +1219,8 @@ static int plan_create(stencil_plan *out, const stencil_desc *desc)
         if (d.rad == 2 && !d.exact && !d.force_bx && !d.force_by && !d.force_vec &&
             (T == 1 || T == 2 || T == 4)) {
             PassCfg2D *c = nullptr;
-            rc = prepare_star2f(p, T, &c);
+            for (int t = T; t >= 1 && rc == ST_OK; t /= 2)   // remainder passes' segments as well
+                rc = prepare_star2f(p, t, &c);
             if (rc == ST_OK) {
                 p->star_rows = 1;
                 p->T = T;
@@ -1310,6 +1334,8 @@ static int plan_create(stencil_plan *out, const stencil_desc *desc)
             if (p->T == 0 || (d.force_T && p->T != d.force_T)) rc = ST_ERR_UNSUPPORTED;
             PassCfg2D *c = nullptr;
             if (rc == ST_OK) rc = prepare2(p, p->T, &c);
+            if (rc == ST_OK && var && !d.exact)   // remainder passes' segments as well
+                for (int ts = 1; ts < p->T && rc == ST_OK; ts++) rc = prepare2(p, kernel_T_for(p, ts), &c);
             if (rc == ST_OK && p->stor) {
                 // coded grids: rows padded to 8 cells (16 bytes), codes per (row, tile column)
                 p->cx = tb2d_tile_width(c->shape) - 2 * tb2d_halo(c->shape);
@@ -1766,7 +1792,6 @@ int stencil_plan_destroy(stencil_plan p)
     if (p->res_flags) stn::dev_free(p->res_flags);
     for (PassCfg2D &c : p->cfg2)
         if (c.segs) stn::dev_free(c.segs);
-    if (p->traj.segs) stn::dev_free(p->traj.segs);
     for (PassCfg3D &c : p->cfg3)
         if (c.segs) stn::dev_free(c.segs);
     delete p;

@@ -75,3 +75,39 @@ def test_star_rows(eng, orc, T):  # noqa: F811
             g = plan.run(u, torch.full_like(u, float("nan")), w.coef, steps).cpu().numpy()
             plan.close()
             assert max_rel(g, orc.run_star(2, w.u0, w.coef, steps)) <= TOL, (nx, ny, steps)
+
+
+@pytest.mark.parametrize("kind,ndim,T,vec,rest", [(0, 2, 8, 8, 1), (0, 2, 8, 8, 3), (1, 2, 8, 8, 2), (1, 2, 8, 4, 1),
+                                                  (0, 2, 12, 4, 5), (0, 3, 3, 0, 1), (1, 3, 3, 0, 2), (1, 3, 4, 0, 1),
+                                                  (2, 2, 4, 0, 1), (2, 2, 4, 0, 3)])
+def test_first_run_captured(eng, orc, kind, ndim, T, vec, rest):  # noqa: F811
+    """A plan's first run under stream capture, its last pass shorter than T: nothing may be
+    allocated there, so the plan's own kernel runs the few steps.  Replayed, then run plainly."""
+    import torch
+    nx, ny, nz = (485, 61, 1) if ndim == 2 else (131, 67, 35)
+    w = synth.make_vdiff(nx, ny, seed=8900 + T + rest) if kind == 2 else \
+        synth.make(kind, ndim, nx, ny, nz, seed=8900 + 7 * T + rest)
+    steps = 2 * T + rest
+    u = torch.from_numpy(w.u0).cuda()
+    p = w.coef if kind == 2 else w.power
+    p = None if p is None else torch.from_numpy(p).cuda()
+    coef = None if kind == 2 else w.coef
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    out = torch.full_like(u, float("nan"))
+    with torch.cuda.stream(s):
+        plan = eng.Plan(kind, ndim, nx, ny, nz, force_T=T, force_vec=vec, resident=-1)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            plan.run(u, out, coef, steps, power=p)
+        graph.replay()
+        s.synchronize()
+        g = out.cpu().numpy()
+        out.fill_(float("nan"))
+        plan.run(u, out, coef, steps, power=p)
+        plan.sync()
+    assert plan.info()["T"] == T
+    plan.close()
+    o = orc.run_vdiff2d(w.u0, w.coef, steps) if kind == 2 else orc.run(kind, w.u0, w.coef, steps, w.power)
+    assert max_rel(g, o) <= TOL
+    assert max_rel(out.cpu().numpy(), o) <= TOL
