@@ -49,8 +49,15 @@ constexpr int ATA = 4;                                                // fused a
 // (a tensor-map copy's innermost coordinate) stays on a 16-byte boundary
 constexpr int AHX = (ATA + 3) / 4 * 4;
 constexpr int ACX = AX - 2 * AHX, ACY = AY - 2 * ATA;                // compute block
-// tile origin x = tx * ACX - AHX: a multiple of 4 floats for every tile (an unaligned innermost
-// coordinate of a tensor-map copy is an illegal instruction)
+// Tiles start at x = tx * ACX, y = ty * ACY; a tile on the grid's edge needs no halo there and its
+// compute block reaches the edge, so that a grid takes as few tiles as it can: 2048^2 17 x 85 in
+// 5 rounds of two blocks per SM (with halos beyond the edges as well: 18 x 86, a sixth round for
+// 28 blocks).  x origins are multiples of 4 floats (an unaligned innermost coordinate of a
+// tensor-map copy is an illegal instruction).
+constexpr int adj_tiles(int n, int c, int h)
+{
+    return n <= c + 2 * h ? 1 : (n - 2 * h + c - 1) / c;
+}
 static_assert(AHX % 4 == 0 && ACX % 4 == 0 && AHX >= ATA, "tile origins on 16-byte boundaries");
 constexpr int NG = 5;                                                 // coefficients
 constexpr int NPART = 3 * NG;                                         // (hi, lo, |.|) x 5
@@ -220,7 +227,10 @@ __device__ __forceinline__ void adj_block(const AdjPass &a, int lane, int ly0, i
     }
     // gradient terms of the compute block (its cells and their neighbours are in the tile);
     // the condition is warp-uniform, so every lane takes part in the shuffles below
-    const bool rows_any = ly0 + 3 >= ATA && ly0 < ATA + ACY;
+    // own cells: the tile without its halos, which an edge tile has only inside the grid
+    const int oy0 = EDGE && y0 == 0 ? 0 : ATA, oy1 = EDGE && y0 + AY >= a.ny ? AY : ATA + ACY;
+    const int ox0 = EDGE && x0 == 0 ? 0 : AHX, ox1 = EDGE && x0 + AX >= a.nx ? AX : AHX + ACX;
+    const bool rows_any = ly0 + 3 >= oy0 && ly0 < oy1;
     if (rows_any) {
         float U[6][4];
 #pragma unroll
@@ -238,7 +248,7 @@ __device__ __forceinline__ void adj_block(const AdjPass &a, int lane, int ly0, i
 #pragma unroll
         for (int r = 0; r < 4; r++) {
             const int ly = ly0 + r, gy = y0 + ly;
-            if (ly < ATA || ly >= ATA + ACY) continue;
+            if (ly < oy0 || ly >= oy1) continue;
             if (EDGE && gy >= a.ny) continue;
             float pr[4] = {0.f, 0.f, 0.f, 0.f};
             if (KIND == ST_THERMAL) {
@@ -248,7 +258,7 @@ __device__ __forceinline__ void adj_block(const AdjPass &a, int lane, int ly0, i
 #pragma unroll
             for (int j = 0; j < 4; j++) {
                 const int lx = lx0 + j, gx = x0 + lx;
-                if (lx < AHX || lx >= AHX + ACX) continue;
+                if (lx < ox0 || lx >= ox1) continue;
                 if (EDGE && gx >= a.nx) continue;
                 const float uc = U[r + 1][j];
                 float uwj = j > 0 ? U[r + 1][j - 1] : uw[r];
@@ -290,7 +300,9 @@ __global__ void __launch_bounds__(ANT, 2) k_adj2d(const AdjPass a, const __grid_
     __shared__ __align__(8) uint64_t bars[2 + ATA];   // lambda, power, state tiles 0 .. ATA-1
     const int tid = threadIdx.x;
     const int tx = blockIdx.x % a.ntx, ty = blockIdx.x / a.ntx;
-    const int x0 = tx * ACX - AHX, y0 = ty * ACY - ATA;
+    const int x0 = tx * ACX, y0 = ty * ACY;
+    const int oy0 = ty == 0 ? 0 : ATA, oy1 = y0 + AY >= a.ny ? AY : ATA + ACY;   // own cells
+    const int ox0 = tx == 0 ? 0 : AHX, ox1 = x0 + AX >= a.nx ? AX : AHX + ACX;
     const bool tma = a.use_tma != 0;
     const uint32_t b0 = sm32(&bars[0]);
     // block-uniform: the whole tile is in the grid and no cell of it lies on the grid's edge
@@ -299,8 +311,11 @@ __global__ void __launch_bounds__(ANT, 2) k_adj2d(const AdjPass a, const __grid_
     // every copy of the tile is requested at once (lambda, power and the state tile of each
     // fused step, each on its own barrier, used once): the steps then wait only for their own
     // state tile, and one block keeps the whole tile's bytes in flight
-    const auto drain = [&](int j0) {   // after a failed wait: let the copies in flight land
-        for (int j = j0; j < a.nsteps; j++) (void)bar_wait(b0 + 8u * (2 + j), 0);
+    bool ok = true;
+    const auto drain = [&]() {   // after a failed wait: let the copies in flight land
+        (void)bar_wait(b0, 0);
+        if (KIND == ST_THERMAL) (void)bar_wait(b0 + 8u, 0);
+        for (int j = 0; j < a.nsteps; j++) (void)bar_wait(b0 + 8u * (2 + j), 0);
     };
     if (tma) {
         if (tid == 0) {
@@ -319,17 +334,8 @@ __global__ void __launch_bounds__(ANT, 2) k_adj2d(const AdjPass a, const __grid_
             }
         }
         __syncthreads();   // barriers initialised before anyone polls them
-        bool ok = bar_wait(b0, 0);
+        ok = bar_wait(b0, 0);
         if (KIND == ST_THERMAL) ok = bar_wait(b0 + 8u, 0) && ok;
-        if (__syncthreads_or(!ok)) {
-            if (tid == 0) {
-                atomicExch(a.err, 1);
-                (void)bar_wait(b0, 0);
-                if (KIND == ST_THERMAL) (void)bar_wait(b0 + 8u, 0);
-                drain(0);
-            }
-            return;
-        }
     } else {
 #pragma unroll
         for (int q = 0; q < ACPT; q++) {
@@ -352,16 +358,8 @@ __global__ void __launch_bounds__(ANT, 2) k_adj2d(const AdjPass a, const __grid_
     for (int j = 0; j < a.nsteps; j++) {
         const float *u = a.states + (long long)(a.k_hi - j) * a.n;   // u_t, t = t_hi - 1 - j
         const float *ut = ubuf + j * AX * AY;                        // its tile (staged path)
-        if (tma) {
-            const bool ok = bar_wait(b0 + 8u * (2 + j), 0);
-            if (__syncthreads_or(!ok)) {
-                if (tid == 0) {
-                    atomicExch(a.err, 1);
-                    drain(j);
-                }
-                return;
-            }
-        }
+        // every thread waits for itself; that a wait gave up is seen at the step's one barrier
+        if (tma) ok = bar_wait(b0 + 8u * (2 + j), 0) && ok;
         if (interior) {
             adj_block<KIND, ABS, false>(a, lane, ly0, x0, y0, cur, nxt, ut, ptile, hi, ab, pacc);
         } else if (tma) {
@@ -388,25 +386,16 @@ __global__ void __launch_bounds__(ANT, 2) k_adj2d(const AdjPass a, const __grid_
                 r = __fmaf_rn(a.ws, ln, r);
                 r = __fmaf_rn(a.wn, ls, r);
                 nxt[idx] = in ? r : 0.f;
-                const bool own = in && lx >= AHX && lx < AHX + ACX && ly >= ATA && ly < ATA + ACY;
+                const bool own = in && lx >= ox0 && lx < ox1 && ly >= oy0 && ly < oy1;
                 if (own) {
                     float g[NG];
-                    if (tma) {
-                        // own cells are ATA >= 1 cells inside the tile; clamp at the domain edges
-                        const int dw = gx > 0 ? 1 : 0, de = gx < a.nx - 1 ? 1 : 0;
-                        const int dn = gy > 0 ? AX : 0, dsn = gy < a.ny - 1 ? AX : 0;
-                        const float p = KIND == ST_THERMAL ? ptile[idx] : 0.f;
-                        dfdtheta<KIND>(a, ut[idx], ut[idx - dw], ut[idx + de], ut[idx + dsn],
-                                       ut[idx - dn], p, g);
-                    } else {
-                        const long long o = (long long)gy * a.nx;
-                        const int xw = gx > 0 ? gx - 1 : 0, xe = gx < a.nx - 1 ? gx + 1 : a.nx - 1;
-                        const long long on = (long long)(gy > 0 ? gy - 1 : 0) * a.nx;
-                        const long long os = (long long)(gy < a.ny - 1 ? gy + 1 : a.ny - 1) * a.nx;
-                        const float p = KIND == ST_THERMAL ? __ldg(a.pw + o + gx) : 0.f;
-                        dfdtheta<KIND>(a, __ldg(u + o + gx), __ldg(u + o + xw), __ldg(u + o + xe),
-                                       __ldg(u + os + gx), __ldg(u + on + gx), p, g);
-                    }
+                    const long long o = (long long)gy * a.nx;
+                    const int xw = gx > 0 ? gx - 1 : 0, xe = gx < a.nx - 1 ? gx + 1 : a.nx - 1;
+                    const long long on = (long long)(gy > 0 ? gy - 1 : 0) * a.nx;
+                    const long long os = (long long)(gy < a.ny - 1 ? gy + 1 : a.ny - 1) * a.nx;
+                    const float p = KIND == ST_THERMAL ? __ldg(a.pw + o + gx) : 0.f;
+                    dfdtheta<KIND>(a, __ldg(u + o + gx), __ldg(u + o + xw), __ldg(u + o + xe),
+                                   __ldg(u + os + gx), __ldg(u + on + gx), p, g);
 #pragma unroll
                     for (int m = 0; m < NG; m++) {
                         hi[m] = __fmaf_rn(l, g[m], hi[m]);
@@ -416,7 +405,13 @@ __global__ void __launch_bounds__(ANT, 2) k_adj2d(const AdjPass a, const __grid_
                 }
             }
         }
-        __syncthreads();
+        if (__syncthreads_or(!ok)) {
+            if (tid == 0) {
+                atomicExch(a.err, 1);
+                drain();
+            }
+            return;
+        }
         float *t = cur;
         cur = nxt;
         nxt = t;
@@ -426,8 +421,7 @@ __global__ void __launch_bounds__(ANT, 2) k_adj2d(const AdjPass a, const __grid_
     for (int c = 0; c < ACPT; c++) {
         const int lx = lx0 + (c & 3), ly = ly0 + (c >> 2), idx = ly * AX + lx;
         const int gx = x0 + lx, gy = y0 + ly;
-        const bool own = gx < a.nx && gy < a.ny && lx >= AHX && lx < AHX + ACX && ly >= ATA &&
-                         ly < ATA + ACY;
+        const bool own = gx < a.nx && gy < a.ny && lx >= ox0 && lx < ox1 && ly >= oy0 && ly < oy1;
         if (own) {
             const long long o = (long long)gy * a.nx + gx;
             a.lam_out[o] = cur[idx];
@@ -437,49 +431,77 @@ __global__ void __launch_bounds__(ANT, 2) k_adj2d(const AdjPass a, const __grid_
 
     // block reduction of the (hi, lo) pairs and the magnitudes, fixed order
     const int wid = tid >> 5;
+    // The five pair trees of a warp share its lanes: a level halves the values a lane keeps (3, 2,
+    // then 1) as well as the lanes per value, 8 pair additions instead of 5 x 5, in the same tree.
+    // (After three levels lane L holds coefficient 3 b16 + 2 b8 + b4 of its bits, if there is one.)
+    const bool u16 = lane & 16, u8 = lane & 8, u4 = lane & 4;
+    float vh[3], vl[3];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1)
+    for (int q = 0; q < 3; q++) {
+        const float up = q < 2 ? hi[3 + q] : 0.f;
+        vh[q] = u16 ? up : hi[q];
+        vl[q] = 0.f;
+        add_pair(vh[q], vl[q], __shfl_xor_sync(0xffffffffu, u16 ? hi[q] : up, 16), 0.f);
+    }
 #pragma unroll
-        for (int m = 0; m < NG; m++) {
-            const float bh = __shfl_down_sync(0xffffffffu, hi[m], off);
-            const float bl = __shfl_down_sync(0xffffffffu, lo[m], off);
-            const float bb = __shfl_down_sync(0xffffffffu, ab[m], off);
-            add_pair(hi[m], lo[m], bh, bl);
-            ab[m] = __fadd_rn(ab[m], bb);
-        }
-    if (lane == 0)
+    for (int q = 0; q < 2; q++) {
+        const float uh = q < 1 ? vh[2] : 0.f, ul = q < 1 ? vl[2] : 0.f;
+        const float bh = __shfl_xor_sync(0xffffffffu, u8 ? vh[q] : uh, 8);
+        const float bl = __shfl_xor_sync(0xffffffffu, u8 ? vl[q] : ul, 8);
+        vh[q] = u8 ? uh : vh[q];
+        vl[q] = u8 ? ul : vl[q];
+        add_pair(vh[q], vl[q], bh, bl);
+    }
+    {
+        const float bh = __shfl_xor_sync(0xffffffffu, u4 ? vh[0] : vh[1], 4);
+        const float bl = __shfl_xor_sync(0xffffffffu, u4 ? vl[0] : vl[1], 4);
+        vh[0] = u4 ? vh[1] : vh[0];
+        vl[0] = u4 ? vl[1] : vl[0];
+        add_pair(vh[0], vl[0], bh, bl);
+    }
 #pragma unroll
-        for (int m = 0; m < NG; m++) {
-            red[wid][3 * m + 0] = hi[m];
-            red[wid][3 * m + 1] = lo[m];
-            red[wid][3 * m + 2] = ab[m];
-        }
-    __syncthreads();
-    if (wid == 0) {
-        constexpr int NWP = ANT / 32;
-#pragma unroll
-        for (int m = 0; m < NG; m++) {
-            hi[m] = lane < NWP ? red[lane][3 * m + 0] : 0.f;
-            lo[m] = lane < NWP ? red[lane][3 * m + 1] : 0.f;
-            ab[m] = lane < NWP ? red[lane][3 * m + 2] : 0.f;
-        }
+    for (int off = 2; off > 0; off >>= 1) {
+        const float bh = __shfl_xor_sync(0xffffffffu, vh[0], off);
+        const float bl = __shfl_xor_sync(0xffffffffu, vl[0], off);
+        add_pair(vh[0], vl[0], bh, bl);
+    }
+    const int half = (u8 ? 2 : 0) + (u4 ? 1 : 0), mine = (u16 ? 3 : 0) + half;
+    if ((lane & 3) == 0 && half < (u16 ? 2 : 3)) {
+        red[wid][3 * mine + 0] = vh[0];
+        red[wid][3 * mine + 1] = vl[0];
+    }
+    if (ABS) {
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1)
 #pragma unroll
-            for (int m = 0; m < NG; m++) {
-                const float bh = __shfl_down_sync(0xffffffffu, hi[m], off);
-                const float bl = __shfl_down_sync(0xffffffffu, lo[m], off);
-                const float bb = __shfl_down_sync(0xffffffffu, ab[m], off);
-                add_pair(hi[m], lo[m], bh, bl);
-                ab[m] = __fadd_rn(ab[m], bb);
-            }
+            for (int m = 0; m < NG; m++) ab[m] = __fadd_rn(ab[m], __shfl_down_sync(0xffffffffu, ab[m], off));
         if (lane == 0)
 #pragma unroll
-            for (int m = 0; m < NG; m++) {
-                a.partials[(long long)blockIdx.x * NPART + 3 * m + 0] = hi[m];
-                a.partials[(long long)blockIdx.x * NPART + 3 * m + 1] = lo[m];
-                a.partials[(long long)blockIdx.x * NPART + 3 * m + 2] = ab[m];
-            }
+            for (int m = 0; m < NG; m++) red[wid][3 * m + 2] = ab[m];
+    }
+    __syncthreads();
+    // the 8 warps' triples: 8 lanes of the first two warps per coefficient
+    constexpr int NWP = ANT / 32;
+    static_assert(NWP == 8 && NG <= 8, "8 lanes per coefficient, two warps");
+    if (wid < 2) {
+        const int m = 4 * wid + lane / NWP;
+        const bool have = m < NG;
+        float h = have ? red[lane % NWP][3 * m + 0] : 0.f;
+        float l = have ? red[lane % NWP][3 * m + 1] : 0.f;
+        float b = have && ABS ? red[lane % NWP][3 * m + 2] : 0.f;
+#pragma unroll
+        for (int off = NWP / 2; off > 0; off >>= 1) {
+            const float bh = __shfl_down_sync(0xffffffffu, h, off, NWP);
+            const float bl = __shfl_down_sync(0xffffffffu, l, off, NWP);
+            add_pair(h, l, bh, bl);
+            if (ABS) b = __fadd_rn(b, __shfl_down_sync(0xffffffffu, b, off, NWP));
+        }
+        if (have && lane % NWP == 0) {
+            float *out = a.partials + (long long)blockIdx.x * NPART + 3 * m;
+            out[0] = h;
+            out[1] = l;
+            out[2] = b;
+        }
     }
 }
 
@@ -586,7 +608,7 @@ int stencil_adjoint_create(stencil_adjoint *out, int kind, int nx, int ny, int s
     a->ckpt = std::min(ckpt, std::max(steps, 1));
     a->nseg = steps > 0 ? (steps + a->ckpt - 1) / a->ckpt : 0;
     a->stream = static_cast<cudaStream_t>(stream);
-    const int ntx = (nx + ACX - 1) / ACX, nty = (ny + ACY - 1) / ACY;
+    const int ntx = adj_tiles(nx, ACX, AHX), nty = adj_tiles(ny, ACY, ATA);
     a->blocks = (long long)ntx * nty;
     for (int sg = 0; sg < a->nseg; sg++) {
         const int len = std::min(steps, (sg + 1) * a->ckpt) - sg * a->ckpt;
@@ -700,7 +722,7 @@ int stencil_adjoint_backward(stencil_adjoint a, const float *grad_out, const flo
     p.gpw = grad_power;
     p.nx = a->nx;
     p.ny = a->ny;
-    p.ntx = (a->nx + ACX - 1) / ACX;
+    p.ntx = adj_tiles(a->nx, ACX, AHX);
     for (int i = 0; i < 5; i++) p.k[i] = a->coef[i];
     if (a->kind == ST_DIFFUSION) {
         p.wc = a->coef[0];
