@@ -217,12 +217,11 @@ double model_gcells_2d(const stencil_desc &d, int sms, const Cand2D &k, int bps,
 // budget is the smallest for which everything is dealt out (bisection).
 // Measured on GB300 against contiguous ranges of (column, plane) units balanced the same way,
 // where neighbours run at unrelated planes: see prepare3 and segments_2d.
-struct Seg3 { int col, z0, z1, pad; };
+struct Seg3 { int col, z0, z1, block; };
 
 // speed: each block's share of the budget (empty: all alike)
 bool deal_segments(int nz, int slots, double fill, double edge, const std::vector<double> &w,
-                   const std::vector<double> &speed, double budget,
-                   std::vector<std::vector<Seg3>> *out)
+                   const std::vector<double> &speed, double budget, std::vector<Seg3> *out)
 {
     struct Rest { int col, z0; };
     struct Block { double left; int id; };
@@ -233,7 +232,7 @@ bool deal_segments(int nz, int slots, double fill, double edge, const std::vecto
     std::vector<Block> blocks(slots), spare;
     for (int b = 0; b < slots; b++) blocks[b] = Block{speed.empty() ? budget : budget * speed[b], b};
     size_t head = 0;
-    if (out) out->assign(slots, {});
+    if (out) out->clear();
     while (!rest.empty()) {
         if (head == blocks.size()) {
             if (spare.empty()) return false;
@@ -265,7 +264,7 @@ bool deal_segments(int nz, int slots, double fill, double edge, const std::vecto
             // a segment that reaches the end pays `edge` too; one that cannot, leaves a rest
             if (take == h && take > 1 && fixed + edge + h * w[q.col] > b.left)
                 take = std::max(1, std::min(h - 1, (int)std::floor((b.left - fixed - edge) / w[q.col])));
-            if (out) (*out)[b.id].push_back(Seg3{q.col, q.z0, q.z0 + take, 0});
+            if (out) out->push_back(Seg3{q.col, q.z0, q.z0 + take, b.id});
             if (take < h) {
                 next.push_back(Rest{q.col, q.z0 + take});
             } else {
@@ -281,11 +280,10 @@ bool deal_segments(int nz, int slots, double fill, double edge, const std::vecto
     return true;
 }
 
-// The smallest budget for `slots` blocks (within tol), and with out != nullptr the segments per
-// block.
+// The smallest budget for `slots` blocks (within tol), and with out != nullptr the segments in
+// the order in which they were dealt.
 double best_segments(int nz, int slots, double fill, double edge, const std::vector<double> &w,
-                     const std::vector<double> &speed, double tol,
-                     std::vector<std::vector<Seg3>> *out)
+                     const std::vector<double> &speed, double tol, std::vector<Seg3> *out)
 {
     double total = 0.0;
     for (double x : w) total += x * nz;
@@ -501,15 +499,24 @@ int kernel_T_for(const stencil_plan_s *p, int want)
 }
 
 // Dealt segments on the device, [first segment of each block | segments], and their block count.
-int upload_segments(std::vector<std::vector<Seg3>> &segs, int *ctas, int *seg_off, void **dev)
+int upload_segments(const std::vector<Seg3> &segs, int *ctas, int *seg_off, void **dev)
 {
-    while (segs.size() > 1 && segs.back().empty()) segs.pop_back();
-    *ctas = (int)segs.size();
-    std::vector<int> host((segs.size() + 1 + 3) / 4 * 4, 0);   // (the segments start 16-byte aligned)
-    *seg_off = (int)host.size();
-    for (size_t i = 0; i < segs.size(); i++) host[i + 1] = host[i] + (int)segs[i].size();
-    for (const auto &v : segs)
-        for (const Seg3 &q : v) host.insert(host.end(), {q.col, q.z0, q.z1, 0});
+    int n = 1;
+    for (const Seg3 &q : segs) n = std::max(n, q.block + 1);
+    *ctas = n;
+    *seg_off = (n + 1 + 3) / 4 * 4;   // (the segments start 16-byte aligned)
+    std::vector<int> host(*seg_off + 4 * segs.size(), 0), at(n, 0);
+    for (const Seg3 &q : segs) at[q.block]++;
+    for (int b = 0; b < n; b++) {
+        host[b + 1] = host[b] + at[b];
+        at[b] = host[b];
+    }
+    for (const Seg3 &q : segs) {
+        int *h = host.data() + *seg_off + 4 * (size_t)at[q.block]++;
+        h[0] = q.col;
+        h[1] = q.z0;
+        h[2] = q.z1;
+    }
     cudaError_t e = stn::dev_malloc(dev, host.size() * sizeof(int));
     if (e == cudaSuccess) e = cudaMemcpy(*dev, host.data(), host.size() * sizeof(int), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
@@ -535,7 +542,7 @@ int segments_2d(stencil_plan_s *p, int bps, int halo, int V, PassCfg2D *c)
     std::vector<double> w(c->ntx, 1.0);
     w.front() = kEdge2;
     w.back() = p->d.nx % V == 0 ? kEdge2 : kGhost2;
-    std::vector<std::vector<Seg3>> segs;
+    std::vector<Seg3> segs;
     // A scheduler issues from its oldest ready warp first, so of the one-warp blocks that share one
     // the first to arrive (blocks arrive in order, one per SM and round, four rounds per warp
     // rank) runs ahead of the others (equal shares, 12000^2 diffusion: the first half of the
@@ -676,7 +683,7 @@ int prepare3(stencil_plan_s *p, int Tk, PassCfg3D **out)
             // diffusion pass 491 -> 302 MB); a plan of few columns is spread over more blocks
             // (187 x 141 x 93 diffusion x 30: 427 -> 242 us)
             const std::vector<double> w = column_weights(c.ntx, c.nty);
-            std::vector<std::vector<Seg3>> segs;
+            std::vector<Seg3> segs;
             best_segments(p->d.nz, p->sms * bps, 3.0 * Tk - 1, 0.0, w, {}, 0.25, &segs);
             const int rc = upload_segments(segs, &c.ctas, &c.seg_off, &c.segs);
             if (rc == ST_ERR_OOM && Tk < p->T) {
