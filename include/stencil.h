@@ -129,7 +129,9 @@ typedef struct {
 } stencil_plan_info;
 
 /* Create a plan for one problem shape on the current CUDA device.  Allocates one grid-sized
- * ping-pong scratch buffer (Sec. 2.1's second buffer) and keeps it until destroy.
+ * ping-pong scratch buffer (Sec. 2.1's second buffer; two where a contracted plan's nx is not a
+ * multiple of 4 and memory allows, so that the inner passes run on aligned rows) and keeps it
+ * until destroy.
  * out: receives the plan (NULL on failure).
  * Errors: ST_ERR_INVALID_ARG (bad desc), ST_ERR_UNSUPPORTED (e.g. a storage type or forced
  * parameter set with no compiled kernel), ST_ERR_OOM, ST_ERR_CUDA. */

@@ -1439,18 +1439,29 @@ static int plan_create(stencil_plan *out, const stencil_desc *desc)
     }
     // Contracted first-order plans on rows that are no whole 16-byte chunks (nx not a multiple of
     // 4): the passes between the first and the last run between two padded scratch grids, so that
-    // only those two touch the caller's rows (staged and stored cell by cell)
+    // only those two touch the caller's rows (staged and stored cell by cell).  The second grid
+    // (and the padded power map of 3D Hotspot) is taken where memory is no concern: up to 16 GiB,
+    // and if there is none left the passes alternate between one scratch grid and the output.
     const bool two = rc == ST_OK && d.nx % 4 != 0 && !d.exact && !p->res && !p->stor &&
-                     (d.rad <= 1 || p->star_rows) && (d.ndim == 2 || p->alg3);
+                     (d.rad <= 1 || p->star_rows) && (d.ndim == 2 || p->alg3) &&
+                     p->scratch_bytes <= (size_t)16 << 30;
     if (rc == ST_OK && p->scratch_bytes) {
         e = stn::dev_malloc(&p->scratch, p->scratch_bytes);
-        if (e == cudaSuccess && two) e = stn::dev_malloc(&p->scratch2, p->scratch_bytes);
-        if (e != cudaSuccess) rc = map_cuda(e);
-        if (two) p->scratch_bytes *= 2;
-    }
-    if (two && rc == ST_OK && d.ndim == 3 && d.kind == ST_THERMAL) {
-        p->ld_src = p->ld_scratch;
-        e = stn::dev_malloc(&p->src, (size_t)p->ld_src * d.ny * d.nz * sizeof(float));
+        if (e == cudaSuccess && two) {
+            const bool pad_pw = d.ndim == 3 && d.kind == ST_THERMAL;
+            e = stn::dev_malloc(&p->scratch2, p->scratch_bytes);
+            if (e == cudaSuccess && pad_pw) e = stn::dev_malloc(&p->src, p->scratch_bytes);
+            if (e == cudaSuccess) {
+                p->scratch_bytes *= 2;
+                if (pad_pw) p->ld_src = p->ld_scratch;
+            } else if (e == cudaErrorMemoryAllocation) {
+                (void)cudaGetLastError();
+                if (p->scratch2) stn::dev_free(p->scratch2);
+                p->scratch2 = nullptr;
+                p->src = nullptr;
+                e = cudaSuccess;
+            }
+        }
         if (e != cudaSuccess) rc = map_cuda(e);
     }
     if (rc == ST_OK && d.ndim == 2 && d.kind == ST_THERMAL && !d.exact && !p->stor) {

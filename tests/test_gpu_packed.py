@@ -111,3 +111,38 @@ def test_first_run_captured(eng, orc, kind, ndim, T, vec, rest):  # noqa: F811
     o = orc.run_vdiff2d(w.u0, w.coef, steps) if kind == 2 else orc.run(kind, w.u0, w.coef, steps, w.power)
     assert max_rel(g, o) <= TOL
     assert max_rel(out.cpu().numpy(), o) <= TOL
+
+
+@pytest.mark.parametrize("kind,ndim", [(0, 2), (1, 2), (0, 3), (1, 3), (2, 2)])
+def test_one_scratch_grid(eng, orc, kind, ndim):  # noqa: F811
+    """Odd widths without memory for the second scratch grid: the plan is created all the same and
+    runs on one (the allocation that fails is injected on the host)."""
+    import torch
+    nx, ny, nz = (485, 61, 1) if ndim == 2 else (131, 67, 35)
+    w = synth.make_vdiff(nx, ny, seed=9100) if kind == 2 else synth.make(kind, ndim, nx, ny, nz, seed=9100 + kind)
+    u = torch.from_numpy(w.u0).cuda()
+    p = w.coef if kind == 2 else w.power
+    p = None if p is None else torch.from_numpy(p).cuda()
+    whole = eng.Plan(kind, ndim, nx, ny, nz, resident=-1)
+    two = whole.info()["scratch_bytes"]
+    whole.close()
+    ran = 0
+    for n in range(1, 12):
+        assert eng.lib.stencil_debug_fail_alloc(n) == eng.ST_OK
+        try:
+            plan = eng.Plan(kind, ndim, nx, ny, nz, resident=-1)
+        except eng.StencilError as e:
+            assert e.code == eng.ST_ERR_OOM
+            continue
+        finally:
+            eng.lib.stencil_debug_fail_alloc(0)
+        if plan.info()["scratch_bytes"] * 2 == two:
+            for steps in (9, 16):
+                out = plan.run(u, torch.full_like(u, float("nan")), None if kind == 2 else w.coef, steps, power=p)
+                plan.sync()
+                o = orc.run_vdiff2d(w.u0, w.coef, steps) if kind == 2 else \
+                    orc.run(kind, w.u0, w.coef, steps, w.power)
+                assert max_rel(out.cpu().numpy(), o) <= TOL, steps
+            ran += 1
+        plan.close()
+    assert ran >= 1
