@@ -157,7 +157,8 @@ int stencil_batch_create_ex(stencil_batch *out, const stencil_batch_grid *grids,
     // launch never reads data it wrote itself except from the padded scratch, through
     // 16-byte copies that bypass L1 (a row of the caller's grids may be unaligned and would be
     // read through L1, which other SMs' writes do not update), and a grid run in place needs no
-    // final copy.
+    // final copy - unless it takes a single pass, whose tiles would overwrite cells that their
+    // neighbours have yet to read: that pass writes the scratch, and copy items bring it back.
     B->passes.assign(count, 0);
     B->scratch.assign(2 * count, nullptr);
     B->src.assign(count, nullptr);
@@ -167,7 +168,8 @@ int stencil_batch_create_ex(stencil_batch *out, const stencil_batch_grid *grids,
         B->passes[g] = q.steps > 0 ? (q.steps + T - 1) / T : 0;
         B->ld_scratch[g] = ((long long)q.nx + 31) / 32 * 32;
         const size_t sb = (size_t)B->ld_scratch[g] * q.ny * sizeof(float);
-        if (B->passes[g] > 1) e = stn::dev_malloc(&B->scratch[2 * g], sb);
+        if (B->passes[g] > 1 || (B->passes[g] == 1 && q.grid_in == q.grid_out))
+            e = stn::dev_malloc(&B->scratch[2 * g], sb);
         if (e == cudaSuccess && B->passes[g] > 2) e = stn::dev_malloc(&B->scratch[2 * g + 1], sb);
         if (e == cudaSuccess && B->passes[g] > 0 && q.kind == ST_THERMAL)   // padded rows too
             e = stn::dev_malloc(&B->src[g], sb);
@@ -205,12 +207,14 @@ int stencil_batch_create_ex(stencil_batch *out, const stencil_batch_grid *grids,
         G.copy_to = static_cast<float *>(q.grid_out);
         maxp = std::max(maxp, P);
         const int last = P > 0 ? q.steps - T * (P - 1) : 0;
+        const bool back = P == 1 && q.grid_in == q.grid_out;
         for (int p = 0; p < P; p++) {
             Pass2D a = {};
             a.in = p == 0 ? static_cast<const float *>(q.grid_in) : B->scratch[2 * g + (p - 1) % 2];
             a.ld_in = p == 0 ? q.nx : B->ld_scratch[g];
-            a.out = p == P - 1 ? static_cast<float *>(q.grid_out) : B->scratch[2 * g + p % 2];
-            a.ld_out = p == P - 1 ? q.nx : B->ld_scratch[g];
+            const bool to_out = p == P - 1 && !back;
+            a.out = to_out ? static_cast<float *>(q.grid_out) : B->scratch[2 * g + p % 2];
+            a.ld_out = to_out ? q.nx : B->ld_scratch[g];
             a.pw = B->src[g];   // Hotspot: sdc*(p + amb*Rz), rebuilt at every replay
             a.ld_pw = B->ld_scratch[g];
             a.nx = q.nx;
@@ -230,6 +234,10 @@ int stencil_batch_create_ex(stencil_batch *out, const stencil_batch_grid *grids,
         if (P == 0 && q.grid_in != q.grid_out) {
             G.copy_from = static_cast<const float *>(q.grid_in);   // no steps: a plain copy
             G.ld_copy = q.nx;
+        }
+        if (back) {
+            G.copy_from = B->scratch[2 * g];
+            G.ld_copy = B->ld_scratch[g];
         }
     }
     // Two queues, one per kind.  Within a queue each grid's pass chain is placed on a timeline

@@ -119,6 +119,8 @@ __global__ void __launch_bounds__(32, 12) k_tb2f_queue(const QueueBatch2D q)
             else if (w.k > 0 && w.k < G.P)
                 ok = q_wait(q.done + G.done_off, G.ntx, max(w.tx - 1, 0), min(w.tx + 1, G.ntx - 1),
                             s0, s1, w.k, q.status, deadline);
+            else if (w.k > 0)   // copy of a single pass run in place: its rows' readers and writers
+                ok = q_wait(q.done + G.done_off, G.ntx, 0, G.ntx - 1, s0, s1, w.k, q.status, deadline);
         }
         if (!ok) break;
         const int r0 = w.seg * q.L, r1 = min(G.ny, r0 + q.L);

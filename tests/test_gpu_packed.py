@@ -146,3 +146,22 @@ def test_one_scratch_grid(eng, orc, kind, ndim):  # noqa: F811
             ran += 1
         plan.close()
     assert ran >= 1
+
+
+@pytest.mark.parametrize("rows", [0, 16, 40])
+def test_batch_one_pass_in_place(eng, orc, rows):  # noqa: F811
+    """Grids of a batch run in place by a single pass (at most 8 steps), cut into several tiles."""
+    import torch
+    items, refs = [], []
+    for i, (nx, ny, steps) in enumerate([(2048, 31, 4), (700, 500, 8), (301, 900, 1), (113, 17, 5), (1, 50, 3)]):
+        w = synth.make(i % 2, 2, nx, ny, steps=steps, seed=9200 + i)
+        u = torch.from_numpy(w.u0).cuda()
+        items.append({"kind": w.kind, "nx": nx, "ny": ny, "steps": steps, "grid_in": u, "grid_out": u,
+                      "power": None if w.power is None else torch.from_numpy(w.power).cuda(), "coeffs": w.coef})
+        refs.append(orc.run(w.kind, w.u0, w.coef, steps, w.power))
+    b = eng.Batch(items, rows_per_item=rows)
+    b.run()
+    b.sync()
+    b.close()
+    for it, o in zip(items, refs):
+        assert max_rel(it["grid_out"].cpu().numpy(), o) <= TOL, (it["nx"], it["ny"], it["steps"])
