@@ -49,10 +49,17 @@ struct stencil_batch_s {
 
 namespace {
 
-// rows per queue item (L), by default: each item streams 2T rows more than it stores, and
-// fewer, longer items leave more blocks waiting for their neighbours (measured on the 64-grid
-// workload, T = 8: 1921 / 1973 / 1980 / 1978 / 1961 GCell/s for L = 128 / 160 / 192 / 224 / 256)
-constexpr int kRows = 192;
+// Rows per queue item (L), by default.  An item streams 2T rows more than it stores, so long
+// items do less work; but a grid's passes follow one another, and where a step of the longest
+// chain has fewer items than there are warps, an item's length sets the time.  So L is seven
+// tenths of the rows that each resident warp gets per step of the longest chain, within [16, 192].
+// Measured on GB300, T = 8, ms at L = 48 / 64 / 96 / 128 / 160 / 192 / 224: 64 grids (281 rows per
+// warp and step) 15.80 / 14.63 / 13.33 / 12.73 / 12.38 / 12.23 / 12.41, 40 grids (140 rows) 8.04 /
+// 7.46 / 6.89 / 7.07 / 7.95 / 9.00 / 9.80, 16 grids (77 rows) 4.50 / 4.43 / 4.69 / 5.62 / 6.55 /
+// 7.31, 20 grids (51 rows) 3.38 / 3.79 / 4.71 / 5.79 / 6.78 / 7.65 (32: 3.47); one 1000 x 1000 grid
+// 1.13 / 1.27 / 1.50 / 1.77 at L = 16 / 24 / 32 / 48, 4.50 at 192.
+constexpr int kRowsMin = 16, kRowsMax = 192;
+constexpr double kRowsShare = 0.7;
 constexpr long long kWaitNs = 1000LL * 1000 * 1000;   // 1 s: a wait of a healthy batch is far shorter
 // (T, V) of the compiled queue kernel: 4 cells per lane (64-grid workload: 12.8 ms; with 8, 255
 // registers and two warps per scheduler, 14.1 ms at its best L; T = 12 with 4 cells, 255
@@ -63,6 +70,19 @@ int status(cudaError_t e)
 {
     if (e == cudaSuccess) return ST_OK;
     return e == cudaErrorMemoryAllocation ? ST_ERR_OOM : ST_ERR_CUDA;
+}
+
+int default_rows(const std::vector<stencil_batch_grid> &grids, int T, int cx, int warps)
+{
+    double rows = 0.0;   // rows of tile columns, all passes
+    int longest = 1;
+    for (const stencil_batch_grid &q : grids) {
+        const int passes = (int)(((long long)q.steps + T - 1) / T);
+        rows += (double)((q.nx + cx - 1) / cx) * q.ny * passes;
+        longest = std::max(longest, passes);
+    }
+    const double l = kRowsShare * rows / ((double)longest * warps);
+    return std::max(kRowsMin, ((int)std::min<double>(kRowsMax, l) + 7) / 8 * 8);
 }
 
 size_t align256(size_t n) { return (n + 255) / 256 * 256; }
@@ -84,7 +104,7 @@ int stencil_batch_create_ex(stencil_batch *out, const stencil_batch_grid *grids,
     *out = nullptr;
     if (!grids || count < 1 || rows_per_item < 0 || force_T < 0 || force_vec < 0)
         return ST_ERR_INVALID_ARG;
-    const int L = rows_per_item ? rows_per_item : kRows;
+    int L = rows_per_item;
     for (int g = 0; g < count; g++) {
         const stencil_batch_grid &q = grids[g];
         if ((q.kind != ST_DIFFUSION && q.kind != ST_THERMAL) || q.nx < 1 || q.ny < 1 ||
@@ -124,19 +144,21 @@ int stencil_batch_create_ex(stencil_batch *out, const stencil_batch_grid *grids,
     *B->h_status = 0;
 
     // one (T, V) for the launch: the compiled candidate with the least predicted total time
-    int bps = 0;
+    int bps = 0, use_rows = 0;
     {
         double best = -1.0;
         for (const auto &tv : kCand) {
             int b = 0;
             if ((force_T && tv[0] != force_T) || (force_vec && tv[1] != force_vec)) continue;
-            if (tv[0] > L) continue;   // an item's halo rows must come from its neighbours
+            if (L && tv[0] > L) continue;   // an item's halo rows must come from its neighbours
             if (tb2q_prepare(tv[0], tv[1], &b) != cudaSuccess || b < 1) continue;
+            const int cols = 32 * tv[1] - 2 * ((tv[0] + tv[1] - 1) / tv[1] * tv[1]);
+            const int rows = L ? L : default_rows(B->grid, tv[0], cols, b * B->sms);
             double t = 0.0;
             for (const stencil_batch_grid &q : B->grid) {
                 if (q.steps <= 0) continue;
                 const double m = batch_model_gcells(q.kind, q.nx, q.ny, q.steps, B->sms, tv[0],
-                                                    tv[1], b, L);
+                                                    tv[1], b, rows);
                 t += (double)q.nx * q.ny * q.steps / std::max(m, 1e-9);
             }
             if (best < 0 || t < best) {
@@ -144,11 +166,13 @@ int stencil_batch_create_ex(stencil_batch *out, const stencil_batch_grid *grids,
                 B->qT = tv[0];
                 B->qV = tv[1];
                 bps = b;
+                use_rows = rows;
             }
         }
         (void)cudaGetLastError();
         if (best < 0) rc = ST_ERR_UNSUPPORTED;
     }
+    L = use_rows;
     const int T = B->qT, V = B->qV;
     const int halo = rc == ST_OK ? (T + V - 1) / V * V : 0, cx = 32 * V - 2 * halo;   // tb2d_halo
 

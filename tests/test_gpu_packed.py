@@ -165,3 +165,27 @@ def test_batch_one_pass_in_place(eng, orc, rows):  # noqa: F811
     b.close()
     for it, o in zip(items, refs):
         assert max_rel(it["grid_out"].cpu().numpy(), o) <= TOL, (it["nx"], it["ny"], it["steps"])
+
+
+@pytest.mark.parametrize("count,lo,hi", [(1, 30, 60), (3, 100, 300), (9, 20, 500), (5, 900, 1500)])
+def test_batch_rows(eng, orc, count, lo, hi):  # noqa: F811
+    """Batches of few grids take short queue items (16 rows up); heights around an item's."""
+    import torch
+    rng = np.random.default_rng(count)
+    items, refs = [], []
+    for i in range(count):
+        nx, ny = int(rng.integers(lo, hi)), int(rng.integers(lo, hi))
+        if i % 3 == 2:
+            ny = ny // 16 * 16 + i % 2
+        w = synth.make(i % 2, 2, nx, ny, steps=int(rng.integers(1, 40)), seed=9300 + i)
+        u = torch.from_numpy(w.u0).cuda()
+        items.append({"kind": w.kind, "nx": nx, "ny": ny, "steps": w.steps, "grid_in": u,
+                      "grid_out": torch.full_like(u, float("nan")),
+                      "power": None if w.power is None else torch.from_numpy(w.power).cuda(), "coeffs": w.coef})
+        refs.append(orc.run(w.kind, w.u0, w.coef, w.steps, w.power))
+    b = eng.Batch(items)
+    b.run()
+    b.sync()
+    b.close()
+    for it, o in zip(items, refs):
+        assert max_rel(it["grid_out"].cpu().numpy(), o) <= TOL, (it["nx"], it["ny"], it["steps"])
