@@ -88,7 +88,8 @@ struct stencil_plan_s {
     float *res_xg = nullptr;      // two exchange grids, rows of res_ld floats
     long long res_ld = 0;
     int *res_flags = nullptr;     // per block: epochs published (grow across runs)
-    int res_epoch = 0;            // epoch base of the next run
+    int res_epoch = 0;            // epoch base of the next run: no counter is above it
+    int res_captured = 0;         // most epochs of a captured run: what a replay leaves counted
     long long res_wait_ns = 1000000000LL;
     int res_hold_block = -1, res_hold_epoch = -1;
 };
@@ -562,7 +563,11 @@ int segments_2d(stencil_plan_s *p, int bps, int halo, int V, PassCfg2D *c)
 bool capturing(const stencil_plan_s *p)
 {
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    return cudaStreamIsCapturing(p->stream, &st) == cudaSuccess && st != cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(p->stream, &st) != cudaSuccess) {   // (the null stream while another captures)
+        (void)cudaGetLastError();
+        return false;
+    }
+    return st != cudaStreamCaptureStatusNone;
 }
 
 int prepare2(stencil_plan_s *p, int Tk, PassCfg2D **out)
@@ -811,8 +816,10 @@ int run_pass2(stencil_plan_s *p, const float *src, long long lds, float *dst, lo
     return map_cuda(e);
 }
 
-// a run of a resident-tile plan: one cooperative launch (after zeroing the blocks' epoch
-// counters)
+// a run of a resident-tile plan: one cooperative launch.  The blocks' epoch counters grow from run
+// to run (each run starts at a base that no counter is above), so a run launched now needs no reset.
+// A captured run does: every replay gets the arguments of the capture, so its graph zeroes the
+// counters and counts from 0, and later plain runs start above what a replay may have left.
 int run_resident(stencil_plan_s *p, const float *in, float *out, const float *pw, const float *k,
                  int steps)
 {
@@ -840,14 +847,17 @@ int run_resident(stencil_plan_s *p, const float *in, float *out, const float *pw
     a.xplane = p->res_ld * d.ny;
     a.ld_x = p->res_ld;
     if (epochs > 1) {
-        if (p->res_epoch > 0x7fffffff - epochs) {
-            // the counters would overflow: start again from zero
+        const bool cap = capturing(p);
+        if (cap) p->res_captured = std::max(p->res_captured, epochs);
+        if (cap || p->res_epoch > 0x7fffffff - epochs) {   // (or the counters would overflow)
             e = cudaMemsetAsync(p->res_flags, 0, (size_t)p->res_nbx * p->res_nby * sizeof(int), p->stream);
             if (e != cudaSuccess) return map_cuda(e);
-            p->res_epoch = 0;
+            a.epoch0 = 0;
+            p->res_epoch = std::max(cap ? p->res_epoch : epochs, p->res_captured);
+        } else {
+            a.epoch0 = p->res_epoch;
+            p->res_epoch += epochs;
         }
-        a.epoch0 = p->res_epoch;
-        p->res_epoch += epochs;
     }
     a.flags = p->res_flags;
     a.status = p->err;

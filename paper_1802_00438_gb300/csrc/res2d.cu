@@ -26,7 +26,8 @@
 // Exchange: two grid-sized buffers alternate by epoch parity.  A block overwrites its cells of
 // epoch e (with epoch e+2) only after its neighbours have published epoch e+1, which they do
 // only after reading epoch e.  flags[b] counts the epochs block b has published (growing
-// across runs from the plan's epoch0, so no reset between runs): after the block's barrier
+// across runs from the plan's epoch0, so no reset between runs; a captured run counts from 0 after
+// a reset that its graph repeats): after the block's barrier
 // one thread publishes it with a release store, and a waiting block polls its (up to 8)
 // neighbours' counters with acquire loads before its barrier and its reads -- no further
 // fences (measured on GB300: an exchange with a gpu-scope fence on either side took ~5 us,

@@ -153,3 +153,50 @@ def test_bounded_wait_runs_out(eng, orc):
     plan.close()
     o = orc.run(1, w.u0, w.coef, 13, w.power)
     assert max_rel(out.cpu().numpy(), o) <= TOL
+
+
+@pytest.mark.parametrize("kind,exact,resident", [(0, False, 0), (0, False, 1), (1, False, 1), (0, True, 1),
+                                                 (1, True, 1)])
+def test_captured_run_replays(eng, orc, kind, exact, resident):
+    """A run captured into a graph exchanges halos in every replay, not only in the first: replays
+    with other inputs, plain runs (shorter and longer) before and between them."""
+    import torch
+    nx, ny = (256, 192) if resident == 0 else (517, 263)
+    ws = [synth.make(kind, 2, nx, ny, seed=7600 + kind + 10 * i) for i in range(3)]
+    coef, power = ws[0].coef, ws[0].power
+    p = None if power is None else torch.from_numpy(power).cuda()
+    s = torch.cuda.Stream()
+    u = torch.from_numpy(ws[0].u0).cuda()
+    out = torch.empty_like(u)
+    s.wait_stream(torch.cuda.current_stream())
+
+    def check(w, steps, what):
+        s.synchronize()
+        g, o = out.cpu().numpy(), orc.run(kind, w.u0, coef, steps, power)
+        assert np.array_equal(g, o) if exact else max_rel(g, o) <= TOL, (what, max_rel(g, o))
+
+    with torch.cuda.stream(s):
+        plan = eng.Plan(kind, 2, nx, ny, exact=exact, resident=resident, force_T=4 if resident else 0)
+        info = plan.info()
+        assert info["resident"] == 1
+        steps = 3 * info["T"] + 1
+        graph, longer = torch.cuda.CUDAGraph(), torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            plan.run(u, out, coef, steps, power=p)
+        with torch.cuda.graph(longer, stream=s):
+            plan.run(u, out, coef, 3 * steps, power=p)
+
+        def plain(n):
+            plan.run(u, out, coef, n, power=p)
+
+        for i, (act, n) in enumerate([(lambda: plain(steps), steps), (graph.replay, steps), (graph.replay, steps),
+                                      (longer.replay, 3 * steps), (lambda: plain(2 * steps), 2 * steps),
+                                      (graph.replay, steps), (lambda: plain(steps), steps),
+                                      (longer.replay, 3 * steps), (graph.replay, steps)]):
+            w = ws[i % 3]
+            u.copy_(torch.from_numpy(w.u0))
+            out.fill_(float("nan"))
+            act()
+            check(w, n, i)
+    plan.sync()
+    plan.close()
