@@ -669,7 +669,7 @@ int stencil_adjoint_create(stencil_adjoint *out, int kind, int nx, int ny, int s
             e = stn::dev_malloc(&a->partials, sizeof(float) * NPART *
                                              (size_t)(a->blocks * a->passes + ADJ_SUM_BLOCKS));
         if (e == cudaSuccess) e = stn::dev_malloc(&a->err, sizeof(int));
-        if (e == cudaSuccess) e = cudaMemset(a->err, 0, sizeof(int));
+        if (e == cudaSuccess) e = stn::dev_zero(a->err, sizeof(int), a->stream);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_adj2d<ST_DIFFUSION, false>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -853,7 +853,7 @@ int stencil_adjoint_sync(stencil_adjoint a)
     e = cudaMemcpy(&flag, a->err, sizeof(int), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return status(e);
     if (flag) {
-        (void)cudaMemset(a->err, 0, sizeof(int));
+        (void)stn::dev_zero(a->err, sizeof(int), a->stream);
         return ST_ERR_TIMEOUT;
     }
     return ST_OK;

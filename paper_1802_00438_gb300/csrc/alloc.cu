@@ -5,6 +5,8 @@
 //     that the call that made it reports ST_ERR_OOM and releases what it had allocated;
 //   - stencil_debug_live_allocs() counts what the library holds, so a test sees a leak as a
 //     count that does not return to its starting value.
+// Uploads and zeroing at creation go through dev_upload / dev_zero, which order them before the
+// work that reads them.
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -29,7 +31,32 @@ bool injected_failure()
     return false;
 }
 
+// a stream under capture: the work would become part of the graph instead of being done now
+bool captured(cudaStream_t st)
+{
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &s) != cudaSuccess) {   // (the null stream while another captures)
+        (void)cudaGetLastError();
+        return false;
+    }
+    return s != cudaStreamCaptureStatusNone;
+}
+
 }  // namespace
+
+cudaError_t dev_upload(void *dst, const void *src, size_t bytes, cudaStream_t st)
+{
+    if (!captured(st)) return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st);
+    const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, cudaStreamLegacy);
+    return e == cudaSuccess ? cudaStreamSynchronize(cudaStreamLegacy) : e;
+}
+
+cudaError_t dev_zero(void *dst, size_t bytes, cudaStream_t st)
+{
+    if (!captured(st)) return cudaMemsetAsync(dst, 0, bytes, st);
+    const cudaError_t e = cudaMemsetAsync(dst, 0, bytes, cudaStreamLegacy);
+    return e == cudaSuccess ? cudaStreamSynchronize(cudaStreamLegacy) : e;
+}
 
 cudaError_t dev_malloc(void **p, size_t bytes)
 {

@@ -500,7 +500,7 @@ int kernel_T_for(const stencil_plan_s *p, int want)
 }
 
 // Dealt segments on the device, [first segment of each block | segments], and their block count.
-int upload_segments(const std::vector<Seg3> &segs, int *ctas, int *seg_off, void **dev)
+int upload_segments(const std::vector<Seg3> &segs, int *ctas, int *seg_off, void **dev, cudaStream_t st)
 {
     int n = 1;
     for (const Seg3 &q : segs) n = std::max(n, q.block + 1);
@@ -519,7 +519,7 @@ int upload_segments(const std::vector<Seg3> &segs, int *ctas, int *seg_off, void
         h[2] = q.z1;
     }
     cudaError_t e = stn::dev_malloc(dev, host.size() * sizeof(int));
-    if (e == cudaSuccess) e = cudaMemcpy(*dev, host.data(), host.size() * sizeof(int), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = stn::dev_upload(*dev, host.data(), host.size() * sizeof(int), st);
     if (e != cudaSuccess) {
         if (*dev) stn::dev_free(*dev);
         *dev = nullptr;
@@ -554,7 +554,7 @@ int segments_2d(stencil_plan_s *p, int bps, int halo, int V, PassCfg2D *c)
     for (int b = 0; b < slots && ranks > 1; b++)
         speed[b] = 1.0 + kAhead2 * (1.0 - 2.0 * (b / p->sms / 4) / (ranks - 1));
     best_segments(p->d.ny, slots, kFill2 * halo, (V == 8 ? kTop2V8 : kTop2V4) * halo, w, speed, 0.5, &segs);
-    return upload_segments(segs, &c->ctas, &c->seg_off, &c->segs);
+    return upload_segments(segs, &c->ctas, &c->seg_off, &c->segs, p->stream);
 }
 
 // A remainder pass (fewer steps than the plan's T) gets its own shorter kernel, whose segments are
@@ -690,7 +690,7 @@ int prepare3(stencil_plan_s *p, int Tk, PassCfg3D **out)
             const std::vector<double> w = column_weights(c.ntx, c.nty);
             std::vector<Seg3> segs;
             best_segments(p->d.nz, p->sms * bps, 3.0 * Tk - 1, 0.0, w, {}, 0.25, &segs);
-            const int rc = upload_segments(segs, &c.ctas, &c.seg_off, &c.segs);
+            const int rc = upload_segments(segs, &c.ctas, &c.seg_off, &c.segs, p->stream);
             if (rc == ST_ERR_OOM && Tk < p->T) {
                 (void)cudaGetLastError();
                 return prepare3(p, p->T, out);
@@ -1484,7 +1484,7 @@ static int plan_create(stencil_plan *out, const stencil_desc *desc)
         const size_t fb = (size_t)p->res_nbx * p->res_nby * sizeof(int);
         e = stn::dev_malloc(&p->res_xg, (size_t)2 * p->res_ld * d.ny * sizeof(float));
         if (e == cudaSuccess) e = stn::dev_malloc(&p->res_flags, fb);
-        if (e == cudaSuccess) e = cudaMemset(p->res_flags, 0, fb);
+        if (e == cudaSuccess) e = stn::dev_zero(p->res_flags, fb, p->stream);
         if (e != cudaSuccess) rc = map_cuda(e);
     }
     if (rc == ST_OK && !p->res && !d.exact && !p->stor && d.rad <= 1 && d.kind != ST_DIFFUSION_VAR) {
@@ -1500,7 +1500,7 @@ static int plan_create(stencil_plan *out, const stencil_desc *desc)
     }
     if (rc == ST_OK) {
         e = stn::dev_malloc(&p->err, sizeof(int));
-        if (e == cudaSuccess) e = cudaMemset(p->err, 0, sizeof(int));
+        if (e == cudaSuccess) e = stn::dev_zero(p->err, sizeof(int), p->stream);
         if (e != cudaSuccess) rc = map_cuda(e);
     }
     if (rc != ST_OK) {
@@ -1684,7 +1684,7 @@ int stencil_plan_sync(stencil_plan p)
         e = cudaMemcpy(&flag, p->err, sizeof(int), cudaMemcpyDeviceToHost);
         if (e != cudaSuccess) return map_cuda(e);
         if (flag) {
-            (void)cudaMemset(p->err, 0, sizeof(int));
+            (void)stn::dev_zero(p->err, sizeof(int), p->stream);
             return ST_ERR_TIMEOUT;
         }
     }

@@ -349,7 +349,7 @@ int stencil_batch_create_ex(stencil_batch *out, const stencil_batch_grid *grids,
         if (!desc.empty()) std::memcpy(host.data() + o_desc, desc.data(), desc.size() * sizeof(Pass2D));
         QueueCtl ctl = {kWaitNs, -1, 0};
         std::memcpy(host.data() + o_ctl, &ctl, sizeof(ctl));
-        e = cudaMemcpy(B->dev, host.data(), o_cnt, cudaMemcpyHostToDevice);
+        e = stn::dev_upload(B->dev, host.data(), o_cnt, B->stream);
         if (e != cudaSuccess) rc = status(e);
         B->ctl = reinterpret_cast<QueueCtl *>(d + o_ctl);
         int *cnt = reinterpret_cast<int *>(d + o_cnt);

@@ -288,6 +288,13 @@ cudaError_t host_malloc(T **p, size_t bytes)
     return host_malloc(reinterpret_cast<void **>(p), bytes);
 }
 
+// What the library writes to its own buffers outside a run - tables, zeroed flags - ordered before
+// everything that is launched on `st` afterwards; `src` may be released on return (pageable memory
+// is staged before the call returns).  A copy on the null stream is not: it may return before the
+// transfer has landed, and a non-blocking stream does not wait for the null stream.
+cudaError_t dev_upload(void *dst, const void *src, size_t bytes, cudaStream_t st);
+cudaError_t dev_zero(void *dst, size_t bytes, cudaStream_t st);
+
 int res2d_rows_per_thread();
 int res2d_max_warps(int kind, int exact, int vx);
 size_t res2d_smem(int vx, int nw);
