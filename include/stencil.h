@@ -117,7 +117,10 @@ typedef struct {
     int warps;          /* warps per block */
     int ctas;           /* blocks per launch (a multiple of the SM count where possible) */
     int sms;            /* streaming multiprocessors on the plan's device */
-    long long scratch_bytes;   /* device scratch the plan owns */
+    long long scratch_bytes;   /* the plan's ping-pong grids: one or two scratch grids, or the two
+                                  exchange grids of resident tiles (0: 16-bit plans).  On top come
+                                  the Hotspot source map (2D) or padded power map (3D, nx not a
+                                  multiple of 4), one grid each, and small tables */
     int exact;          /* as requested */
     int kernel_id;      /* internal kernel family (diagnostics) */
     double model_gcells;   /* the GPU restatement of Eqs. 3-9 with the library's calibration,
@@ -129,9 +132,11 @@ typedef struct {
 } stencil_plan_info;
 
 /* Create a plan for one problem shape on the current CUDA device.  Allocates one grid-sized
- * ping-pong scratch buffer (Sec. 2.1's second buffer; two where a contracted plan's nx is not a
- * multiple of 4 and memory allows, so that the inner passes run on aligned rows) and keeps it
- * until destroy.
+ * ping-pong scratch buffer (Sec. 2.1's second buffer) and keeps it until destroy.  Where a
+ * contracted plan's nx is not a multiple of 4 it takes a second one, so that the inner passes run
+ * on aligned rows, and for 3D Hotspot a copy of the power map with aligned rows: only up to a
+ * quarter of the device memory left free by everything it needs, and a failure to get them is no
+ * error.
  * out: receives the plan (NULL on failure).
  * Errors: ST_ERR_INVALID_ARG (bad desc), ST_ERR_UNSUPPORTED (e.g. a storage type or forced
  * parameter set with no compiled kernel), ST_ERR_OOM, ST_ERR_CUDA. */

@@ -1074,6 +1074,40 @@ int run_pass3(stencil_plan_s *p, const float *src, long long lds, float *dst, lo
     return map_cuda(e);
 }
 
+// Contracted first-order plans on rows that are no whole 16-byte chunks (nx not a multiple of 4):
+// the passes between the first and the last run between two padded scratch grids, so that only
+// those two touch the caller's rows (staged and stored cell by cell).  The second grid (and the
+// padded power map of 3D Hotspot) is taken where memory is no concern: up to 16 GiB a grid and a
+// quarter of what is free once the plan has all it needs.  Otherwise, and if the allocation fails,
+// the passes alternate between one scratch grid and the output.
+int extra_grids(stencil_plan_s *p)
+{
+    const stencil_desc &d = p->d;
+    if (d.nx % 4 == 0 || d.exact || p->res || p->stor || (d.rad > 1 && !p->star_rows) ||
+        (d.ndim == 3 && !p->alg3) || p->scratch_bytes > (size_t)16 << 30)
+        return ST_OK;
+    const bool pad_pw = d.ndim == 3 && d.kind == ST_THERMAL;
+    size_t free_b = 0, total_b = 0;
+    cudaError_t e = cudaMemGetInfo(&free_b, &total_b);
+    if (e != cudaSuccess) return map_cuda(e);
+    if (p->scratch_bytes * (pad_pw ? 2 : 1) > free_b / 4) return ST_OK;
+    float *grid = nullptr, *pw = nullptr;
+    e = stn::dev_malloc(&grid, p->scratch_bytes);
+    if (e == cudaSuccess && pad_pw) e = stn::dev_malloc(&pw, p->scratch_bytes);
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();
+        if (grid) stn::dev_free(grid);
+        return e == cudaErrorMemoryAllocation ? ST_OK : map_cuda(e);
+    }
+    p->scratch2 = grid;
+    p->scratch_bytes *= 2;
+    if (pad_pw) {
+        p->src = pw;
+        p->ld_src = p->ld_scratch;
+    }
+    return ST_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -1351,8 +1385,6 @@ static int plan_create(stencil_plan *out, const stencil_desc *desc)
             if (p->T == 0 || (d.force_T && p->T != d.force_T)) rc = ST_ERR_UNSUPPORTED;
             PassCfg2D *c = nullptr;
             if (rc == ST_OK) rc = prepare2(p, p->T, &c);
-            if (rc == ST_OK && var && !d.exact)   // remainder passes' segments as well
-                for (int ts = 1; ts < p->T && rc == ST_OK; ts++) rc = prepare2(p, kernel_T_for(p, ts), &c);
             if (rc == ST_OK && p->stor) {
                 // coded grids: rows padded to 8 cells (16 bytes), codes per (row, tile column)
                 p->cx = tb2d_tile_width(c->shape) - 2 * tb2d_halo(c->shape);
@@ -1447,31 +1479,8 @@ static int plan_create(stencil_plan *out, const stencil_desc *desc)
         p->ld_scratch = p->alg3 ? ((long long)d.nx + 3) / 4 * 4 : d.nx;
         p->scratch_bytes = (size_t)p->ld_scratch * d.ny * d.nz * sizeof(float);
     }
-    // Contracted first-order plans on rows that are no whole 16-byte chunks (nx not a multiple of
-    // 4): the passes between the first and the last run between two padded scratch grids, so that
-    // only those two touch the caller's rows (staged and stored cell by cell).  The second grid
-    // (and the padded power map of 3D Hotspot) is taken where memory is no concern: up to 16 GiB,
-    // and if there is none left the passes alternate between one scratch grid and the output.
-    const bool two = rc == ST_OK && d.nx % 4 != 0 && !d.exact && !p->res && !p->stor &&
-                     (d.rad <= 1 || p->star_rows) && (d.ndim == 2 || p->alg3) &&
-                     p->scratch_bytes <= (size_t)16 << 30;
     if (rc == ST_OK && p->scratch_bytes) {
         e = stn::dev_malloc(&p->scratch, p->scratch_bytes);
-        if (e == cudaSuccess && two) {
-            const bool pad_pw = d.ndim == 3 && d.kind == ST_THERMAL;
-            e = stn::dev_malloc(&p->scratch2, p->scratch_bytes);
-            if (e == cudaSuccess && pad_pw) e = stn::dev_malloc(&p->src, p->scratch_bytes);
-            if (e == cudaSuccess) {
-                p->scratch_bytes *= 2;
-                if (pad_pw) p->ld_src = p->ld_scratch;
-            } else if (e == cudaErrorMemoryAllocation) {
-                (void)cudaGetLastError();
-                if (p->scratch2) stn::dev_free(p->scratch2);
-                p->scratch2 = nullptr;
-                p->src = nullptr;
-                e = cudaSuccess;
-            }
-        }
         if (e != cudaSuccess) rc = map_cuda(e);
     }
     if (rc == ST_OK && d.ndim == 2 && d.kind == ST_THERMAL && !d.exact && !p->stor) {
@@ -1503,6 +1512,14 @@ static int plan_create(stencil_plan *out, const stencil_desc *desc)
         if (e == cudaSuccess) e = stn::dev_zero(p->err, sizeof(int), p->stream);
         if (e != cudaSuccess) rc = map_cuda(e);
     }
+    // last what the plan can do without: the remainder passes' segments (per-cell coefficients; the
+    // others prepare theirs when they first run one) and the extra grids
+    if (d.kind == ST_DIFFUSION_VAR && !d.exact)
+        for (int ts = 1; ts < p->T && rc == ST_OK; ts++) {
+            PassCfg2D *c = nullptr;
+            rc = prepare2(p, kernel_T_for(p, ts), &c);
+        }
+    if (rc == ST_OK) rc = extra_grids(p);
     if (rc != ST_OK) {
         stencil_plan_destroy(p);
         return rc;
