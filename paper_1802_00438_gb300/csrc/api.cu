@@ -16,6 +16,7 @@
 
 #include "../../include/stencil.h"
 #include "internal.h"
+#include "segments.h"
 
 using namespace stn;
 
@@ -197,108 +198,6 @@ double model_gcells_2d(const stencil_desc &d, int sms, const Cand2D &k, int bps,
     return r.gcells;
 }
 
-// 3D partial-sum kernel: the same restatement.  Issue-equivalent work per computed cell update
-// including halos, by T: 16 / 13.5 / 11.2 / 13 operations (Diffusion, T = 1 .. 4; T = 4 spills
-// registers), 18.6 / 15.7 / 12.9 / 13.7 (Hotspot), at an issue efficiency of 0.61 for one 16-warp
-// block per SM, x1.04 for two 8-warp blocks, x0.80 for 32-warp blocks of 2 x 2 cells (twice the y
-// exchange per cell).  A pass costs 9 us besides (launch, first planes, drain).  Device memory:
-// with the columns streamed in step most halo re-reads hit L2: three tenths of the tile fit's
-// excess reads, at 90 % of the copy bandwidth.  Calibrated on GB300 over 512^3, 512^2 x 256,
-// 256^3, 300 x 200 x 400 and 187 x 141 x 93, both kinds, T = 2 .. 4, 64- and 32-row tiles.
-// Segments of the contracted passes: which planes (2D: rows) of which tile columns each block
-// streams.  A segment costs w[col] per plane plus `fill` planes of pipeline fill, plus `edge` at
-// the first and the last plane of the grid (boundary handling), and the slowest block sets the
-// pass time.
-// The tile columns overlap, so neighbouring columns should be at nearby planes at the same time:
-// then the halo cells a tile reads again (and the partial sectors of its rows) are still in L2.
-// So, level by level: with at least as many blocks as columns left, every column gets one block,
-// all from the same first plane, for as many planes as the budget allows, and what is left of the
-// columns goes to the blocks without work; with fewer blocks than columns, each block takes one
-// whole rest of a column, the costliest first, and goes on with the budget that leaves it.  The
-// budget is the smallest for which everything is dealt out (bisection).
-// Measured on GB300 against contiguous ranges of (column, plane) units balanced the same way,
-// where neighbours run at unrelated planes: see prepare3 and segments_2d.
-struct Seg3 { int col, z0, z1, block; };
-
-// speed: each block's share of the budget (empty: all alike)
-bool deal_segments(int nz, int slots, double fill, double edge, const std::vector<double> &w,
-                   const std::vector<double> &speed, double budget, std::vector<Seg3> *out)
-{
-    struct Rest { int col, z0; };
-    struct Block { double left; int id; };
-    std::vector<Rest> rest(w.size()), next;
-    for (size_t c = 0; c < w.size(); c++) rest[c] = Rest{(int)c, 0};
-    // blocks with work to take, the largest budget first, from `head` on; `spare`: those that have
-    // a segment and budget left, taken up when the others have run out
-    std::vector<Block> blocks(slots), spare;
-    for (int b = 0; b < slots; b++) blocks[b] = Block{speed.empty() ? budget : budget * speed[b], b};
-    size_t head = 0;
-    if (out) out->clear();
-    while (!rest.empty()) {
-        if (head == blocks.size()) {
-            if (spare.empty()) return false;
-            std::sort(spare.begin(), spare.end(), [](const Block &a, const Block &b) {
-                return a.left != b.left ? a.left > b.left : a.id < b.id;
-            });
-            blocks.swap(spare);
-            spare.clear();
-            head = 0;
-        }
-        const size_t avail = blocks.size() - head;
-        const bool whole = rest.size() > avail;   // fewer blocks than columns: whole rests
-        if (whole)
-            std::sort(rest.begin(), rest.end(), [&](const Rest &a, const Rest &b) {
-                const double ca = (nz - a.z0) * w[a.col], cb = (nz - b.z0) * w[b.col];
-                return ca != cb ? ca > cb : a.col < b.col;
-            });
-        next.clear();
-        for (size_t i = 0; i < rest.size(); i++) {
-            const Rest &q = rest[i];
-            if (i >= avail) {
-                next.push_back(q);
-                continue;
-            }
-            Block &b = blocks[head + i];
-            const int h = nz - q.z0;
-            const double fixed = fill + (q.z0 == 0 ? edge : 0.0);
-            int take = std::max(1, (int)std::min<double>(h, std::floor((b.left - fixed) / w[q.col])));
-            // a segment that reaches the end pays `edge` too; one that cannot, leaves a rest
-            if (take == h && take > 1 && fixed + edge + h * w[q.col] > b.left)
-                take = std::max(1, std::min(h - 1, (int)std::floor((b.left - fixed - edge) / w[q.col])));
-            if (out) out->push_back(Seg3{q.col, q.z0, q.z0 + take, b.id});
-            if (take < h) {
-                next.push_back(Rest{q.col, q.z0 + take});
-            } else {
-                b.left -= fixed + edge + take * w[q.col];
-                if (b.left >= fill + 4) spare.push_back(b);
-            }
-        }
-        head += std::min(avail, rest.size());
-        if (whole)
-            std::sort(next.begin(), next.end(), [](const Rest &a, const Rest &b) { return a.col < b.col; });
-        rest.swap(next);
-    }
-    return true;
-}
-
-// The smallest budget for `slots` blocks (within tol), and with out != nullptr the segments in
-// the order in which they were dealt.
-double best_segments(int nz, int slots, double fill, double edge, const std::vector<double> &w,
-                     const std::vector<double> &speed, double tol, std::vector<Seg3> *out)
-{
-    double total = 0.0;
-    for (double x : w) total += x * nz;
-    double lo = std::max(total / slots, fill + 4.0), hi = lo + 3.0 * fill + edge;
-    while (!deal_segments(nz, slots, fill, edge, w, speed, hi, nullptr)) hi *= 1.5;
-    for (int i = 0; i < 40 && hi - lo > tol; i++) {
-        const double mid = 0.5 * (lo + hi);
-        if (deal_segments(nz, slots, fill, edge, w, speed, mid, nullptr)) hi = mid;
-        else lo = mid;
-    }
-    if (out) deal_segments(nz, slots, fill, edge, w, speed, hi, out);
-    return hi;
-}
-
 // relative cost of a plane of each tile column (kWX3, kWY3: see prepare3)
 constexpr double kWX3 = 1.4, kWY3 = 1.2;
 
@@ -314,6 +213,14 @@ std::vector<double> column_weights(int ntx, int nty)
     return w;
 }
 
+// 3D partial-sum kernel: the same restatement.  Issue-equivalent work per computed cell update
+// including halos, by T: 16 / 13.5 / 11.2 / 13 operations (Diffusion, T = 1 .. 4; T = 4 spills
+// registers), 18.6 / 15.7 / 12.9 / 13.7 (Hotspot), at an issue efficiency of 0.61 for one 16-warp
+// block per SM, x1.04 for two 8-warp blocks, x0.80 for 32-warp blocks of 2 x 2 cells (twice the y
+// exchange per cell).  A pass costs 9 us besides (launch, first planes, drain).  Device memory:
+// with the columns streamed in step most halo re-reads hit L2: three tenths of the tile fit's
+// excess reads, at 90 % of the copy bandwidth.  Calibrated on GB300 over 512^3, 512^2 x 256,
+// 256^3, 300 x 200 x 400 and 187 x 141 x 93, both kinds, T = 2 .. 4, 64- and 32-row tiles.
 // `bound`: an upper bound instead, with segments dealt at no loss (no bisection)
 double model_gcells_3d(const stencil_desc &d, int sms, int T, int VX, int VY, int NW,
                        bool bound = false)
@@ -340,9 +247,9 @@ double model_gcells_3d(const stencil_desc &d, int sms, int T, int VX, int VY, in
     const long long slots = (long long)sms * (NW <= 8 ? 2 : 1);
     const double seg_cost =
         bound ? 0.0
-              : best_segments(d.nz, (int)slots, 3.0 * T - 1, 0.0,
-                              column_weights((int)std::ceil(d.nx / cx), (int)std::ceil(d.ny / cy)), {},
-                              0.02 * cols * d.nz / slots + 0.5, nullptr);
+              : SegmentDealer(d.nz, (int)slots, 3.0 * T - 1, 0.0,
+                              column_weights((int)std::ceil(d.nx / cx), (int)std::ceil(d.ny / cy)))
+                    .best(0.02 * cols * d.nz / slots + 0.5, nullptr);
     const double alg = d.kind == ST_DIFFUSION ? 8.0 : 12.0;
     const double read = alg - 4.0;   // field (and power) in; the field out is written once
     m.bytes_per_cell = alg;
@@ -500,19 +407,19 @@ int kernel_T_for(const stencil_plan_s *p, int want)
 }
 
 // Dealt segments on the device, [first segment of each block | segments], and their block count.
-int upload_segments(const std::vector<Seg3> &segs, int *ctas, int *seg_off, void **dev, cudaStream_t st)
+int upload_segments(const std::vector<Segment> &segs, int *ctas, int *seg_off, void **dev, cudaStream_t st)
 {
     int n = 1;
-    for (const Seg3 &q : segs) n = std::max(n, q.block + 1);
+    for (const Segment &q : segs) n = std::max(n, q.block + 1);
     *ctas = n;
     *seg_off = (n + 1 + 3) / 4 * 4;   // (the segments start 16-byte aligned)
     std::vector<int> host(*seg_off + 4 * segs.size(), 0), at(n, 0);
-    for (const Seg3 &q : segs) at[q.block]++;
+    for (const Segment &q : segs) at[q.block]++;
     for (int b = 0; b < n; b++) {
         host[b + 1] = host[b] + at[b];
         at[b] = host[b];
     }
-    for (const Seg3 &q : segs) {
+    for (const Segment &q : segs) {
         int *h = host.data() + *seg_off + 4 * (size_t)at[q.block]++;
         h[0] = q.col;
         h[1] = q.z0;
@@ -528,7 +435,7 @@ int upload_segments(const std::vector<Seg3> &segs, int *ctas, int *seg_off, void
 }
 
 // Segments of a contracted 2D pass: rows of tile columns dealt like the planes of the 3D passes
-// (best_segments), so that neighbouring columns stream the same rows at the same time and share
+// (SegmentDealer), so that neighbouring columns stream the same rows at the same time and share
 // their halo cells, and the partial sectors of their rows, in L2.  A segment's fill is 2T rows of
 // which the idle stages are skipped.  A row of a tile column whose edge lies on a lane boundary
 // (x = 0 always, x = nx-1 when nx is a multiple of the cells per thread) costs kEdge2, one whose
@@ -543,7 +450,7 @@ int segments_2d(stencil_plan_s *p, int bps, int halo, int V, PassCfg2D *c)
     std::vector<double> w(c->ntx, 1.0);
     w.front() = kEdge2;
     w.back() = p->d.nx % V == 0 ? kEdge2 : kGhost2;
-    std::vector<Seg3> segs;
+    std::vector<Segment> segs;
     // A scheduler issues from its oldest ready warp first, so of the one-warp blocks that share one
     // the first to arrive (blocks arrive in order, one per SM and round, four rounds per warp
     // rank) runs ahead of the others (equal shares, 12000^2 diffusion: the first half of the
@@ -553,7 +460,7 @@ int segments_2d(stencil_plan_s *p, int bps, int halo, int V, PassCfg2D *c)
     std::vector<double> speed(slots, 1.0);
     for (int b = 0; b < slots && ranks > 1; b++)
         speed[b] = 1.0 + kAhead2 * (1.0 - 2.0 * (b / p->sms / 4) / (ranks - 1));
-    best_segments(p->d.ny, slots, kFill2 * halo, (V == 8 ? kTop2V8 : kTop2V4) * halo, w, speed, 0.5, &segs);
+    SegmentDealer(p->d.ny, slots, kFill2 * halo, (V == 8 ? kTop2V8 : kTop2V4) * halo, w, speed).best(0.5, &segs);
     return upload_segments(segs, &c->ctas, &c->seg_off, &c->segs, p->stream);
 }
 
@@ -679,7 +586,7 @@ int prepare3(stencil_plan_s *p, int Tk, PassCfg3D **out)
         c.planes_per_cta = (total + ctas - 1) / ctas;
         c.ctas = (int)((total + c.planes_per_cta - 1) / c.planes_per_cta);
         if (p->alg3) {
-            // segments dealt to the blocks (best_segments): a plane of a tile column at the x
+            // segments dealt to the blocks (SegmentDealer): a plane of a tile column at the x
             // edge costs 1.4, at the y edge 1.2 (only they run instances with the clamp fix-ups,
             // and the barrier makes a block wait for its slowest warp; swept 1.0-1.4 on GB300,
             // T = 3: 512^3 diffusion 1188 GCell/s at 1.1 / 1.05, 1318 at 1.4 / 1.2).  Dealt
@@ -687,9 +594,8 @@ int prepare3(stencil_plan_s *p, int Tk, PassCfg3D **out)
             // 940 -> 1044 GCell/s at T = 3, 611 -> 912 at T = 2 (DRAM reads of a 512^2 x 256
             // diffusion pass 491 -> 302 MB); a plan of few columns is spread over more blocks
             // (187 x 141 x 93 diffusion x 30: 427 -> 242 us)
-            const std::vector<double> w = column_weights(c.ntx, c.nty);
-            std::vector<Seg3> segs;
-            best_segments(p->d.nz, p->sms * bps, 3.0 * Tk - 1, 0.0, w, {}, 0.25, &segs);
+            std::vector<Segment> segs;
+            SegmentDealer(p->d.nz, p->sms * bps, 3.0 * Tk - 1, 0.0, column_weights(c.ntx, c.nty)).best(0.25, &segs);
             const int rc = upload_segments(segs, &c.ctas, &c.seg_off, &c.segs, p->stream);
             if (rc == ST_ERR_OOM && Tk < p->T) {
                 (void)cudaGetLastError();

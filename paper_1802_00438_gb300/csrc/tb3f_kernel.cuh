@@ -27,7 +27,7 @@
 //   Clamped z boundaries: at z = 0 the missing plane z-1 is plane 0 itself (Q is started from
 //   d before it is used); on arrival of plane nz-1 a stage completes P with ca*d (the missing
 //   plane nz is plane nz-1), and emits it unchanged one iteration later.
-//   Tile columns of one pass are streamed in step (see best_segments in api.cu).
+//   Tile columns of one pass are streamed in step (see segments.h).
 //   Measured (GB300), kernel with one barrier per stage and scalar arithmetic -> this one: 512^3
 //   diffusion 1022 -> 1330 GCell/s, 512^2 x 256 Hotspot 837 -> 1033, 187 x 141 x 93 diffusion 172
 //   -> 304.  What bounds it now (ncu, 512^2 x 256, T = 3): issue 57 % active with 275
