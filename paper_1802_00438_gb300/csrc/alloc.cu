@@ -31,8 +31,25 @@ bool injected_failure()
     return false;
 }
 
-// a stream under capture: the work would become part of the graph instead of being done now
-bool captured(cudaStream_t st)
+// Do f(stream) on st, or, where st is being captured (the work would become part of the graph), now
+// on a stream of its own, which is waited for.
+template <class F>
+cudaError_t ahead_of(cudaStream_t st, F f)
+{
+    if (!stream_captured(st)) return f(st);
+    const RelaxedCapture relaxed;
+    cudaStream_t own = nullptr;
+    cudaError_t e = cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking);
+    if (e != cudaSuccess) return e;
+    e = f(own);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(own);
+    cudaStreamDestroy(own);
+    return e;
+}
+
+}  // namespace
+
+bool stream_captured(cudaStream_t st)
 {
     cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &s) != cudaSuccess) {   // (the null stream while another captures)
@@ -42,20 +59,14 @@ bool captured(cudaStream_t st)
     return s != cudaStreamCaptureStatusNone;
 }
 
-}  // namespace
-
 cudaError_t dev_upload(void *dst, const void *src, size_t bytes, cudaStream_t st)
 {
-    if (!captured(st)) return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st);
-    const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, cudaStreamLegacy);
-    return e == cudaSuccess ? cudaStreamSynchronize(cudaStreamLegacy) : e;
+    return ahead_of(st, [=](cudaStream_t s) { return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s); });
 }
 
 cudaError_t dev_zero(void *dst, size_t bytes, cudaStream_t st)
 {
-    if (!captured(st)) return cudaMemsetAsync(dst, 0, bytes, st);
-    const cudaError_t e = cudaMemsetAsync(dst, 0, bytes, cudaStreamLegacy);
-    return e == cudaSuccess ? cudaStreamSynchronize(cudaStreamLegacy) : e;
+    return ahead_of(st, [=](cudaStream_t s) { return cudaMemsetAsync(dst, 0, bytes, s); });
 }
 
 cudaError_t dev_malloc(void **p, size_t bytes)

@@ -465,18 +465,8 @@ int segments_2d(stencil_plan_s *p, int bps, int halo, int V, PassCfg2D *c)
 }
 
 // A remainder pass (fewer steps than the plan's T) gets its own shorter kernel, whose segments are
-// allocated on its first use.  Where that cannot be done - the stream is being captured, or no
-// memory is left - the plan's own kernel runs the fewer steps instead.
-bool capturing(const stencil_plan_s *p)
-{
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(p->stream, &st) != cudaSuccess) {   // (the null stream while another captures)
-        (void)cudaGetLastError();
-        return false;
-    }
-    return st != cudaStreamCaptureStatusNone;
-}
-
+// dealt and uploaded on its first use, under stream capture too (the graph then holds that kernel).
+// Where no memory is left for them, the plan's own kernel runs the fewer steps instead.
 int prepare2(stencil_plan_s *p, int Tk, PassCfg2D **out)
 {
     if ((int)p->cfg2.size() <= Tk) p->cfg2.resize(Tk + 1);
@@ -484,7 +474,7 @@ int prepare2(stencil_plan_s *p, int Tk, PassCfg2D **out)
     if (!c.ready) {
         c.shape = Shape2D{p->d.kind, p->d.exact ? 1 : 0, Tk, p->V, p->W, shape_stor(p)};
         if (!tb2d_available(c.shape)) return ST_ERR_UNSUPPORTED;
-        if (Tk < p->T && tb2d_segments(c.shape) && capturing(p)) return prepare2(p, p->T, out);
+        const stn::RelaxedCapture relaxed;
         int bps = 0;
         cudaError_t e = tb2d_prepare(c.shape, &bps);
         if (e != cudaSuccess) return map_cuda(e);
@@ -569,7 +559,7 @@ int prepare3(stencil_plan_s *p, int Tk, PassCfg3D **out)
     if (!c.ready) {
         c.shape = Shape3D{p->d.kind, p->d.exact ? 1 : 0, Tk, p->VY, p->NW, p->alg3, p->VX3};
         if (!tb3d_available(c.shape)) return ST_ERR_UNSUPPORTED;
-        if (Tk < p->T && p->alg3 && capturing(p)) return prepare3(p, p->T, out);
+        const stn::RelaxedCapture relaxed;
         int bps = 0;
         cudaError_t e = tb3d_prepare(c.shape, &bps);
         if (e != cudaSuccess) return map_cuda(e);
@@ -753,7 +743,7 @@ int run_resident(stencil_plan_s *p, const float *in, float *out, const float *pw
     a.xplane = p->res_ld * d.ny;
     a.ld_x = p->res_ld;
     if (epochs > 1) {
-        const bool cap = capturing(p);
+        const bool cap = stn::stream_captured(p->stream);
         if (cap) p->res_captured = std::max(p->res_captured, epochs);
         if (cap || p->res_epoch > 0x7fffffff - epochs) {   // (or the counters would overflow)
             e = cudaMemsetAsync(p->res_flags, 0, (size_t)p->res_nbx * p->res_nby * sizeof(int), p->stream);

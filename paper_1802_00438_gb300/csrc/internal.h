@@ -292,8 +292,24 @@ cudaError_t host_malloc(T **p, size_t bytes)
 // everything that is launched on `st` afterwards; `src` may be released on return (pageable memory
 // is staged before the call returns).  A copy on the null stream is not: it may return before the
 // transfer has landed, and a non-blocking stream does not wait for the null stream.
+// Where `st` is being captured they are done at once, not by the graph.
 cudaError_t dev_upload(void *dst, const void *src, size_t bytes, cudaStream_t st);
 cudaError_t dev_zero(void *dst, size_t bytes, cudaStream_t st);
+
+bool stream_captured(cudaStream_t st);
+
+// While one lives, the thread may allocate although a stream (this one or another thread's) is being
+// captured: the capture takes no part in it.
+class RelaxedCapture {
+public:
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode_); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode_); }
+    RelaxedCapture(const RelaxedCapture &) = delete;
+    RelaxedCapture &operator=(const RelaxedCapture &) = delete;
+
+private:
+    cudaStreamCaptureMode mode_ = cudaStreamCaptureModeRelaxed;
+};
 
 int res2d_rows_per_thread();
 int res2d_max_warps(int kind, int exact, int vx);
