@@ -305,6 +305,8 @@ struct ResGeom {
     double t = 0.0;   // predicted seconds for 1000 steps
 };
 
+constexpr long long kMaxBlocksSM = 32, kMaxWarpsSM = 64;   // what one SM (compute capability 10.x) holds
+
 double res_time(const stencil_desc &d, int sms, const ResGeom &g, int steps)
 {
     const int VY = res2d_rows_per_thread();
@@ -331,15 +333,18 @@ bool res_geometry(const stencil_desc &d, int sms, int T, int vx, ResGeom *out)
     if (cw < 1) return false;
     const int nbx = (d.nx + cw - 1) / cw;
     if (nbx > 1 && cw < hx) return false;   // a halo must not reach past the next block
+    const int ch_max = maxw * VY - 2 * hy;   // rows a block can hold besides its halos
+    if (ch_max < 1) return false;
     std::vector<int> bps(maxw + 1, 0);
     bool found = false;
     ResGeom best;
-    for (int nby = 1; nby <= d.ny; nby++) {
+    for (int nby = (d.ny + ch_max - 1) / ch_max; nby <= d.ny; nby++) {
         const int ch = (d.ny + nby - 1) / nby;
         if (nby > 1 && ch < hy) break;
+        if ((long long)nbx * nby > sms * kMaxBlocksSM) break;   // more than the device can hold
         if ((long long)(nby - 1) * ch >= d.ny) continue;   // the last block would be empty
         const int nw = (ch + 2 * hy + VY - 1) / VY;
-        if (nw > maxw) continue;
+        if ((long long)nbx * nby * nw > sms * kMaxWarpsSM) continue;
         if (!bps[nw]) {
             int b = 0;
             if (res2d_occupancy(kind, d.exact, vx, nw, &b) != cudaSuccess) {
@@ -539,12 +544,18 @@ int prepare_star2f(stencil_plan_s *p, int Tk, PassCfg2D **out)
     if ((int)p->cfg2.size() <= Tk) p->cfg2.resize(Tk + 1);
     PassCfg2D &c = p->cfg2[Tk];
     if (!c.ready) {
+        const stn::RelaxedCapture relaxed;
         int bps = 0;
         const cudaError_t e = star2f_prepare(Tk, &bps);
         if (e != cudaSuccess) return map_cuda(e);
         if (bps < 1) return ST_ERR_UNSUPPORTED;
+        c.shape.T = Tk;
         c.ntx = (p->d.nx + star2f_compute_width() - 1) / star2f_compute_width();
         const int rc = segments_2d(p, bps, 2 * Tk, 8, &c);
+        if (rc == ST_ERR_OOM && Tk < p->T) {
+            (void)cudaGetLastError();
+            return prepare_star2f(p, p->T, out);
+        }
         if (rc != ST_OK) return rc;
         c.ready = true;
     }
@@ -884,7 +895,7 @@ int run_pass_star2f(stencil_plan_s *p, const float *src, long long lds, float *d
         if (rc != ST_OK) return rc;
     }
     cudaError_t e = record(p, true);
-    if (e == cudaSuccess) e = star2f_launch(tsteps <= 1 ? 1 : tsteps <= 2 ? 2 : 4, a, ks, p->stream);
+    if (e == cudaSuccess) e = star2f_launch(c->shape.T, a, ks, p->stream);
     if (e == cudaSuccess) e = record(p, false);
     return map_cuda(e);
 }
@@ -1166,11 +1177,10 @@ static int plan_create(stencil_plan *out, const stencil_desc *desc)
         if (d.rad == 2 && !d.exact && !d.force_bx && !d.force_by && !d.force_vec &&
             (T == 1 || T == 2 || T == 4)) {
             PassCfg2D *c = nullptr;
-            for (int t = T; t >= 1 && rc == ST_OK; t /= 2)   // remainder passes' segments as well
-                rc = prepare_star2f(p, t, &c);
+            p->T = T;
+            rc = prepare_star2f(p, T, &c);
             if (rc == ST_OK) {
                 p->star_rows = 1;
-                p->T = T;
                 p->ld_scratch = ((long long)d.nx + 31) / 32 * 32;
                 p->scratch_bytes = (size_t)p->ld_scratch * d.ny * sizeof(float);
             }
@@ -1279,8 +1289,18 @@ static int plan_create(stencil_plan *out, const stencil_desc *desc)
                 (void)cudaGetLastError();
             }
             if (p->T == 0 || (d.force_T && p->T != d.force_T)) rc = ST_ERR_UNSUPPORTED;
+            if (res && d.resident == 0 && rc == ST_OK && !d.exact) {
+                // contracted: resident tiles only where the model rates them above the passes
+                // (exact plans: always when the grid fits; the exact passes have no calibration)
+                int bps = 0;
+                const Shape2D sh{d.kind, 0, p->T, p->V, p->W, d.kind == ST_THERMAL ? STOR_SRC : 0};
+                if (tb2d_prepare(sh, &bps) == cudaSuccess && bps > 0 &&
+                    model_gcells_2d(d, p->sms, Cand2D{p->T, p->V, p->W}, bps, 1000) >= res_g)
+                    res = false;
+                (void)cudaGetLastError();
+            }
             PassCfg2D *c = nullptr;
-            if (rc == ST_OK) rc = prepare2(p, p->T, &c);
+            if (rc == ST_OK && !res) rc = prepare2(p, p->T, &c);
             if (rc == ST_OK && p->stor) {
                 // coded grids: rows padded to 8 cells (16 bytes), codes per (row, tile column)
                 p->cx = tb2d_tile_width(c->shape) - 2 * tb2d_halo(c->shape);
@@ -1298,20 +1318,10 @@ static int plan_create(stencil_plan *out, const stencil_desc *desc)
                     if (e != cudaSuccess) rc = map_cuda(e);
                 }
                 p->scratch_bytes = 0;   // no float32 scratch: the coded grids take its place
-            } else if (rc == ST_OK) {
+            } else if (rc == ST_OK && !res) {
                 p->ld_scratch = ((long long)d.nx + 31) / 32 * 32;
                 p->scratch_bytes = (size_t)p->ld_scratch * d.ny * sizeof(float);
             }
-        }
-        if (res && d.resident == 0 && rc == ST_OK && !d.exact) {
-            // contracted: resident tiles only where the model rates them above the passes
-            // (exact plans: always when the grid fits; the exact passes have no calibration)
-            int bps = 0;
-            const Shape2D sh{d.kind, 0, p->T, p->V, p->W, d.kind == ST_THERMAL ? STOR_SRC : 0};
-            if (tb2d_prepare(sh, &bps) == cudaSuccess && bps > 0 &&
-                model_gcells_2d(d, p->sms, Cand2D{p->T, p->V, p->W}, bps, 1000) >= res_g)
-                res = false;
-            (void)cudaGetLastError();
         }
         if (res && rc == ST_OK) {
             p->res = 1;
@@ -1340,21 +1350,31 @@ static int plan_create(stencil_plan *out, const stencil_desc *desc)
             // nothing forced, contracted: the compiled partial-sum (tile, T) the calibrated
             // model rates best
             const int shapes[][3] = {{64, 64, 8}, {64, 32, 8}, {128, 32, 8}, {64, 64, 4}};
-            double best = -1.0;
+            // (the rating of one deals its segments, so the most promising come first and the search
+            // ends where the upper bound of the next is no better)
+            struct Cand3 { double bound; int bx, by, cells, t; };
+            std::vector<Cand3> cands;
             for (const auto &sh : shapes)
                 for (int t : {3, 2, 4, 1}) {
                     const int vx = sh[0] / 32, vy = sh[2] / vx, nw = sh[1] / vy;
-                    if (!tb3d_available(Shape3D{d.kind, 0, t, vy, nw, 1, vx})) continue;
-                    if (model_gcells_3d(d, p->sms, t, vx, vy, nw, true) <= best) continue;
-                    const double g = model_gcells_3d(d, p->sms, t, vx, vy, nw);
-                    if (g > best) {
-                        best = g;
-                        bx = sh[0];
-                        by = sh[1];
-                        cells = sh[2];
-                        model_T = t;
-                    }
+                    if (tb3d_available(Shape3D{d.kind, 0, t, vy, nw, 1, vx}))
+                        cands.push_back({model_gcells_3d(d, p->sms, t, vx, vy, nw, true), sh[0], sh[1], sh[2], t});
                 }
+            std::stable_sort(cands.begin(), cands.end(), [](const Cand3 &a, const Cand3 &b) { return a.bound > b.bound; });
+            double best = -1.0;
+            for (const Cand3 &k : cands) {
+                if (k.bound <= best) break;
+                const int vx = k.bx / 32, vy = k.cells / vx;
+                const double g = model_gcells_3d(d, p->sms, k.t, vx, vy, k.by / vy);
+                if (g > best) {
+                    best = g;
+                    bx = k.bx;
+                    by = k.by;
+                    cells = k.cells;
+                    model_T = k.t;
+                }
+            }
+            p->model = std::max(best, 0.0);
         }
         if (bx != 64 && bx != 128) rc = ST_ERR_UNSUPPORTED;
         p->VX3 = bx / 32;
@@ -1399,7 +1419,7 @@ static int plan_create(stencil_plan *out, const stencil_desc *desc)
             if (tb2d_prepare(sh, &bps) == cudaSuccess && bps > 0)
                 p->model = model_gcells_2d(d, p->sms, Cand2D{p->T, p->V, p->W}, bps, 1000);
             (void)cudaGetLastError();
-        } else if (p->alg3) {
+        } else if (p->alg3 && p->model <= 0.0) {   // forced
             p->model = model_gcells_3d(d, p->sms, p->T, p->VX3, p->VY, p->NW);
         }
     }
@@ -1408,14 +1428,7 @@ static int plan_create(stencil_plan *out, const stencil_desc *desc)
         if (e == cudaSuccess) e = stn::dev_zero(p->err, sizeof(int), p->stream);
         if (e != cudaSuccess) rc = map_cuda(e);
     }
-    // last what the plan can do without: the remainder passes' segments (per-cell coefficients; the
-    // others prepare theirs when they first run one) and the extra grids
-    if (d.kind == ST_DIFFUSION_VAR && !d.exact)
-        for (int ts = 1; ts < p->T && rc == ST_OK; ts++) {
-            PassCfg2D *c = nullptr;
-            rc = prepare2(p, kernel_T_for(p, ts), &c);
-        }
-    if (rc == ST_OK) rc = extra_grids(p);
+    if (rc == ST_OK) rc = extra_grids(p);   // last: nothing the plan needs comes after it
     if (rc != ST_OK) {
         stencil_plan_destroy(p);
         return rc;

@@ -50,15 +50,24 @@ public:
                 while (!deal(b, out)) b *= 1.0025;
             return b;
         }
-        double lo = std::max(total_ / slots_, fill_ + 4.0), hi = lo + 3.0 * fill_ + edge_;
-        while (!deal(hi, nullptr)) hi *= 1.5;
-        for (int i = 0; i < 40 && hi - lo > tol; i++) {
-            const double mid = 0.5 * (lo + hi);
-            if (deal(mid, nullptr)) hi = mid;
-            else lo = mid;
+        // (the upper end of the bracket is dealt only if nothing below it suffices)
+        const double first = std::max(total_ / slots_, fill_ + 4.0);
+        std::vector<Segment> list;
+        for (double end = first + 3.0 * fill_ + edge_;; end *= 1.5) {
+            double lo = first, hi = end;
+            bool done = false;
+            for (int i = 0; i < 40 && hi - lo > tol; i++) {
+                const double mid = 0.5 * (lo + hi);
+                if (deal(mid, out ? &list : nullptr)) {
+                    hi = mid;
+                    done = true;
+                    if (out) out->swap(list);
+                } else {
+                    lo = mid;
+                }
+            }
+            if (done || deal(hi, out)) return hi;
         }
-        if (out) deal(hi, out);
-        return hi;
     }
 
 private:
@@ -73,15 +82,16 @@ private:
         return ca != cb ? ca > cb : a.col < b.col;
     }
 
-    // Block b takes what it can of q; false: it takes all of it, else q becomes the rest.
+    // Block b takes what it can of q; true: q is now the rest, false: nothing is left of it.
     bool cut(Block &b, Rest &q, std::vector<Block> &spare, std::vector<Segment> *out) const
     {
         const int h = nz_ - q.z0;
-        const double wc = w_[q.col], fixed = fill_ + (q.z0 == 0 ? edge_ : 0.0);
-        int take = std::max(1, (int)std::min<double>(h, std::floor((b.left - fixed) / wc)));
+        const double wc = w_[q.col], fixed = fill_ + (q.z0 == 0 ? edge_ : 0.0), room = b.left - fixed;
+        const double fit = wc == 1.0 ? room : room / wc;   // (most columns weigh 1: no division)
+        int take = fit >= h ? h : std::max(1, (int)fit);
         // a segment that reaches the end pays `edge` too; one that cannot, leaves a rest
         if (take == h && take > 1 && fixed + edge_ + h * wc > b.left)
-            take = std::max(1, std::min(h - 1, (int)std::floor((b.left - fixed - edge_) / wc)));
+            take = std::max(1, std::min(h - 1, (int)((room - edge_) / wc)));
         if (out) out->push_back(Segment{q.col, q.z0, q.z0 + take, b.id});
         if (take < h) {
             q.z0 += take;
@@ -96,7 +106,9 @@ private:
     {
         // blocks with work to take, the largest budget first, from `head` on; `spare`: those that
         // have a segment and budget left, taken up when the others have run out
-        std::vector<Block> blocks(slots_), spare;
+        std::vector<Block> &blocks = blocks_, &spare = spare_;
+        blocks.resize(slots_);
+        spare.clear();
         for (int b = 0; b < slots_; b++) blocks[b] = Block{speed_.empty() ? budget : budget * speed_[b], b};
         size_t head = 0;
         if (out) out->clear();
@@ -114,7 +126,8 @@ private:
         const auto by_cost = [this](const Rest &a, const Rest &b) { return costlier(a, b); };
         const auto by_col = [](const Rest &a, const Rest &b) { return a.col < b.col; };
         const auto heap_less = [this](const Rest &a, const Rest &b) { return costlier(b, a); };
-        std::vector<Rest> rest, next;
+        std::vector<Rest> &rest = rest_, &next = next_;
+        rest.clear();
 
         // more columns than blocks: whole columns in the order of their cost, and the rests of
         // those that were cut (a heap), whichever is costlier
@@ -173,6 +186,8 @@ private:
     const double fill_, edge_;
     const std::vector<double> w_, speed_;
     double total_ = 0.0;
+    std::vector<Block> blocks_, spare_;   // a deal's, kept for the next one
+    std::vector<Rest> rest_, next_;
     std::vector<Rest> whole_;   // whole columns, the costliest first (only with more columns than blocks)
 };
 

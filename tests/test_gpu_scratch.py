@@ -54,3 +54,19 @@ def test_little_free_memory(eng, orc):  # noqa: F811
     plan.sync()
     assert max_rel(out.cpu().numpy(), orc.run(1, w.u0, w.coef, 7, w.power)) <= TOL
     plan.close()
+
+
+@pytest.mark.parametrize("kind,ndim,nx,ny,nz,kw,holds", [
+    (0, 2, 256, 192, 1, {}, 3),             # resident tiles: exchange grids, counters, flag
+    (0, 2, 300, 200, 1, {"exact": True}, 3),
+    (1, 2, 1024, 1024, 1, {"resident": 1}, 4),   # (and the source map)
+    (0, 2, 484, 61, 1, {"resident": -1}, 3),     # passes: scratch, one list of segments, flag
+    (0, 3, 132, 67, 35, {}, 3), (2, 2, 484, 61, 1, {}, 3), (0, 2, 484, 61, 1, {"rad": 2}, 3)])
+def test_creation_prepares_what_runs(eng, kind, ndim, nx, ny, nz, kw, holds):  # noqa: F811
+    """No segments for passes that a plan may never run: none for resident tiles, none for remainder
+    passes."""
+    live = eng.lib.stencil_debug_live_allocs()
+    plan = eng.Plan(kind, ndim, nx, ny, nz, **kw)
+    assert eng.lib.stencil_debug_live_allocs() - live == holds, plan.info()
+    plan.close()
+    assert eng.lib.stencil_debug_live_allocs() == live
