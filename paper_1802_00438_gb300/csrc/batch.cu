@@ -58,8 +58,11 @@ namespace {
 // 7.46 / 6.89 / 7.07 / 7.95 / 9.00 / 9.80, 16 grids (77 rows) 4.50 / 4.43 / 4.69 / 5.62 / 6.55 /
 // 7.31, 20 grids (51 rows) 3.38 / 3.79 / 4.71 / 5.79 / 6.78 / 7.65 (32: 3.47); one 1000 x 1000 grid
 // 1.13 / 1.27 / 1.50 / 1.77 at L = 16 / 24 / 32 / 48, 4.50 at 192.
+// The queue lists every item of the whole run (16 bytes each), so very long chains get longer items
+// again: at most kItemsMax (256 MiB), as far as kRowsMax allows.
 constexpr int kRowsMin = 16, kRowsMax = 192;
 constexpr double kRowsShare = 0.7;
+constexpr double kItemsMax = 1 << 24;
 constexpr long long kWaitNs = 1000LL * 1000 * 1000;   // 1 s: a wait of a healthy batch is far shorter
 // (T, V) of the compiled queue kernel: 4 cells per lane (64-grid workload: 12.8 ms; with 8, 255
 // registers and two warps per scheduler, 14.1 ms at its best L; T = 12 with 4 cells, 255
@@ -81,8 +84,16 @@ int default_rows(const std::vector<stencil_batch_grid> &grids, int T, int cx, in
         rows += (double)((q.nx + cx - 1) / cx) * q.ny * passes;
         longest = std::max(longest, passes);
     }
-    const double l = kRowsShare * rows / ((double)longest * warps);
-    return std::max(kRowsMin, ((int)std::min<double>(kRowsMax, l) + 7) / 8 * 8);
+    const double share = kRowsShare * rows / ((double)longest * warps);
+    int l = std::max(kRowsMin, ((int)std::min<double>(kRowsMax, share) + 7) / 8 * 8);
+    const auto items = [&]() {
+        double n = 0.0;
+        for (const stencil_batch_grid &q : grids)
+            n += (double)((q.nx + cx - 1) / cx) * ((q.ny + l - 1) / l) * (((long long)q.steps + T - 1) / T);
+        return n;
+    };
+    while (l < kRowsMax && items() > kItemsMax) l = std::min(kRowsMax, 2 * l);
+    return l;
 }
 
 size_t align256(size_t n) { return (n + 255) / 256 * 256; }

@@ -109,3 +109,20 @@ def test_batch_bounded_wait_runs_out(eng, orc):
         b2 = eng.Batch(items)
         b2.set_wait(0)                        # a limit must be positive
     assert e.value.code == eng.ST_ERR_INVALID_ARG
+
+
+def test_long_chain_table(eng):
+    """The device table of a long run (10^6 passes of a small grid) stays in proportion: its items
+    get longer, so that there are at most 2^24 of them (16 bytes each)."""
+    import torch
+    u = torch.zeros(256, 256, device="cuda")
+    item = {"kind": 0, "nx": 256, "ny": 256, "steps": 8 * 10 ** 6, "grid_in": u, "grid_out": torch.empty_like(u),
+            "power": None, "coeffs": [0.2] * 5}
+    eng.Batch([dict(item, steps=80)]).close()   # (what a first batch loads once)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    b = eng.Batch([item])
+    used = free - torch.cuda.mem_get_info()[0]
+    b.close()
+    # besides the items: one descriptor a pass (below 256 bytes), scratch and allocation granularity
+    assert used <= 16 * 2 ** 24 + 256 * 10 ** 6 + 2 ** 24, used
