@@ -265,3 +265,16 @@ def test_adjoint_full_size(eng, orc, kind):
     wt = synth.loss_weights(7601, w.shape)
     res = _run(eng, w, wt, 200, 20)
     _check(orc, w, wt, 200, res)
+
+
+@pytest.mark.parametrize("kind", [0, 1])
+@pytest.mark.parametrize("nx", [127, 128, 129, 132, 247, 248, 249, 252, 368])
+def test_adjoint_tiles_that_end_on_the_edge(eng, orc, kind, nx):
+    """Tiles own cells up to the grid's edges: widths and heights where the last tile (128 x 32, a
+    120 x 24 step) ends exactly on the edge, one cell before and one after it; rows aligned (the
+    staged path) and not."""
+    for ny in (31, 32, 33, 55, 56, 57, 80):
+        steps, ckpt = 5 + ny % 3, 4
+        w = synth.make(kind, 2, nx, ny, steps=steps, seed=7400 + 13 * nx + ny + kind)
+        wt = synth.loss_weights(7500 + nx, w.shape)
+        _check(orc, w, wt, steps, _run(eng, w, wt, steps, ckpt))

@@ -81,3 +81,48 @@ def test_star_in_place_and_errors(eng, orc, R):
         eng.Plan(1, 2, 64, 64, rad=2)
     with pytest.raises(eng.StencilError):      # 2D star tiles are 128 wide
         eng.Plan(0, 2, 64, 64, rad=2, force_bx=64)
+
+
+@pytest.mark.parametrize("one", [False, True])
+@pytest.mark.parametrize("nx", [260, 261])
+@pytest.mark.parametrize("T,steps", [(4, 3), (4, 4), (4, 7), (4, 11), (2, 5), (1, 2)])
+def test_star_rows_in_place(eng, orc, nx, T, steps, one):
+    """Contracted radius 2, in place with one, two and three passes, rows aligned and not; with one
+    scratch grid where an odd width would have two (the allocation that fails is injected)."""
+    import torch
+    w = synth.make_star(2, 2, nx, 70, seed=9300 + steps)
+    u = torch.from_numpy(np.ascontiguousarray(w.u0)).cuda()
+    plan = eng.Plan(0, 2, nx, 70, rad=2, force_T=T)
+    whole = plan.info()["scratch_bytes"]
+    if one and nx % 4:
+        plan.close()
+        for n in range(1, 12):
+            assert eng.lib.stencil_debug_fail_alloc(n) == eng.ST_OK
+            try:
+                plan = eng.Plan(0, 2, nx, 70, rad=2, force_T=T)
+                break
+            except eng.StencilError as e:
+                assert e.code == eng.ST_ERR_OOM
+            finally:
+                eng.lib.stencil_debug_fail_alloc(0)
+        assert plan.info()["scratch_bytes"] * 2 == whole
+    assert plan.info()["kernel_id"] == 8
+    plan.run(u, u, w.coef, steps)
+    plan.sync()
+    plan.close()
+    assert max_rel(u.cpu().numpy(), orc.run_star(2, w.u0, w.coef, steps)) <= TOL
+
+
+@pytest.mark.parametrize("T", [1, 2, 4])
+def test_star_forced_tile_contracted(eng, orc, T):
+    """Contracted radius 2 in shared-memory tiles, which only a forced tile still runs."""
+    import torch
+    for t, (nx, ny) in enumerate(SIZES[3:] + [(1000, 300)]):
+        w = synth.make_star(2, 2, nx, ny, seed=9400 + t)
+        u = torch.from_numpy(np.ascontiguousarray(w.u0)).cuda()
+        plan = eng.Plan(0, 2, nx, ny, rad=2, force_T=T, force_bx=128)
+        assert plan.info()["kernel_id"] == 5
+        for steps in (1, T + 1, 3 * T + 2):
+            g = plan.run(u, torch.full_like(u, float("nan")), w.coef, steps).cpu().numpy()
+            assert max_rel(g, orc.run_star(2, w.u0, w.coef, steps)) <= TOL, (nx, ny, steps)
+        plan.close()
