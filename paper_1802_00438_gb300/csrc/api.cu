@@ -1216,8 +1216,9 @@ static int plan_create(stencil_plan *out, const stencil_desc *desc)
             // Contracted plans run one-warp tiles of V = 8 cells per thread (bsize_x = 256) with
             // partial-sum stages; exact plans run the rotating-window kernel, V = 4, with W warps
             // per tile (bsize_x = 128 W).
-            // measured on GB300 (16384^2, T = 8): Hotspot runs best with V = 4 (its V = 8 body
-            // overflows the instruction cache), Diffusion with V = 8
+            // Where only T is forced, Hotspot takes V = 4: T = 8 against V = 8 (the better of its two
+            // variants) 601 / 677 us on 3000 x 2000 x 160, 1467 / 1570 on 4096^2 x 200, 3985 / 3700 on
+            // 8192^2 x 160, 7517 / 6951 on 16384^2 x 80.  With nothing forced the model chooses below.
             const bool var = d.kind == ST_DIFFUSION_VAR;   // windowed kernel, exact or contracted
             p->V = d.force_vec ? d.force_vec : ((d.exact || d.kind != ST_DIFFUSION) ? 4 : 8);
             if (d.force_bx) {
@@ -1232,9 +1233,9 @@ static int plan_create(stencil_plan *out, const stencil_desc *desc)
             if (p->stor && !d.force_T && !d.force_vec && !d.force_bx && !d.partial_rows) {
                 // 16-bit storage, nothing forced: T = 8 with 8 cells per lane, rows in place, or,
                 // where a block has few rows, 4 cells per lane (three warps per scheduler).  The
-                // line is the float32 kernels' (their model): measured on GB300, 8192^2 Hotspot
-                // bf16 x 200 5241 against 6171 us, 3000 x 2000 887 against 846, 1100 x 6000 x 100
-                // 611 against 521
+                // line is the float32 kernels' (their model).  Measured on GB300, 8 against 4 cells,
+                // bf16 Hotspot: 8192^2 x 200 5222 / 6396 us, 16384^2 x 80 8993 / 11093; on the other
+                // side of the line 3000 x 2000 x 150 703 / 713, 1100 x 6000 x 100 578 / 541
                 int b8 = 0, b4 = 0;
                 const Shape2D s8{d.kind, 0, 8, 8, 0, shape_stor(p)}, s4{d.kind, 0, 8, 4, 1, shape_stor(p)};
                 p->V = 8;

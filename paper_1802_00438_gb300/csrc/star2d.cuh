@@ -1,7 +1,7 @@
 // Star diffusion of radius R in 2D (4R+1 points), in shared-memory tiles (exact plans, radii 3 and
-// 4, forced tiles; contracted plans of radius 2 stream rows instead, star2f.cu): combined spatial and temporal blocking with
-// halos of width R*T (arXiv 1802.00438, Eqs. 1-2 with rad = R > 1, the paper's named
-// extension to higher-order stencils; Sec. 3.2's fused steps; Sec. 5.1's clamped boundary).
+// 4, forced tiles; contracted plans of radius 2 stream rows instead, star2f.cu): combined spatial
+// and temporal blocking with halos of width R*T (arXiv 1802.00438, Eqs. 1-2 with rad = R > 1, the
+// paper's named extension to higher-order stencils; Sec. 3.2's fused steps; Sec. 5.1's clamped boundary).
 //
 // Persistent blocks, one per SM, take the 128 x 128 tiles (halos included) round-robin.  A tile
 // arrives in shared memory by one tensor-map copy (or plain loads when rows are not 16-byte

@@ -62,7 +62,8 @@ struct TB2 {
 };
 
 enum { MODE_PLAIN = 0, MODE_EDGE = 1, MODE_SPECIAL = 2,
-       MODE_HEAD = 3, MODE_GHOST = 4 };   // k_tb2f only: segment fill rows; x = nx-1 inside a lane
+       MODE_HEAD = 3, MODE_GHOST = 4 };   // k_tb2f, k_star2f, k_vd2f: segment fill rows; x = nx-1
+                                          // inside a lane
 
 struct Ctx2 {
     const float *__restrict__ in;

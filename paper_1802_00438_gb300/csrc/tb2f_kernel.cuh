@@ -42,7 +42,7 @@
 // (every stage reads its source row), two warps per scheduler; diffusion 58 / 52 / 30 %.
 //
 // GPU mapping: one warp per block; a tile is BX = 32*V cells wide incl. halos of
-// H = roundup(T, 4) cells per side; thread = V consecutive cells; x-neighbours of a thread's
+// H = roundup(T, V) cells per side; thread = V consecutive cells; x-neighbours of a thread's
 // edge cells by shuffle (the warp edge is the tile edge, inside the halo).  Field and power
 // rows arrive through shared-memory rings filled by cp.async PF rows ahead.  The power ring
 // keeps a mirrored copy of its first PW-1 slots, so the PW = T + 1 power rows an iteration may
