@@ -251,7 +251,7 @@ struct Res2D {
     float src_sdc, src_a;  // contracted Hotspot: the source map sdc*(p + amb*Rz), a = amb*Rz
     float *xg;             // two exchange grids (epoch parity), rows of ld_x floats
     long long xplane, ld_x;
-    int *flags;            // per block: epochs published, as epoch0 + e + 1 (never reset)
+    int *flags;            // per block: epochs published, as epoch0 + e + 1 (reset only by captured runs)
     int epoch0;
     int *status;           // set to 1 by a wait that gave up
     long long wait_ns;     // bound of every wait
